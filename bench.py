@@ -66,13 +66,12 @@ def peaks():
         return 6800.0, "fallback"
 
 
-def tma_kernel_source_sha():
-    """sha256 (16 hex) of the TMA step kernel's source text (from its section
-    comment to the slice-conversion code that follows it)."""
-    src = open(os.path.join(ROOT, "paper_2005_09534_gb300", "csrc", "hamiltonian.cu")).read()
-    a = src.index("// ------------------------------------------------- TMA-pipelined step kernel")
-    b = src.index("template <class NT>\nstruct Conv;")
-    return hashlib.sha256(src[a:b].encode()).hexdigest()[:16]
+def step_kernel_source_sha():
+    """sha256 (16 hex) of the step kernel's source text (from its section comment
+    to the end of the file)."""
+    src = open(os.path.join(ROOT, "paper_2005_09534_gb300", "csrc", "rows.h")).read()
+    a = src.index("// ---------------------------------------------------------------- step kernel")
+    return hashlib.sha256(src[a:].encode()).hexdigest()[:16]
 
 
 def step_kernel_traffic(precision, workload):
@@ -80,7 +79,7 @@ def step_kernel_traffic(precision, workload):
     this workload and precision, if it was taken on the current kernel source
     (else None)."""
     try:
-        sha = tma_kernel_source_sha()
+        sha = step_kernel_source_sha()
         with open(os.path.join(ROOT, "profiles", "step_kernel_traffic.json")) as f:
             d = json.load(f)
         e = d.get(f"{workload}:{precision}")
@@ -537,7 +536,7 @@ def run_single(args, pf, torch, dev, world, rank, local, dist):
             "frac": round(d["achieved_gbs"] / peak, 4),
             "traffic": (tr or {}).get("dram_bytes_per_launch_scaled"),
             "peak_kind": f"of {peak_kind}",
-            "kernel": f"k_ham_step_tma<{dom}> (Clenshaw step on a 128-byte column slice)",
+            "kernel": f"k_step_rows<{dom}> (Clenshaw steps on 128-byte column slices, many steps to a launch)",
             "alg_bytes_per_launch": d["alg_bytes_per_launch"], "avg_launch_us": d["avg_launch_us"],
             "launches": d["launches"], "share_of_step": d["share_of_step"], "by_kind": kinds}
     if tr:
@@ -589,8 +588,8 @@ def run_single(args, pf, torch, dev, world, rank, local, dist):
 
 def run_filter_only(args, pf, torch, dev):
     """One polfed_cheb_filter call (sigma = 0, order --K) on a seeded block of the
-    workload's Hamiltonian, for kernel profiling (ncu): K + 1 step-kernel launches
-    per 128-byte column slice.  Batched workloads: one polfed_cheb_filter_batched
+    workload's Hamiltonian, for kernel profiling (ncu): one cooperative launch of
+    all K steps per 128-byte column slice.  Batched workloads: one polfed_cheb_filter_batched
     call over their realizations (n_b = 16)."""
     kind = PREC[args.precision]
     dt = torch.float32 if kind == pf.F32 else torch.float64
@@ -617,7 +616,7 @@ def run_filter_only(args, pf, torch, dev):
     Y = torch.empty_like(X)
     b = field_free_bound(m)
     reps = max(1, args.reps)
-    stream = torch.cuda.Stream(device=dev)  # a capturable stream (the Clenshaw loop may run as a CUDA graph)
+    stream = torch.cuda.Stream(device=dev)
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     c0 = pf.get_counters()
     torch.cuda.synchronize()
@@ -841,7 +840,7 @@ def run_batched(args, pf, torch, dev, world, rank, local, dist):
                        "l2": "instances of 12870-48620 rows: filter working sets partly L2-resident, no flush"},
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(achieved / peak, 4), "traffic": None, "peak_kind": f"of {peak_kind}",
-                         "kernel": "k_filter_batched (all realizations' Clenshaw steps, one cooperative launch)",
+                         "kernel": "k_step_rows (all realizations' Clenshaw steps, one cooperative launch)",
                          "alg_bytes_per_launch": fa / max(1, sum(i["rounds"] for i in infos)),
                          "avg_launch_us": round(1e6 * fg / max(1, sum(i["rounds"] for i in infos)), 1)},
             "e2e": {"value": round(pairs_all / wall_s, 4), "unit": "eigenpairs/s",

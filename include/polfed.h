@@ -120,7 +120,7 @@ typedef struct polfed_stats {
   double max_resid;      /* max ||H u - E u|| over the returned pairs (H units) */
   double t_bounds, t_filter, t_reorth, t_qr, t_teig, t_ritz, t_total; /* seconds */
   int64_t n_launches;      /* kernels this library launched during the call */
-  int64_t n_step_launches; /* launches of the Chebyshev step kernels inside event-timed filter runs */
+  int64_t n_step_launches; /* launches of the Chebyshev step kernel (many steps each) inside event-timed filter runs */
   double step_gpu_s;       /* device time of those launches (CUDA events on the launching stream) */
   double step_alg_bytes;   /* algorithmic bytes of those launches: N * cols * w * (3 + [c_k != 0]) each */
   int32_t dos_rule;        /* rule that set K */
@@ -171,7 +171,8 @@ int polfed_h_apply(const polfed_model* model, const uint32_t* d_states, int64_t 
  *            D = sum_n c_n T_n(sigma)); else a HOST array of K + 1 doubles used as
  *            Y = sum_n coeffs[n] T_n(H~) X.
  *   other arguments as in polfed_h_apply.
- * Enqueues about K + 3 kernels per 128-byte column slice; synchronizes the
+ * Runs the K steps of the block's column slices in a few cooperative launches
+ * (one at a time per device in a process); synchronizes the
  * stream before returning (it owns stream-ordered scratch).  Returns
  * POLFED_EBOUNDS if the output is not finite (spectrum outside [e_lo, e_hi]). */
 int polfed_cheb_filter(const polfed_model* model, const uint32_t* d_states, int64_t dim, double e_lo, double e_hi,
@@ -430,7 +431,7 @@ int polfed_mlp_predict(polfed_mlp* net, const polfed_model* model, double W, dou
 /* Eq. (2) filter of many realizations in ONE cooperative kernel launch: every
  * (realization, 128-byte column slice) job runs its own Clenshaw recurrence of
  * order K[i] with the paper's coefficients for sigma[i], on its own H~ (plans
- * with the low/high split b = min(10, L - 4)).  Launch step t performs step t
+ * with a low/high split of their own).  Launch step t performs step t
  * of every job with t < K[i]; CTAs meet at a grid barrier between steps
  * (bounded wait: POLFED_ETIMEOUT, never a hang).
  *   n_inst       : number of realizations (>= 1); all with J2 == 0 or all with J2 != 0.
@@ -440,7 +441,7 @@ int polfed_mlp_predict(polfed_mlp* net, const polfed_model* model, double W, dou
  *                  (float for POLFED_F32, double for POLFED_DF64); X_i, Y_i must not overlap.
  *   n_b          : 1..128 (the same for all).
  *   dtype        : POLFED_F32 or POLFED_DF64.
- *   ctas_per_sm  : 0 = as many as fit (1 or 2), else 1 or 2.
+ *   ctas_per_sm  : 0 or 2 = all six teams of four warps per SM, 1 = half of them.
  * Synchronizes the stream.  POLFED_EBOUNDS if an output grew beyond the
  * Chebyshev bound. */
 int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const double* e_lo, const double* e_hi,
@@ -450,7 +451,7 @@ int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const
 /* What polfed_eigs_batched did. */
 typedef struct polfed_batch_info {
   int32_t n_b;              /* block width of realization 0 */
-  int32_t ctas_per_sm;      /* grid of the batched filter (0 = all that fit) */
+  int32_t ctas_per_sm;      /* team setting of the batched filter (as in polfed_cheb_filter_batched) */
   int32_t rounds;           /* batched filter launches */
   int32_t workers;          /* host threads */
   int32_t n_width16, n_width32, n_width64; /* realizations per block width */
@@ -459,7 +460,7 @@ typedef struct polfed_batch_info {
   double t_tune;            /* seconds spent autotuning */
   double filter_gpu_s;      /* device time of the batched filter launches (CUDA events) */
   double filter_alg_bytes;  /* their algorithmic bytes (Clenshaw minimum) */
-  double tune_step_s[3][2]; /* autotuner: seconds per filter step for widths 16/32/64 x 1/2 CTAs per SM */
+  double tune_step_s[3][2]; /* autotuner: seconds per filter step for widths 16/32/64 x team settings 1/2 */
   int64_t n_launches;       /* kernels launched by the call */
 } polfed_batch_info;
 
@@ -471,7 +472,7 @@ typedef struct polfed_batch_info {
  *   device     : CUDA device ordinal.
  *   eps_target, N_ev, K : host arrays of n_inst (K may be NULL = all automatic).
  *   n_b        : block width for all, or 0 = autotune: the batched filter is timed on the
- *                realizations' operators for widths 16/32/64 and 1/2 CTAs per SM, and each
+ *                realizations' operators for widths 16/32/64 and team settings 1/2, and each
  *                realization takes the width with the least predicted filter time.
  *   opts       : options (precision POLFED_F32 or POLFED_DF64), or NULL.
  *   evals      : host out, sum(N_ev) values: realization i at offset sum_{j<i} N_ev[j].
@@ -489,14 +490,12 @@ int polfed_eigs_batched(int32_t device, int32_t n_inst, const polfed_model* mode
                         polfed_stats* stats, int32_t* status, polfed_batch_info* info);
 
 /* Test support for the failure path (the paper has no counterpart).  Every
- * device-side wait of this library is bounded: the bulk-copy pipeline of the
- * step kernel polls its mbarriers at most 2^22 times, the grid barrier of the
- * batched filter at most 2^24 times (about a second); a wait that runs out
- * makes the kernel stop, wait with the full cap for the copies it already
- * issued, and the call returns POLFED_ETIMEOUT with its output discarded.
- * polfed_set_wait_limit(polls) lowers both caps to `polls` for the calls that
- * follow in this process (0 restores the defaults), so a test can make the
- * waits run out without stalling anything.  Not for production use. */
+ * device-side wait of this library is bounded: the grid barrier between the
+ * steps of a filter polls at most 2^24 times (tens of seconds); a wait that runs out
+ * makes the kernel stop, and the call returns POLFED_ETIMEOUT with its output
+ * discarded.  polfed_set_wait_limit(polls) lowers the cap to `polls` for the
+ * calls that follow in this process (0 restores the default), so a test can make
+ * the waits run out without stalling anything.  Not for production use. */
 int polfed_set_wait_limit(uint32_t polls);
 
 /* ------------------------------------------------------------------------

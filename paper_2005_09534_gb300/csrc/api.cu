@@ -116,14 +116,13 @@ int polfed_h_apply(const polfed_model* model, const uint32_t* d_states, int64_t 
   HamPlan plan;
   PF_CHECK(plan.init(model, s, true));
   PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
-  const int lpr = choose_lpr(dtype, n_b);
   StreamScratch mem;
   mem.s = s;
   FilterScratch scr;
-  scr.bytes = filter_scratch_bytes(plan, dtype, lpr);
+  scr.bytes = filter_scratch_bytes(plan, dtype, n_b);
   PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
   scr.xs = mem.p;
-  PF_CHECK(apply_block(plan, dtype, d_X, d_Y, n_b, dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64, scr, s, lpr));
+  PF_CHECK(apply_block(plan, dtype, d_X, d_Y, n_b, dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64, scr, s));
   PF_CUDA(cudaStreamSynchronize(s));
   return POLFED_OK;
 }
@@ -153,15 +152,14 @@ int polfed_cheb_filter(const polfed_model* model, const uint32_t* d_states, int6
   HamPlan plan;
   PF_CHECK(plan.init(model, s, true));
   PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
-  const int lpr = choose_lpr(dtype, n_b);
   StreamScratch mem;
   mem.s = s;
   FilterScratch scr;
-  scr.bytes = filter_scratch_bytes(plan, dtype, lpr);
+  scr.bytes = filter_scratch_bytes(plan, dtype, n_b);
   PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
   scr.xs = mem.p;
   PF_CHECK(filter_block(plan, dtype, c.data(), K, invD, d_X, d_Y, n_b, dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64,
-                        scr, s, lpr));
+                        scr, s));
   float flag[3] = {0, 0, 0};
   PF_CUDA(cudaMemcpyAsync(flag, scr.flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
   PF_CUDA(cudaStreamSynchronize(s));
@@ -195,12 +193,11 @@ int polfed_cheb_filter_cols(const polfed_model* model, const uint32_t* d_states,
   HamPlan plan;
   PF_CHECK(plan.init(model, s, true));
   PF_CHECK(plan.prepare_typed(POLFED_F32, e_lo, e_hi));
-  const int lpr = choose_lpr(POLFED_F32, n_b);
   StreamScratch mem, cmem;
   mem.s = s;
   cmem.s = s;
   FilterScratch scr;
-  scr.bytes = filter_scratch_bytes(plan, POLFED_F32, lpr);
+  scr.bytes = filter_scratch_bytes(plan, POLFED_F32, n_b);
   PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
   scr.xs = mem.p;
   PF_CUDA(cudaMallocAsync(&cmem.p, cf.size() * sizeof(float), s));

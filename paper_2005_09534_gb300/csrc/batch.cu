@@ -13,7 +13,7 @@
 //
 // Autotuner: before the run, the batched filter kernel is timed on the
 // realizations' own operators for each candidate block width (16, 32, 64
-// columns) and grid (1 or 2 CTAs per SM); each realization then takes the
+// columns) and team setting (half or all of an SM's teams); each realization then takes the
 // width that minimizes (measured time per filter step of width S) x (steps
 // its Lanczos run needs, about max(16, ceil(2.64 N_ev / S) + 8)).
 #include <algorithm>
@@ -101,6 +101,7 @@ class Rendezvous : public FilterHook {
     r.in.assign(in, in + npan);
     r.out.assign(out, out + npan);
     r.S = S;
+    PF_CHECK(plan.prepare_rec(kBatchLpr, s));
     if (cudaEventCreateWithFlags(&r.ready, cudaEventDisableTiming) != cudaSuccess)
       return fail(POLFED_ECUDA, "cudaEventCreate failed");
     cudaEventRecord(r.ready, s);
@@ -247,6 +248,7 @@ int autotune(const std::vector<polfed_model>& models, const std::vector<int>& N_
     PF_CHECK(plans[i].init(&models[i], s, false, batch_b(models[i].L)));
     const double b = norm_bound(models[i]);
     PF_CHECK(plans[i].prepare_typed(kind, -b, b));
+    PF_CHECK(plans[i].prepare_rec(kBatchLpr, s));
     vec_bytes += (size_t)plans[i].geo.dim * 64 * sizeof(double);
   }
   DeviceBuffer X, Y, scr;
@@ -331,6 +333,7 @@ int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const
     if (!d_X[i] || !d_Y[i] || d_X[i] == d_Y[i]) return fail(POLFED_EINVAL, "bad X / Y pointers");
     PF_CHECK(plans[i].init(&models[i], s, true, batch_b(models[i].L)));
     PF_CHECK(plans[i].prepare_typed(dtype, e_lo[i], e_hi[i]));
+    PF_CHECK(plans[i].prepare_rec(kBatchLpr, s));
     double D = 1.0;
     cheb_coeffs(sigma[i], K[i], coefs[i], D);
     items.push_back(BatchFilterItem{&plans[i], coefs[i].data(), K[i], 1.0 / D, d_X[i], d_Y[i], n_b, false});

@@ -104,15 +104,14 @@ int kpm_run(HamPlan& plan, int kind, const T* r, int R, int n_mom, double* mu, c
   T* prev = (T*)b.t0;
   T* cur = (T*)b.t1;
   T* y = (T*)b.y;
-  const int lpr = choose_lpr(kind, R);
   PF_CUDA(cudaMemcpyAsync(prev, r, (size_t)n * sizeof(T), cudaMemcpyDeviceToDevice, s));
-  PF_CHECK(apply_block(plan, kind, prev, cur, R, abi, scr, s, lpr));
+  PF_CHECK(apply_block(plan, kind, prev, cur, R, abi, scr, s));
   k_kpm_dots<T><<<kDotBlocks, kDotThreads, 0, s>>>(prev, cur, n, b.part);
   k_kpm_reduce<<<1, kDotThreads, 0, s>>>(b.part, kDotBlocks, b.mu);
   count_launch(2);
   const int half = (n_mom + 1) / 2;  // t_0 .. t_half are needed
   for (int k = 1; k < half; k++) {
-    PF_CHECK(apply_block(plan, kind, cur, y, R, abi, scr, s, lpr));
+    PF_CHECK(apply_block(plan, kind, cur, y, R, abi, scr, s));
     k_kpm_step<T><<<kDotBlocks, kDotThreads, 0, s>>>(y, prev, cur, n, b.part);
     k_kpm_reduce<<<1, kDotThreads, 0, s>>>(b.part, kDotBlocks, b.mu + 2 * k);
     count_launch(2);
@@ -200,8 +199,7 @@ int polfed_kpm_moments(const polfed_model* model, const uint32_t* d_states, int6
   PF_CHECK(plan.init(model, s, true));
   PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
   const int abi = dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64;
-  const int lpr = choose_lpr(dtype, R);
-  const size_t fb = (filter_scratch_bytes(plan, dtype, lpr) + 255) & ~(size_t)255;
+  const size_t fb = (filter_scratch_bytes(plan, dtype, R) + 255) & ~(size_t)255;
   void* mem = nullptr;
   PF_CUDA(cudaMallocAsync(&mem, fb + kpm_buffer_bytes(dim, R, abi), s));
   FilterScratch scr;

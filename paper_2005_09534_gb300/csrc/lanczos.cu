@@ -212,12 +212,11 @@ struct LanczosParams {
 // Y_q = invD sum_n coef[n] T_n(H~) X_q for the panels q (dim x S each), directly
 // or through the batched runner's rendezvous.
 int run_filter(HamPlan& plan, const LanczosParams& P, int kind, const double* coef, int K, double invD,
-               const double* const* in, double* const* out, int npan, int S, FilterScratch& scr, cudaStream_t s,
-               int lpr) {
+               const double* const* in, double* const* out, int npan, int S, FilterScratch& scr, cudaStream_t s) {
   if (P.hook && (kind == POLFED_F32 || kind == POLFED_DF64))
     return P.hook->filter(plan, kind, coef, K, invD, in, out, npan, S, s);
   for (int q = 0; q < npan; q++)
-    PF_CHECK(filter_block(plan, kind, coef, K, invD, in[q], out[q], S, POLFED_F64, scr, s, lpr));
+    PF_CHECK(filter_block(plan, kind, coef, K, invD, in[q], out[q], S, POLFED_F64, scr, s));
   return POLFED_OK;
 }
 
@@ -255,8 +254,7 @@ int run_lanczos(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, double* d_
   const int64_t pstride = dim * S;
   PF_CHECK(c->basis.ensure((size_t)(m_max + 1) * pstride * sizeof(double), &c->ws_total, c->ws_limit));
   PF_CHECK(c->U.ensure((size_t)pstride * sizeof(double), &c->ws_total, c->ws_limit));
-  const int lpr = choose_lpr(kind, S);
-  PF_CHECK(c->fscr.ensure(filter_scratch_bytes(plan, kind, lpr), &c->ws_total, c->ws_limit));
+  PF_CHECK(c->fscr.ensure(filter_scratch_bytes(plan, kind, S), &c->ws_total, c->ws_limit));
   PF_CHECK(plan.prepare_typed(kind, P.e_lo, P.e_hi));
   FilterScratch scr;
   scr.xs = c->fscr.p;
@@ -293,7 +291,7 @@ int run_lanczos(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, double* d_
     {
       const double* in1[1] = {Qj};
       double* out1[1] = {Ub};
-      PF_CHECK(run_filter(plan, P, kind, coef.data(), P.K, invD, in1, out1, 1, S, scr, s, lpr));
+      PF_CHECK(run_filter(plan, P, kind, coef.data(), P.K, invD, in1, out1, 1, S, scr, s));
     }
     PF_CHECK(D.coldot(Ub, Ub, S, colnrm.data(), s));  // synchronizes
     out.matvec_cols += (int64_t)P.K * S;
@@ -510,15 +508,13 @@ int rr_select(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, const double
   double* Uo = Rl.Uo;  // selected eigenvectors
   double* Wo = Rl.Wo;  // their images
   PF_CHECK(plan.prepare_typed(POLFED_F64, P.e_lo, P.e_hi));
-  const int lpr64 = choose_lpr(POLFED_F64, S);
-  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, lpr64)), &c->ws_total,
+  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, S)), &c->ws_total,
                           c->ws_limit));
   FilterScratch scr64;
   scr64.xs = c->fscr.p;
   scr64.bytes = c->fscr.n;
   for (int q = 0; q < npan; q++)
-    PF_CHECK(apply_block(plan, POLFED_F64, U + (size_t)q * pstride, Wr + (size_t)q * pstride, S, POLFED_F64, scr64, s,
-                         lpr64));
+    PF_CHECK(apply_block(plan, POLFED_F64, U + (size_t)q * pstride, Wr + (size_t)q * pstride, S, POLFED_F64, scr64, s));
   out.matvec_cols += nr_pad;
   // G = U^T W (nr_pad x nr_pad); the eigen-solve of its leading nr x nr block
   PF_CHECK(c->evbuf.ensure(((size_t)nr_pad * nr_pad + nr_pad) * sizeof(double), &c->ws_total, c->ws_limit));
@@ -700,15 +696,14 @@ int refine_dd(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, int Kr, int 
   const double t0 = now_s();
   // 1. Rayleigh-Ritz basis of span(U): W = H~ U (FP64), G = U^T W = Y diag(lam) Y^T
   PF_CHECK(plan.prepare_typed(POLFED_F64, P.e_lo, P.e_hi));
-  const int lpr64 = choose_lpr(POLFED_F64, S);
-  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, lpr64)), &c->ws_total,
+  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, S)), &c->ws_total,
                           c->ws_limit));
   FilterScratch scr64;
   scr64.xs = c->fscr.p;
   scr64.bytes = c->fscr.n;
   for (int q = 0; q < npan; q++)
     PF_CHECK(apply_block(plan, POLFED_F64, R.U + (size_t)q * pstride, R.Wr + (size_t)q * pstride, S, POLFED_F64, scr64,
-                         s, lpr64));
+                         s));
   out.matvec_cols += nr_pad;
   PF_CHECK(c->evbuf.ensure(((size_t)nr_pad * nr_pad + nr_pad) * sizeof(double), &c->ws_total, c->ws_limit));
   double* G = c->evbuf.as<double>();
@@ -791,8 +786,7 @@ int refine_dd(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, int Kr, int 
   if (nc > 0) {
     PF_CHECK(D.gather_cols(R.T, idx_d, nc, npc * S, R.Wr, s));
     PF_CHECK(plan.prepare_typed(POLFED_F32, P.e_lo, P.e_hi));
-    const int lpr32 = choose_lpr(POLFED_F32, S);
-    PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F32, lpr32)), &c->ws_total,
+    PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F32, S)), &c->ws_total,
                             c->ws_limit));
     FilterScratch scr;
     scr.xs = c->fscr.p;
@@ -815,8 +809,7 @@ int spectral_bounds(polfed_ctx* c, HamPlan& plan, const polfed_opts& o, double* 
   cudaStream_t s = c->stream;
   const int64_t dim = plan.geo.dim;
   PF_CHECK(plan.prepare_typed(POLFED_F64, 0.0, 0.0));
-  const int lpr = choose_lpr(POLFED_F64, 1);
-  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, lpr)), &c->ws_total, c->ws_limit));
+  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, 1)), &c->ws_total, c->ws_limit));
   FilterScratch scr;
   scr.xs = c->fscr.p;
   scr.bytes = c->fscr.n;
@@ -836,7 +829,7 @@ int spectral_bounds(polfed_ctx* c, HamPlan& plan, const polfed_opts& o, double* 
   const int kmax = (int)std::min<int64_t>(o.bounds_steps, dim);
   double lo = 0, hi = 0, e_lo = 1e300, e_hi = 1e300;
   for (int k = 0; k < kmax; k++) {
-    PF_CHECK(apply_block(plan, POLFED_F64, v1, w, 1, POLFED_F64, scr, s, lpr));
+    PF_CHECK(apply_block(plan, POLFED_F64, v1, w, 1, POLFED_F64, scr, s));
     (*matvecs)++;
     double a = 0.0;
     PF_CHECK(D.coldot(v1, w, 1, &a, s));
@@ -892,8 +885,7 @@ int kpm_rho(polfed_ctx* c, HamPlan& plan, double e_lo, double e_hi, double sigma
   const int64_t dim = plan.geo.dim;
   const int kind = POLFED_DF64;
   PF_CHECK(plan.prepare_typed(kind, e_lo, e_hi));
-  const int lpr = choose_lpr(kind, R);
-  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, kind, lpr)), &c->ws_total, c->ws_limit));
+  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, kind, R)), &c->ws_total, c->ws_limit));
   FilterScratch scr;
   scr.xs = c->fscr.p;
   scr.bytes = c->fscr.n;

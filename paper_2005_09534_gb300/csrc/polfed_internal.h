@@ -104,17 +104,15 @@ struct HamTables {
   double* F_lo;     // [2^b] diagonal part from low bonds and low fields (H units)
   double* F_hi;     // [2^nh] diagonal part from high bonds and high fields
   double* C_x;      // [2^n_cross] diagonal part from cross bonds by "differ" pattern
-  // [2^b * rec_stride] per-row neighbour record, indexed by cls_off[c] + local index:
-  //   entry 0: s_lo; entry 1: n1 | n2 << 8 (active low bonds of class 1 and 2);
-  //   entries 2..: local indices of the active low-bond neighbours, class 1 first;
-  //   last entries (from the end): local index, in the neighbouring popcount
-  //   class, of s_lo with the low site of cross bond k flipped
-  uint16_t* rec;
-  // [2^b * rec_stride] bytes: the same records with one-byte entries (local
-  // indices are < 256), for the shared-memory copy of the bulk-copy kernel:
-  //   bytes 0-1: s_lo; byte 2: n1; byte 3: n2; bytes 4..: active low-bond
-  //   neighbours (class 1 first); last bytes (from the end): cross neighbours
-  uint8_t* rec8;
+  // [2^b * rec_stride] per-row neighbour records, indexed by cls_off[c] + local
+  // index; one table per lanes-per-row 1, 2, 4, 8 (entries are byte offsets
+  // (local index + 1) * row bytes into a tile whose first row is zero):
+  //   entry 0: bits of s_lo at the low sites of the cross bonds (bit k: bond k);
+  //   entry 1: n1 | n2 << 8 (active low bonds of class 1 and 2);
+  //   from entry 2: cross bond k's neighbour (s_lo with its low site flipped, in
+  //   the neighbouring popcount class), 2 entries or 6 with J2; then the active
+  //   class 1 neighbours (10 entries) and class 2, zero padded
+  uint16_t* rec[4];
   // [n_groups] per-group constants in schedule order (see GroupRec)
   struct GroupRec* grec;
 };
@@ -130,54 +128,29 @@ struct alignas(16) GroupRec {
 
 int build_geometry(const polfed_model* m, int b_override, HamGeometry* g);
 
-// A captured run of Clenshaw step launches (see filter_block).
-struct StepGraph {
-  int kind = 0, K = 0, lpr = 0;
-  double invD = 0.0, lo = 0.0, hi = 0.0;
-  uint64_t coef_hash = 0;
-  uint32_t wait_cap = 0;
-  const void *xs = nullptr, *ba = nullptr, *bb = nullptr;
-  cudaGraphExec_t exec = nullptr;  // null: key seen once, not captured yet
-  int64_t launches = 0;             // step launches of one replay
-  double alg_bytes = 0.0;           // their algorithmic bytes
-  int uses = 0;
-};
-
 class HamPlan {
  public:
   HamGeometry geo;
   HamTables tab{};
   void* dev = nullptr;       // one allocation for all tables
   int* err_flag = nullptr;   // set by a kernel whose bounded wait expired
-  // per-precision alpha/beta-scaled tables (F_lo, F_hi, C_x), indexed by dtype
+  unsigned bar_base = 0;     // arrivals counted so far on the grid barrier (err_flag + 16)
+  // per-precision alpha/beta-scaled tables (k_typed), indexed by dtype
   void* typed[3] = {nullptr, nullptr, nullptr};
-  size_t typed_bytes[3] = {0, 0, 0};
   bool typed_ok[3] = {false, false, false};
   double typed_lo[3] = {0, 0, 0}, typed_hi[3] = {0, 0, 0};
+  bool rec_ok[4] = {false, false, false, false};
   cudaStream_t stream = nullptr;
   bool stream_alloc = false;  // tables from cudaMallocAsync
-  std::vector<StepGraph> graphs;  // captured Clenshaw runs on this plan's tables (destroyed with it)
 
+  // All of these only enqueue work on the stream.
   int init(const polfed_model* m, cudaStream_t s, bool stream_ordered, int b_override = -1);
+  int bind(char* base, cudaStream_t s);                   // tables in caller memory (geo already set)
   int prepare_typed(int kind, double e_lo, double e_hi);  // alpha/beta-scaled tables
+  int prepare_rec(int lpr, cudaStream_t s);               // neighbour records for this lanes-per-row
   void release();
   ~HamPlan() { release(); }
 };
-
-// Arguments of one H~-slice kernel launch: out = cX*X + cH*(H~ b1) + cB*b2, all
-// operands slice-major (ld = W elements, W = VEC * LPR).
-struct StepArgs {
-  const void* b1;
-  const void* b2;  // may be null when cB == 0
-  const void* x;   // may be null when cX == 0
-  void* out;
-  double cX, cH, cB;
-  int lpr;         // lanes per row: slice = 16 * lpr bytes
-  const float* cxcol = nullptr;  // F32 only: per-column cX (device, W floats) in place of cX
-};
-
-// Launch one step (kind = POLFED_F32 / F64 / DF64 storage type).
-int launch_ham_step(const HamPlan& plan, int kind, const StepArgs& a, cudaStream_t s);
 
 // Elements per slice for a precision and lanes-per-row.
 int slice_width(int kind, int lpr);
@@ -186,14 +159,12 @@ size_t elem_bytes(int kind);  // internal storage element size (DF64: 8 = two fl
 // Filter engine over an arbitrary-width ABI block.  in/out are row-major
 // dim x n_b of "abi_kind" (POLFED_F32: float, else double).
 struct FilterScratch {
-  void* xs = nullptr;  // slice buffers (dim x W each)
-  void* ba = nullptr;
-  void* bb = nullptr;
+  void* xs = nullptr;     // slice buffers (dim x W each; see filter_scratch_bytes)
   float* flag = nullptr;  // [4] max |x|, max |y| (as float bits)
   size_t bytes = 0;
 };
 int filter_block(HamPlan& plan, int kind, const double* coeffs, int K, double invD, const void* in, void* out,
-                 int n_b, int abi_kind, FilterScratch& scr, cudaStream_t s, int lpr_hint = 0);
+                 int n_b, int abi_kind, FilterScratch& scr, cudaStream_t s);
 // FP32 filter with its own coefficients per column: out[:, j] = sum_n coef_j[n] T_n(H~) in[:, j].
 // The block is filtered in slices of W = slice_width(POLFED_F32, choose_lpr(POLFED_F32, n_b)) columns;
 // d_coef (device) holds, per slice q, (K + 1) rows of W floats:
@@ -201,15 +172,16 @@ int filter_block(HamPlan& plan, int kind, const double* coeffs, int K, double in
 int filter_block_cols(HamPlan& plan, const float* d_coef, int K, const void* in, void* out, int n_b, int abi_kind,
                       FilterScratch& scr, cudaStream_t s);
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
-                cudaStream_t s, int lpr_hint = 0);
-size_t filter_scratch_bytes(const HamPlan& plan, int kind, int lpr);
+                cudaStream_t s);
+size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 int choose_lpr(int kind, int n_b);
 
 // Batched filter: one cooperative launch runs the Clenshaw recurrences of
 // many (realization, 128-byte column slice) jobs, each with its own plan,
 // order and coefficients (F32 or DF64 storage; all jobs J2 == 0 or all not).
+constexpr int kBatchLpr = 8;  // 128-byte slices
 struct BatchFilterItem {
-  HamPlan* plan;          // prepare_typed(kind, ...) done
+  HamPlan* plan;          // prepare_typed(kind, ...) and prepare_rec(kBatchLpr, ...) done
   const double* coef;     // host, K + 1 coefficients: Y = invD * sum_n coef[n] T_n(H~) X
   int K;
   double invD;

@@ -1,0 +1,669 @@
+// Device code of the Clenshaw / H~ step: number policies, the group routine and
+// the step kernel (included by hamiltonian.cu only).
+#pragma once
+
+#include <type_traits>
+
+#include "polfed_internal.h"
+
+namespace polfed {
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Reads of the work item in shared memory are volatile: they are repeated where
+// they are used instead of being held in registers.
+__device__ __forceinline__ uint64_t lds64(const void* p) {
+  uint64_t v;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)));
+  return v;
+}
+__device__ __forceinline__ int lds32(const void* p) {
+  int v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)));
+  return v;
+}
+
+// --------------------------------------------------------- number policies
+// Float-float arithmetic: a value is hi + lo with |lo| <= ulp(hi)/2.
+// two_sum: Knuth (TAOCP vol. 2, 4.2.2); fast_two_sum: Dekker (1971);
+// products use the FMA-based exact product error.
+__device__ __forceinline__ float2 fast_two_sum(float a, float b) {
+  float s = a + b;
+  float e = b - (s - a);
+  return make_float2(s, e);
+}
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  float s = a + b;
+  float bb = s - a;
+  float e = (a - (s - bb)) + (b - bb);
+  return make_float2(s, e);
+}
+__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
+  float2 s = two_sum(a.x, b.x);
+  s.y += a.y + b.y;
+  return fast_two_sum(s.x, s.y);
+}
+__device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
+  float p = a.x * b.x;
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  return fast_two_sum(p, e);
+}
+
+// A policy works on 16-byte chunks of a row (int4 as loaded):
+//   S, C         storage element and constant type
+//   Acc          running sums over a row's neighbours (zero / add1 / add2: coupling class 1 / 2)
+//   Coef         the step's constants (make)
+//   fin          cX x + cH (d own + o1 sum1 + o2 sum2) + cB b2
+// FP32 and FP64 fold cH into the couplings and accumulate s_l v by FMA straight
+// into the result; float-float sums first and scales once (a float-float
+// product costs as much as two additions).
+
+// Typed constants of a job (StepJob::con), in the order of the enum.
+enum { kConS1, kConS2, kConS1Last, kConS2Last, kConInvD, kConN };
+
+struct RF32 {
+  using S = float;
+  using C = float;
+  struct Coef {
+    float s1, s2, cH, cX, cB;
+  };
+  struct Sum {
+    float s1, s2;
+  };
+  static __device__ __forceinline__ Sum load_sum(const Coef* k) {
+    return Sum{__int_as_float(lds32(&k->s1)), __int_as_float(lds32(&k->s2))};
+  }
+  static __device__ __forceinline__ Coef load_fin(const Coef* k) {
+    return Coef{0.f, 0.f, __int_as_float(lds32(&k->cH)), __int_as_float(lds32(&k->cX)), __int_as_float(lds32(&k->cB))};
+  }
+  template <bool J2>
+  struct Acc {
+    float2 p, q;
+  };
+  static __device__ __forceinline__ Coef make(const double* con, bool last, bool first, float cx) {
+    const float* f = reinterpret_cast<const float*>(con);
+    Coef k;
+    k.s1 = f[2 * (last ? kConS1Last : kConS1)];
+    k.s2 = f[2 * (last ? kConS2Last : kConS2)];
+    k.cH = last ? f[2 * kConInvD] : 2.f;
+    k.cB = first ? 0.f : (last ? -f[2 * kConInvD] : -1.f);
+    k.cX = cx;
+    return k;
+  }
+  static __device__ __forceinline__ bool has_x(const Coef& k) { return k.cX != 0.f; }
+  static __device__ __forceinline__ bool has_b(const Coef& k) { return k.cB != 0.f; }
+  template <bool J2>
+  static __device__ __forceinline__ void zero(Acc<J2>& a) {
+    a.p = a.q = make_float2(0.f, 0.f);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void fma(Acc<J2>& a, float s, const int4& u) {  // packed two-wide FMAs
+    const float2 ss = make_float2(s, s);
+    a.p = __ffma2_rn(ss, make_float2(__int_as_float(u.x), __int_as_float(u.y)), a.p);
+    a.q = __ffma2_rn(ss, make_float2(__int_as_float(u.z), __int_as_float(u.w)), a.q);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add1(Acc<J2>& a, const Sum& k, const int4& u) {
+    fma<J2>(a, k.s1, u);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add2(Acc<J2>& a, const Sum& k, const int4& u) {
+    fma<J2>(a, k.s2, u);
+  }
+  static __device__ __forceinline__ float add3(float a, float b, float c) { return a + b + c; }
+  // cxv: per-column cX of the lane's chunk (cols) instead of the step's scalar
+  template <bool J2>
+  static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, float d, const int4& own, const int4& x,
+                                             const int4& b, bool hx, bool hb, bool cols, const float4& cxv) {
+    fma<J2>(a, k.cH * d, own);
+    if (hx) {
+      if (cols) {
+        a.p = __ffma2_rn(make_float2(cxv.x, cxv.y), make_float2(__int_as_float(x.x), __int_as_float(x.y)), a.p);
+        a.q = __ffma2_rn(make_float2(cxv.z, cxv.w), make_float2(__int_as_float(x.z), __int_as_float(x.w)), a.q);
+      } else {
+        fma<J2>(a, k.cX, x);
+      }
+    }
+    if (hb) fma<J2>(a, k.cB, b);
+    return make_int4(__float_as_int(a.p.x), __float_as_int(a.p.y), __float_as_int(a.q.x), __float_as_int(a.q.y));
+  }
+};
+
+struct RF64 {
+  using S = double;
+  using C = double;
+  struct Coef {
+    double s1, s2, cH, cX, cB;
+  };
+  struct Sum {
+    double s1, s2;
+  };
+  static __device__ __forceinline__ Sum load_sum(const Coef* k) {
+    return Sum{__longlong_as_double(lds64(&k->s1)), __longlong_as_double(lds64(&k->s2))};
+  }
+  static __device__ __forceinline__ Coef load_fin(const Coef* k) {
+    return Coef{0.0, 0.0, __longlong_as_double(lds64(&k->cH)), __longlong_as_double(lds64(&k->cX)),
+                __longlong_as_double(lds64(&k->cB))};
+  }
+  template <bool J2>
+  struct Acc {
+    double p, q;
+  };
+  static __device__ __forceinline__ Coef make(const double* con, bool last, bool first, double cx) {
+    Coef k;
+    k.s1 = con[last ? kConS1Last : kConS1];
+    k.s2 = con[last ? kConS2Last : kConS2];
+    k.cH = last ? con[kConInvD] : 2.0;
+    k.cB = first ? 0.0 : (last ? -con[kConInvD] : -1.0);
+    k.cX = cx;
+    return k;
+  }
+  static __device__ __forceinline__ bool has_x(const Coef& k) { return k.cX != 0.0; }
+  static __device__ __forceinline__ bool has_b(const Coef& k) { return k.cB != 0.0; }
+  template <bool J2>
+  static __device__ __forceinline__ void zero(Acc<J2>& a) {
+    a.p = a.q = 0.0;
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void fma(Acc<J2>& a, double s, const int4& u) {
+    a.p = ::fma(s, __hiloint2double(u.y, u.x), a.p);
+    a.q = ::fma(s, __hiloint2double(u.w, u.z), a.q);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add1(Acc<J2>& a, const Sum& k, const int4& u) {
+    fma<J2>(a, k.s1, u);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add2(Acc<J2>& a, const Sum& k, const int4& u) {
+    fma<J2>(a, k.s2, u);
+  }
+  static __device__ __forceinline__ double add3(double a, double b, double c) { return a + b + c; }
+  template <bool J2>
+  static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, double d, const int4& own, const int4& x,
+                                             const int4& b, bool hx, bool hb, bool, const float4&) {
+    fma<J2>(a, k.cH * d, own);
+    if (hx) fma<J2>(a, k.cX, x);
+    if (hb) fma<J2>(a, k.cB, b);
+    return make_int4(__double2loint(a.p), __double2hiint(a.p), __double2loint(a.q), __double2hiint(a.q));
+  }
+};
+
+struct RDF {
+  using S = float2;  // (hi, lo)
+  using C = float2;
+  struct Coef {
+    float2 o1, o2, cH, cX, cB;
+    bool exact;  // cX, cH, cB are 0 or +-2^k: multiply hi and lo separately (exact)
+  };
+  struct Sum {};
+  static __device__ __forceinline__ Sum load_sum(const Coef*) { return Sum{}; }
+  static __device__ __forceinline__ Coef load_fin(const Coef* k) { return *k; }
+  template <bool J2>
+  struct Acc {
+    float2 a[2];  // per element (running hi sum, accumulated low parts and rounding errors)
+    float2 c[J2 ? 2 : 1];
+  };
+  static __device__ __forceinline__ bool pow2(float2 v) {
+    return v.y == 0.f && (__float_as_uint(v.x) & 0x7FFFFFu) == 0;
+  }
+  static __device__ __forceinline__ Coef make(const double* con, bool last, bool first, float2 cx) {
+    const float2* f = reinterpret_cast<const float2*>(con);
+    Coef k;
+    k.o1 = f[kConS1];
+    k.o2 = f[kConS2];
+    const float2 iv = f[kConInvD];
+    k.cH = last ? iv : make_float2(2.f, 0.f);
+    k.cB = first ? make_float2(0.f, 0.f) : (last ? make_float2(-iv.x, -iv.y) : make_float2(-1.f, 0.f));
+    k.cX = cx;
+    k.exact = pow2(k.cX) && pow2(k.cH) && pow2(k.cB);
+    return k;
+  }
+  static __device__ __forceinline__ bool has_x(const Coef& k) { return k.cX.x != 0.f; }
+  static __device__ __forceinline__ bool has_b(const Coef& k) { return k.cB.x != 0.f; }
+  template <bool J2>
+  static __device__ __forceinline__ void zero(Acc<J2>& a) {
+    a.a[0] = a.a[1] = make_float2(0.f, 0.f);
+    if constexpr (J2) a.c[0] = a.c[1] = make_float2(0.f, 0.f);
+  }
+  static __device__ __forceinline__ void acc(float2& a, int hi, int lo) {
+    const float2 s = two_sum(a.x, __int_as_float(hi));
+    a.x = s.x;
+    a.y += s.y + __int_as_float(lo);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add1(Acc<J2>& a, const Sum&, const int4& u) {
+    acc(a.a[0], u.x, u.y);
+    acc(a.a[1], u.z, u.w);
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add2(Acc<J2>& a, const Sum&, const int4& u) {
+    acc(a.c[0], u.x, u.y);
+    acc(a.c[J2 ? 1 : 0], u.z, u.w);
+  }
+  static __device__ __forceinline__ float2 add3(float2 a, float2 b, float2 c) { return df_add(df_add(a, b), c); }
+  template <bool J2>
+  static __device__ __forceinline__ float2 one(float2 s1, float2 s2, const Coef& k, float2 d, float2 own, float2 x,
+                                               float2 b, bool hx, bool hb) {
+    float2 y = df_add(df_mul(d, own), df_mul(k.o1, fast_two_sum(s1.x, s1.y)));
+    if constexpr (J2) y = df_add(y, df_mul(k.o2, fast_two_sum(s2.x, s2.y)));
+    if (k.exact) {
+      float2 r = make_float2(k.cH.x * y.x, k.cH.x * y.y);
+      if (hx) r = df_add(r, make_float2(k.cX.x * x.x, k.cX.x * x.y));
+      if (hb) r = df_add(r, make_float2(k.cB.x * b.x, k.cB.x * b.y));
+      return r;
+    }
+    float2 r = df_mul(k.cH, y);
+    if (hx) r = df_add(r, df_mul(k.cX, x));
+    if (hb) r = df_add(r, df_mul(k.cB, b));
+    return r;
+  }
+  template <bool J2>
+  static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, float2 d, const int4& own, const int4& x,
+                                             const int4& b, bool hx, bool hb, bool, const float4&) {
+    auto lo = [](const int4& v) { return make_float2(__int_as_float(v.x), __int_as_float(v.y)); };
+    auto hi = [](const int4& v) { return make_float2(__int_as_float(v.z), __int_as_float(v.w)); };
+    const float2 r0 = one<J2>(a.a[0], a.c[0], k, d, lo(own), lo(x), lo(b), hx, hb);
+    const float2 r1 = one<J2>(a.a[1], a.c[J2 ? 1 : 0], k, d, hi(own), hi(x), hi(b), hx, hb);
+    return make_int4(__float_as_int(r0.x), __float_as_int(r0.y), __float_as_int(r1.x), __float_as_int(r1.y));
+  }
+};
+
+// ------------------------------------------------------------------- jobs
+// One column slice of one operator going through its Clenshaw steps.
+struct StepJob {
+  const uint16_t* rec;  // neighbour records (k_tables_rec)
+  const GroupRec* grec;
+  const void* Fc;       // typed, alpha-scaled diagonal of the low part, by cls_off + local index
+  const void* Fhi;      // of the high part (schedule order, includes -alpha*beta)
+  const void* Cx;       // of the cross bonds, by pattern
+  const void* cx;       // typed cX in step order (a job of StepRun::jobs)
+  const float* colcx;   // FP32: per-column cX, row n = order n (W floats each), or null
+  char *xs, *ba, *bb;   // x, b_{k+1}, b_{k+2} (overwritten by b_k)
+  double con[kConN];    // typed constants (each in its own 8 bytes)
+  int K, n_groups, n_cross, c2mask;
+};
+
+constexpr int kParamSteps = 448;  // step coefficients that travel in the kernel parameters
+
+struct StepRun {
+  StepJob one;            // jobs == nullptr: n_jobs slices of this operator, buffers `stride` bytes apart
+  const StepJob* jobs;
+  int n_jobs;
+  int st0, st1;           // steps of this launch
+  int64_t stride, colstride;
+  unsigned* bar;          // arrivals of the grid barrier, bar_base before this launch
+  unsigned bar_base;
+  uint32_t cap;
+  int* err;
+  double cx[kParamSteps]; // jobs == nullptr: cX of the steps from st0 on, each in its own 8 bytes
+};
+
+// ------------------------------------------------------------ memory helpers
+__device__ __forceinline__ void cp_async16(void* s, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// L2 only: earlier steps of the same launch wrote these rows from other SMs
+__device__ __forceinline__ int4 ld_l2(const char* p) {
+  int4 v;
+  asm volatile("ld.global.cg.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+// tables: cached in L1, repeated at the place of use (volatile) to keep registers free
+__device__ __forceinline__ uint4 ld_tab(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int4 ld_stream(const char* p) {
+  int4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.s32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// ---------------------------------------------------------------- step kernel
+constexpr int kTeam = 128;       // threads of a team (4 warps, one group at a time)
+constexpr int kMaxTeams = 6;     // 768 threads at 80 registers
+
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(kTeam) : "memory");
+}
+// What a team needs for its group, in shared memory (double buffered).
+template <class NT>
+struct alignas(16) WorkItem {
+  GroupRec g;
+  typename NT::C fhi;
+  int64_t pad;
+  const char *b1, *x, *rec, *fc, *cxt, *col;  // col: the step's per-column cX
+  char* out;                                  // and b2
+  typename NT::Coef k;
+  int n_cross, c2mask, flags;                 // flags: 1 = reads x, 2 = reads b2
+};
+
+// One step of one group (the rows sharing s_hi) by a team:
+//   out = cX x + cH (H~ b1) + cB b2,  out in place of b2.
+template <class NT, int LPR, bool J2, bool COLS, int RMAX>
+struct GroupStep {
+  using C = typename NT::C;
+  using Acc = typename NT::template Acc<J2>;
+  using Coef = typename NT::Coef;
+  using Item = WorkItem<NT>;
+  static constexpr int ROWB = 16 * LPR;
+  static constexpr int RPW = 32 / LPR;             // rows of a warp's block
+  static constexpr int NW = kTeam / 32;
+  static constexpr int MAXCR = J2 ? 6 : 2;
+  static constexpr int RS = J2 ? 32 : 16;          // uint16 entries of a record
+  static constexpr int RSB = 2 * RS;
+  static constexpr int HU = 2;                     // high neighbours in flight per row
+  static constexpr int STEP = kTeam * 16;          // bytes between a thread's consecutive rows
+
+  template <int R>
+  static __device__ __forceinline__ void pass(const Item* I, int blk, int n_g, const unsigned char* tile, bool& ready,
+                                              int team) {
+    const int l32 = threadIdx.x & 31, lane16 = (l32 % LPR) * 16;
+    int row = blk * RPW + l32 / LPR;
+    bool live = true;
+    if constexpr (R == 1) {
+      live = row < n_g;
+      row = min(row, n_g - 1);
+    }
+    const uint32_t ro = (uint32_t)(row * ROWB + lane16);
+    const size_t goff = (size_t)(uint32_t)lds32(&I->g.r0) * ROWB + ro;
+    const int flags = lds32(&I->flags);
+    const bool hx = flags & 1, hb = flags & 2;
+    const typename NT::Sum k = NT::load_sum(&I->k);
+    Acc acc[R];
+    int4 xv[R], bv[R];
+#pragma unroll
+    for (int i = 0; i < R; i++) NT::template zero<J2>(acc[i]);
+    if (hx) {
+      const char* p = (const char*)lds64(&I->x) + goff;
+#pragma unroll
+      for (int i = 0; i < R; i++) xv[i] = ld_stream(p + i * STEP);
+    }
+    if (hb) {
+      const char* p = (const char*)lds64(&I->out) + goff;
+#pragma unroll
+      for (int i = 0; i < R; i++) bv[i] = ld_l2(p + i * STEP);
+    }
+    // high bonds: the same local rows of other groups
+    const char* b1 = (const char*)lds64(&I->b1);
+    auto add = [&](Acc& a, bool c1, const int4& u) {
+      if (!J2 || c1)
+        NT::template add1<J2>(a, k, u);
+      else
+        NT::template add2<J2>(a, k, u);
+    };
+    {
+      const char* hp = b1 + ro;
+      auto high = [&](int k0, int k1, bool c1) {
+        int kk = k0;
+        for (; kk + HU <= k1; kk += HU) {
+          int4 u[HU][R];
+#pragma unroll
+          for (int j = 0; j < HU; j++) {
+            const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk + j]) * ROWB;
+#pragma unroll
+            for (int i = 0; i < R; i++) u[j][i] = ld_l2(p + i * STEP);
+          }
+#pragma unroll
+          for (int j = 0; j < HU; j++)
+#pragma unroll
+            for (int i = 0; i < R; i++) add(acc[i], c1, u[j][i]);
+        }
+        for (; kk < k1; kk++) {
+          int4 u[R];
+          const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk]) * ROWB;
+#pragma unroll
+          for (int i = 0; i < R; i++) u[i] = ld_l2(p + i * STEP);
+#pragma unroll
+          for (int i = 0; i < R; i++) add(acc[i], c1, u[i]);
+        }
+      };
+      const int n_hn1 = lds32(&I->g.n_hn1);
+      high(0, n_hn1, true);
+      if constexpr (J2) high(n_hn1, lds32(&I->g.n_hn), false);
+    }
+    // neighbour records of the rows: header and cross neighbours
+    const char* rp0 = (const char*)lds64(&I->rec) + (size_t)(uint32_t)((lds32(&I->g.cls_base) + row) * RSB);
+    constexpr int RSTEP = kTeam / LPR * RSB;
+    uint4 hd[R];
+#pragma unroll
+    for (int i = 0; i < R; i++) hd[i] = ld_tab(rp0 + i * RSTEP);
+    auto half = [](const uint4& v, int e) {  // entry e = 0..7 of a 16-byte piece
+      const uint32_t x = e < 2 ? v.x : (e < 4 ? v.y : (e < 6 ? v.z : v.w));
+      return (e & 1) ? (x >> 16) : (x & 0xFFFFu);
+    };
+    // cross bonds: rows of another group, where the bond is antiparallel
+    uint32_t pat[R];
+    const int n_cross = lds32(&I->n_cross);
+    {
+      const uint32_t need = (uint32_t)lds32(&I->g.need_mask);
+#pragma unroll
+      for (int i = 0; i < R; i++) pat[i] = ~(half(hd[i], 0) ^ need) & ((1u << n_cross) - 1u);
+    }
+#pragma unroll
+    for (int c = 0; c < MAXCR; c++) {
+      if (c < n_cross) {
+        const char* p = b1 + lane16 + (size_t)(uint32_t)lds32(&I->g.cr_base[c]) * ROWB - ROWB;
+        const bool c1 = !J2 || !((lds32(&I->c2mask) >> c) & 1);
+        int4 u[R];
+#pragma unroll
+        for (int i = 0; i < R; i++)
+          if ((pat[i] >> c) & 1) u[i] = ld_l2(p + half(hd[i], 2 + c));
+#pragma unroll
+        for (int i = 0; i < R; i++)
+          if ((pat[i] >> c) & 1) add(acc[i], c1, u[i]);
+      }
+    }
+    if (!ready) {
+      cp_async_wait();
+      team_sync(team);
+      ready = true;
+    }
+    // low bonds: rows of the staged group; lists are padded with the zero row at tile offset 0
+    const unsigned char* tl = tile + lane16;
+    auto low = [&](Acc& a, bool c1, uint32_t e0, uint32_t e1) {
+      const int4 u0 = *reinterpret_cast<const int4*>(tl + e0), u1 = *reinterpret_cast<const int4*>(tl + e1);
+      add(a, c1, u0);
+      add(a, c1, u1);
+    };
+#pragma unroll
+    for (int i = 0; i < R; i++) {
+      const uint32_t cnt = half(hd[i], 1);
+      const int n1 = __reduce_max_sync(~0u, cnt & 0xFF);
+      const char* rp = rp0 + i * RSTEP;
+      if constexpr (J2) {
+        const int n2 = __reduce_max_sync(~0u, cnt >> 8);
+        const uint4 q1 = ld_tab(rp + 16), q2 = ld_tab(rp + 32);
+        if (n1 > 0) low(acc[i], true, half(q1, 0), half(q1, 1));
+        if (n1 > 2) low(acc[i], true, half(q1, 2), half(q1, 3));
+        if (n1 > 4) low(acc[i], true, half(q1, 4), half(q1, 5));
+        if (n1 > 6) low(acc[i], true, half(q1, 6), half(q1, 7));
+        if (n1 > 8) low(acc[i], true, half(q2, 0), half(q2, 1));
+        const uint4 q3 = ld_tab(rp + 48);
+        if (n2 > 0) low(acc[i], false, half(q2, 2), half(q2, 3));
+        if (n2 > 2) low(acc[i], false, half(q2, 4), half(q2, 5));
+        if (n2 > 4) low(acc[i], false, half(q2, 6), half(q2, 7));
+        if (n2 > 6) low(acc[i], false, half(q3, 0), half(q3, 1));
+        if (n2 > 8) low(acc[i], false, half(q3, 2), half(q3, 3));
+      } else {
+        if (n1 > 0) low(acc[i], true, half(hd[i], 4), half(hd[i], 5));
+        if (n1 > 2) low(acc[i], true, half(hd[i], 6), half(hd[i], 7));
+        if (n1 > 4) {
+          const uint4 q1 = ld_tab(rp + 16);
+          low(acc[i], true, half(q1, 0), half(q1, 1));
+          if (n1 > 6) low(acc[i], true, half(q1, 2), half(q1, 3));
+          if (n1 > 8) low(acc[i], true, half(q1, 4), half(q1, 5));
+        }
+      }
+    }
+    {
+      const C* fc = (const C*)lds64(&I->fc) + lds32(&I->g.cls_base) + row;
+      const C* cxt = (const C*)lds64(&I->cxt);
+      char* out = (char*)lds64(&I->out) + goff;
+      float4 cxv = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (COLS) cxv = __ldg(reinterpret_cast<const float4*>((const char*)lds64(&I->col) + lane16));
+      const C fhi = I->fhi;
+      const Coef kf = NT::load_fin(&I->k);
+#pragma unroll
+      for (int i = 0; i < R; i++) {
+        const C d = NT::add3(__ldg(fc + i * (kTeam / LPR)), fhi, __ldg(cxt + pat[i]));
+        const int4 own = *reinterpret_cast<const int4*>(tile + ROWB + ro + i * STEP);
+        const int4 r = NT::template fin<J2>(acc[i], kf, d, own, xv[i], bv[i], hx, hb, COLS, cxv);
+        if (R > 1 || live) __stcg(reinterpret_cast<int4*>(out + i * STEP), r);
+      }
+    }
+  }
+
+  static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w) {
+    const int n_g = lds32(&I->g.n_g);
+    {
+      const char* src = (const char*)lds64(&I->b1) + (size_t)(uint32_t)lds32(&I->g.r0) * ROWB;
+      const int nb = n_g * ROWB;
+      for (int c = (threadIdx.x % kTeam) * 16; c < nb; c += STEP) cp_async16(tile + ROWB + c, src + c);
+      cp_async_commit();
+    }
+    bool ready = false;
+    const int nblk = (n_g + RPW - 1) / RPW, nfull = n_g / RPW;
+    int blk = w;
+    if constexpr (RMAX >= 2)
+      for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team);
+    for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team);
+    if (!ready) {
+      cp_async_wait();
+      team_sync(team);
+    }
+  }
+};
+
+// Grid barrier of a cooperative launch: arrivals are counted on one monotone
+// counter; waits are bounded (cap polls), a wait that runs out sets *err and
+// every CTA leaves at its next barrier.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int* err, uint32_t cap) {
+  __syncthreads();
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    uint32_t it = 0;
+    while ((int)(*(volatile unsigned*)count - target) < 0) {
+      if (++it > cap) {
+        atomicExch(err, 1);
+        ok = 0;
+        break;
+      }
+      if ((it & 15) == 0) {
+        if (*(volatile int*)err) {
+          ok = 0;
+          break;
+        }
+        __nanosleep(64);
+      }
+    }
+    __threadfence();
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// Steps st0..st1-1 of every job with st < K.  Work items are (job, group)
+// pairs, groups largest first, dealt to the teams of all CTAs in alternating
+// direction; CTAs meet at the grid barrier between steps.  The record of a
+// team's next group is fetched while the current one is worked on.
+//
+// What bounds it.  A row reads 9.3 rows of 128 bytes through L2 at L = 22 XXZ
+// (itself 1, high bonds 5.8, cross bonds 1, b2 1, x on half of the steps) and
+// 5 more from the staged group: 0.84 GB per step against the 0.32 GB a step
+// cannot do without, of which 0.40 GB come from DRAM.  The time is the latency
+// of those loads (long-scoreboard stalls; issue slots 30%, L2 28%, DRAM 57%
+// busy), so the kernel holds as many independent warps as its registers allow
+// (six teams of four per SM, each with its own group and barrier), keeps
+// uniform values in shared memory and reads everything but the own group
+// straight into registers.  A bulk-copy ring that staged every neighbour block
+// was slower (129 us per step at L = 22; 360 instead of 190 instructions per
+// four rows), deeper per-warp prefetch was too (the scoreboards of a warp make
+// its loads wait for one another).
+// Many steps per launch save a launch of about 5 us each, which at L <= 18 is
+// most of the step: the barrier costs 1.4 us.
+// Measured, us per step and slice of 128 bytes (one launch per step before):
+// L = 14 FP64 37 -> 6.3, L = 18 float-float 28 -> 9, L = 20 J1-J2 float-float
+// 91 -> 66, L = 20 J1-J2 FP32 71 -> 40, L = 22 FP32 128 -> 111, L = 24 J1-J2
+// FP32 1183 -> 800.
+template <class NT, int LPR, bool J2, bool COLS>
+__global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_constant__ StepRun R, int tile_bytes) {
+  using C = typename NT::C;
+  using Item = WorkItem<NT>;
+  constexpr int RMAX = (std::is_same<NT, RDF>::value) ? 1 : 2;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int team = threadIdx.x / kTeam, tt = threadIdx.x % kTeam;
+  unsigned char* tile = smem + (size_t)team * tile_bytes;
+  Item* items = reinterpret_cast<Item*>(smem + (size_t)(blockDim.x / kTeam) * tile_bytes) + 2 * team;
+  const int n_teams = (blockDim.x / kTeam) * gridDim.x;
+  const int me = team * gridDim.x + blockIdx.x;  // neighbouring items go to different SMs
+  if (tt < LPR) *reinterpret_cast<int4*>(tile + tt * 16) = make_int4(0, 0, 0, 0);  // the zero row
+  unsigned target = R.bar_base;
+  for (int st = R.st0; st < R.st1; st++) {
+    int j = 0, base = 0, r = 0;
+    // fetch the r-th item of this team into items[r & 1]; false if there is none
+    auto fetch = [&]() -> bool {
+      const int item = r * n_teams + ((r & 1) ? n_teams - 1 - me : me);
+      const StepJob* J = nullptr;
+      for (; j < R.n_jobs; j++) {
+        J = R.jobs ? R.jobs + j : &R.one;
+        const int ng = st < J->K ? J->n_groups : 0;
+        if (item < base + ng) break;
+        base += ng;
+      }
+      if (j >= R.n_jobs) return false;
+      Item* I = items + (r & 1);
+      const int gidx = item - base;
+      constexpr int NG = sizeof(GroupRec) / 16;
+      if (tt < NG) cp_async16(reinterpret_cast<char*>(&I->g) + tt * 16, reinterpret_cast<const char*>(J->grec + gidx) + tt * 16);
+      if (tt == NG)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(&I->fhi)),
+                     "l"(reinterpret_cast<const C*>(J->Fhi) + gidx), "n"(sizeof(C))
+                     : "memory");
+      cp_async_commit();
+      if (tt == 32) {
+        const size_t so = R.jobs ? 0 : (size_t)j * R.stride;
+        I->b1 = ((st & 1) ? J->bb : J->ba) + so;
+        I->out = ((st & 1) ? J->ba : J->bb) + so;
+        I->x = J->xs + so;
+        I->rec = reinterpret_cast<const char*>(J->rec);
+        I->fc = reinterpret_cast<const char*>(J->Fc);
+        I->cxt = reinterpret_cast<const char*>(J->Cx);
+        I->n_cross = J->n_cross;
+        I->c2mask = J->c2mask;
+        const int kk = J->K - 1 - st;
+        C cx = C();
+        if constexpr (COLS)
+          I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * (4 * LPR));
+        else
+          cx = R.jobs ? __ldg(reinterpret_cast<const C*>(J->cx) + st) : *reinterpret_cast<const C*>(&R.cx[st - R.st0]);
+        const typename NT::Coef k = NT::make(J->con, kk == 0, st == 0, cx);
+        I->k = k;
+        I->flags = (COLS || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
+      }
+      return true;
+    };
+    bool more = fetch();
+    while (more) {
+      cp_async_wait();
+      team_sync(team);  // the item is complete, the previous group's tile is no longer read
+      const Item* I = items + (r & 1);
+      r++;
+      more = fetch();
+      GroupStep<NT, LPR, J2, COLS, RMAX>::run(I, tile, team, tt >> 5);
+    }
+    if (st + 1 < R.st1) {
+      target += gridDim.x;
+      if (!grid_barrier(R.bar, target, R.err, R.cap)) return;
+    }
+  }
+}
+
+}  // namespace polfed
