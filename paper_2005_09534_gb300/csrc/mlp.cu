@@ -2,12 +2,15 @@
 // connected FP32 network, x -> tanh(W1 x' + b1) -> tanh(W2 . + b2) -> W3 . + b3,
 // with x' = (x - x_mean) / x_std and outputs in standardized target units.
 // Forward, backward (hand-derived; deterministic reductions, no atomics) and
-// the Adam update are plain CUDA kernels: the network is tiny (about 20k
-// parameters), so each kernel maps one thread to one output, one parameter
-// gradient or one activation.
+// the Adam update are plain CUDA kernels.  The network is tiny (about 20k
+// parameters), so launches and serial sums are what it costs: with up to
+// kFusedMax inputs and hidden units a gradient takes three kernels (everything
+// of a batch row; the weight gradients, split over the batch; their sum with
+// the Adam update).  Wider networks keep one kernel per layer.
 //
 // Parameter layout (one contiguous float array):
 //   W1 [H x d_in] row-major, b1 [H], W2 [H x H], b2 [H], W3 [d_out x H], b3 [d_out].
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -153,6 +156,264 @@ __global__ void k_mlp_init(float* p, int n, uint64_t seed, int d_in, int H, int 
   p[e] = a * u;
 }
 
+// ------------------------------------------------------- fused batch rows
+constexpr int kFusedMax = 512;  // inputs and hidden units of the fused kernels
+constexpr int kRowThreads = 256;
+
+struct RowArgs {
+  const float *W1, *b1, *W2, *b2, *W3, *b3, *xm, *xinv, *ym, *ysd;
+  const float *x, *t;  // t == nullptr: forward only
+  float *xs, *a1, *a2, *dy, *dz2, *dz1, *lossp, *y;
+  int B, d_in, H, d_out;
+};
+
+// out[j * TB + r] = sum_i W[j * n_in + i] in[i * TB + r]: a warp takes 16 / TB
+// rows of W at a time (lanes along i, coalesced) for all TB batch rows and
+// reduces its 16 sums by exchanging halves.  fin(j, r, sum) consumes them.
+template <int TB, class F>
+__device__ __forceinline__ void rows_dot(const float* __restrict__ W, const float* in, int n_in, int n_out, F fin) {
+  constexpr int JT = 16 / TB;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int j0 = warp * JT; j0 < n_out; j0 += JT * (kRowThreads / 32)) {
+    float v[16];
+#pragma unroll
+    for (int q = 0; q < 16; q++) v[q] = 0.f;
+#pragma unroll 4
+    for (int i = lane; i < n_in; i += 32) {
+      float xr[TB];
+#pragma unroll
+      for (int r = 0; r < TB; r += 4) *reinterpret_cast<float4*>(xr + r) = *reinterpret_cast<const float4*>(in + i * TB + r);
+#pragma unroll
+      for (int j = 0; j < JT; j++) {
+        const float w = j0 + j < n_out ? __ldg(W + (size_t)(j0 + j) * n_in + i) : 0.f;
+#pragma unroll
+        for (int r = 0; r < TB; r++) v[j * TB + r] = fmaf(w, xr[r], v[j * TB + r]);
+      }
+    }
+#pragma unroll
+    for (int m = 16, c = 8; m >= 2; m >>= 1, c >>= 1) {
+      const bool up = lane & m;
+#pragma unroll
+      for (int q = 0; q < 8; q++)
+        if (q < c) {
+          const float send = up ? v[q] : v[q + c], keep = up ? v[q + c] : v[q];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+    const float s = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+    const int idx = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+    const int j = j0 + idx / TB;
+    if (!(lane & 1) && j < n_out) fin(j, idx % TB, s);
+  }
+}
+
+// Everything of TB batch rows: standardization, the three layers, the output
+// delta and loss, and the deltas of both hidden layers.  Bound by latency (a
+// CTA's chain of dot products; the weights come from L2, read once per CTA).
+// 23 inputs, 2 x 128 hidden units, batch 256: a whole gradient call 194 -> 45 us,
+// this kernel 12, the weight gradients 4.5 (101 before, serial over the batch),
+// their sum 2 us.
+template <int TB>
+__global__ void __launch_bounds__(kRowThreads) k_mlp_rows(const RowArgs A) {
+  extern __shared__ __align__(16) float sh[];
+  const int H = A.H, b0 = blockIdx.x * TB, tid = threadIdx.x;
+  float* sx = sh;                    // [d_in][TB]
+  float* s1 = sx + A.d_in * TB;      // [H][TB] a1
+  float* s2 = s1 + H * TB;           // a2
+  float* sd = s2 + H * TB;           // dz2
+  float* so = sd + H * TB;           // [d_out][TB] dy
+  float* sl = so + A.d_out * TB;     // loss terms
+  for (int e = tid; e < A.d_in * TB; e += kRowThreads) {
+    const int r = e / A.d_in, i = e - r * A.d_in;
+    float v = 0.f;
+    if (b0 + r < A.B) {
+      const size_t g = (size_t)(b0 + r) * A.d_in + i;
+      v = (A.x[g] - A.xm[i]) * A.xinv[i];
+      if (A.t) A.xs[g] = v;
+    }
+    sx[i * TB + r] = v;
+  }
+  __syncthreads();
+  rows_dot<TB>(A.W1, sx, A.d_in, H, [&](int j, int r, float s) {
+    s = tanhf(s + A.b1[j]);
+    s1[j * TB + r] = s;
+    if (A.t && b0 + r < A.B) A.a1[(size_t)(b0 + r) * H + j] = s;
+  });
+  __syncthreads();
+  rows_dot<TB>(A.W2, s1, H, H, [&](int j, int r, float s) {
+    s = tanhf(s + A.b2[j]);
+    s2[j * TB + r] = s;
+    if (A.t && b0 + r < A.B) A.a2[(size_t)(b0 + r) * H + j] = s;
+  });
+  __syncthreads();
+  rows_dot<TB>(A.W3, s2, H, A.d_out, [&](int o, int r, float s) {
+    s += A.b3[o];
+    const bool in = b0 + r < A.B;
+    const size_t g = (size_t)(b0 + r) * A.d_out + o;
+    if (!A.t) {
+      if (in) A.y[g] = fmaf(s, A.ysd[o], A.ym[o]);
+      return;
+    }
+    const float e = in ? s - (A.t[g] - A.ym[o]) / A.ysd[o] : 0.f;
+    const float dy = e / (float)A.B;
+    so[o * TB + r] = dy;
+    sl[o * TB + r] = 0.5f * e * e / (float)A.B;
+    if (in) A.dy[g] = dy;
+  });
+  if (!A.t) return;
+  __syncthreads();
+  if (tid == 0) {
+    float l = 0.f;
+    for (int q = 0; q < A.d_out * TB; q++) l += sl[q];
+    A.lossp[blockIdx.x] = l;
+  }
+  // dz2 = (W3^T dy) (1 - a2^2)
+  for (int i = tid; i < H; i += kRowThreads) {
+    float z[TB];
+#pragma unroll
+    for (int r = 0; r < TB; r++) z[r] = 0.f;
+    for (int o = 0; o < A.d_out; o++) {
+      const float w = __ldg(A.W3 + (size_t)o * H + i);
+#pragma unroll
+      for (int r = 0; r < TB; r++) z[r] = fmaf(w, so[o * TB + r], z[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < TB; r++) {
+      const float a = s2[i * TB + r];
+      z[r] *= 1.f - a * a;
+      sd[i * TB + r] = z[r];
+      if (b0 + r < A.B) A.dz2[(size_t)(b0 + r) * H + i] = z[r];
+    }
+  }
+  __syncthreads();
+  // dz1 = (W2^T dz2) (1 - a1^2): one thread per (hidden unit, share of the sum); shares meet in s2
+  const int Hr = (H + 31) & ~31, ng = Hr >= kRowThreads ? 1 : kRowThreads / Hr;
+  const int g = Hr >= kRowThreads ? 0 : tid / Hr;
+  for (int i = Hr >= kRowThreads ? tid : tid - g * Hr; i < H; i += kRowThreads) {
+    if (g >= ng) break;
+    float z[TB];
+#pragma unroll
+    for (int r = 0; r < TB; r++) z[r] = 0.f;
+    const int jn = (H + ng - 1) / ng, j1 = min(H, (g + 1) * jn);
+#pragma unroll 8
+    for (int j = g * jn; j < j1; j++) {
+      const float w = __ldg(A.W2 + (size_t)j * H + i);
+#pragma unroll
+      for (int r = 0; r < TB; r += 4) {
+        const float4 d = *reinterpret_cast<const float4*>(sd + j * TB + r);
+        z[r] = fmaf(w, d.x, z[r]);
+        z[r + 1] = fmaf(w, d.y, z[r + 1]);
+        z[r + 2] = fmaf(w, d.z, z[r + 2]);
+        z[r + 3] = fmaf(w, d.w, z[r + 3]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < TB; r++) (g == 0 ? s2 : sl + A.d_out * TB + (size_t)(g - 1) * H * TB)[i * TB + r] = z[r];
+  }
+  __syncthreads();
+  for (int e = tid; e < H * TB; e += kRowThreads) {
+    const int r = e / H, i = e - r * H;
+    float z = s2[i * TB + r];
+    for (int q = 1; q < ng; q++) z += sl[A.d_out * TB + (size_t)(q - 1) * H * TB + i * TB + r];
+    const float a = s1[i * TB + r];
+    if (b0 + r < A.B) A.dz1[(size_t)(b0 + r) * H + i] = z * (1.f - a * a);
+  }
+}
+
+size_t rows_smem(int TB, int d_in, int H, int d_out) {
+  const int Hr = (H + 31) & ~31, ng = Hr >= kRowThreads ? 1 : kRowThreads / Hr;
+  return (size_t)TB * (d_in + 3 * H + 2 * d_out + (ng - 1) * H) * sizeof(float);
+}
+
+// One of the three weight matrices: dW[j][i] = sum_b dz[b][j] in[b][i], db[j] = sum_b dz[b][j].
+struct WMat {
+  const float *dz, *in;
+  int n_in, n_out, off_w, off_b, tile0;  // offsets in the parameters, first tile
+};
+struct WArgs {
+  WMat m[3];
+  int B, rows;  // rows of the batch per split
+  int64_t n_params;
+  float* part;  // [splits][n_params]
+};
+
+// 32 x 32 tiles of the weight gradients over one share of the batch.
+__global__ void __launch_bounds__(256) k_mlp_wgrad_tiles(const WArgs A) {
+  __shared__ __align__(16) float sz[32][32], si[32][32];
+  int q = 2;
+  while (q > 0 && (int)blockIdx.x < A.m[q].tile0) q--;
+  const WMat m = A.m[q];
+  const int tcols = (m.n_in + 31) / 32, tl = blockIdx.x - m.tile0;
+  const int j0 = (tl / tcols) * 32, i0 = (tl % tcols) * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int b0 = blockIdx.y * A.rows, b1 = min(A.B, b0 + A.rows);
+  float acc[4] = {0.f, 0.f, 0.f, 0.f}, ab[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int b = b0; b < b1; b += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const int r = ty + 8 * u;
+      const bool in = b + r < b1;
+      sz[r][tx] = in && j0 + tx < m.n_out ? m.dz[(size_t)(b + r) * m.n_out + j0 + tx] : 0.f;
+      si[r][tx] = in && i0 + tx < m.n_in ? m.in[(size_t)(b + r) * m.n_in + i0 + tx] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int r = 0; r < 32; r++) {
+      const float4 z = *reinterpret_cast<const float4*>(&sz[r][ty * 4]);
+      const float x = si[r][tx];
+      acc[0] = fmaf(z.x, x, acc[0]);
+      acc[1] = fmaf(z.y, x, acc[1]);
+      acc[2] = fmaf(z.z, x, acc[2]);
+      acc[3] = fmaf(z.w, x, acc[3]);
+      ab[0] += z.x;
+      ab[1] += z.y;
+      ab[2] += z.z;
+      ab[3] += z.w;
+    }
+  }
+  float* P = A.part + blockIdx.y * A.n_params;
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const int j = j0 + ty * 4 + u, i = i0 + tx;
+    if (j < m.n_out && i < m.n_in) P[m.off_w + (size_t)j * m.n_in + i] = acc[u];
+    if (j < m.n_out && i == 0) P[m.off_b + j] = ab[u];
+  }
+}
+
+// Sum of the shares in order, the Adam update if lr > 0, and (last CTA) the loss.
+__global__ void k_mlp_combine(const float* __restrict__ part, int splits, int n, float* __restrict__ grad,
+                              float* __restrict__ out, const float* __restrict__ lossp, int n_loss,
+                              float* __restrict__ loss, float* __restrict__ p, float* __restrict__ m,
+                              float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
+  __shared__ float sh[256];
+  if (blockIdx.x == gridDim.x - 1) {
+    float s = 0.f;
+    for (int i = threadIdx.x; i < n_loss; i += 256) s += lossp[i];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o; o >>= 1) {
+      if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = sh[0];
+    return;
+  }
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= n) return;
+  float s = 0.f;
+  for (int q = 0; q < splits; q++) s += part[(size_t)q * n + e];
+  grad[e] = s;
+  if (out) out[e] = s;
+  if (lr > 0.f) {
+    const float mi = b1 * m[e] + (1.f - b1) * s;
+    const float vi = b2 * v[e] + (1.f - b2) * s * s;
+    m[e] = mi;
+    v[e] = vi;
+    p[e] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  }
+}
+
 unsigned nblk(int n) { return (unsigned)((n + 255) / 256); }
 
 struct Views {
@@ -183,12 +444,21 @@ Views views(const polfed_mlp* n) {
 }
 
 // Work buffer: xs [B d_in] | a1 [B H] | a2 [B H] | y [B d_out] | dy [B d_out] | dz2 [B H] | dz1 [B H] | loss [1]
+// | loss terms and gradient shares of the fused kernels
 struct Work {
-  float *xs, *a1, *a2, *y, *dy, *dz2, *dz1, *loss;
+  float *xs, *a1, *a2, *y, *dy, *dz2, *dz1, *loss, *lossp, *part;
+  int tb, splits;
 };
 
+bool fused(const polfed_mlp* n) { return n->d_in <= kFusedMax && n->H <= kFusedMax; }
+
 int ensure_work(polfed_mlp* n, int B, Work* w) {
-  const size_t need = (size_t)B * (n->d_in + 4 * n->H + 2 * n->d_out) + 64;
+  // 4 batch rows to a CTA, 8 for large batches (W2 is read once per CTA); shares of at least 64 rows
+  w->tb = B <= 1024 ? 4 : 8;
+  w->splits = std::max(1, std::min(16, (B + 63) / 64));
+  const size_t rows = (size_t)B * (n->d_in + 4 * n->H + 2 * n->d_out) + 64;
+  const size_t nl = fused(n) ? ((size_t)(B + w->tb - 1) / w->tb + 63) & ~(size_t)63 : 0;
+  const size_t need = rows + (fused(n) ? nl + (size_t)w->splits * n->n_params : 0);
   if (!n->work || n->work_floats < need) {
     if (n->work) cudaFree(n->work);
     n->work = nullptr;
@@ -207,6 +477,27 @@ int ensure_work(polfed_mlp* n, int B, Work* w) {
   w->dz2 = w->dy + (size_t)B * n->d_out;
   w->dz1 = w->dz2 + (size_t)B * n->H;
   w->loss = w->dz1 + (size_t)B * n->H;
+  w->lossp = n->work + rows;
+  w->part = w->lossp + nl;
+  return POLFED_OK;
+}
+
+// The fused row kernel: forward into y (t == nullptr), or forward and deltas.
+int run_rows(polfed_mlp* n, const float* x, const float* t, int B, float* y, const Work& w, cudaStream_t s) {
+  const Views v = views(n);
+  const RowArgs A{v.W1, v.b1, v.W2, v.b2, v.W3, v.b3, v.xm, v.xinv, v.ym, v.ysd, x, t, w.xs, w.a1, w.a2, w.dy,
+                  w.dz2, w.dz1, w.lossp, y, B, n->d_in, n->H, n->d_out};
+  const size_t smem = rows_smem(w.tb, n->d_in, n->H, n->d_out);
+  const int grid = (B + w.tb - 1) / w.tb;
+  if (w.tb == 4) {
+    if (smem > 48 * 1024) PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_mlp_rows<4><<<grid, kRowThreads, smem, s>>>(A);
+  } else {
+    if (smem > 48 * 1024) PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_mlp_rows<8><<<grid, kRowThreads, smem, s>>>(A);
+  }
+  PF_CUDA(cudaGetLastError());
+  count_launch();
   return POLFED_OK;
 }
 
@@ -223,12 +514,42 @@ int forward(polfed_mlp* n, const float* x, int B, cudaStream_t s, Work* w) {
   return POLFED_OK;
 }
 
-// gradient of 0.5/B sum |y - t'|^2 into n->grad; the loss partials go to dz1
-// before it is overwritten (d_out <= H)
-int backward(polfed_mlp* n, const float* x, const float* t, int B, cudaStream_t s, float* loss_host) {
+struct AdamStep {
+  float lr = 0.f, b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, c1 = 1.f, c2 = 1.f;  // lr == 0: gradient only
+};
+
+// gradient of 0.5/B sum |y - t'|^2 into n->grad (and d_grad), with the Adam
+// update of the parameters if ad.lr > 0; wide networks: the loss partials go to
+// dz1 before it is overwritten (d_out <= H)
+int backward(polfed_mlp* n, const float* x, const float* t, int B, cudaStream_t s, float* d_grad, const AdamStep& ad,
+             float* loss_host) {
   Work w;
-  PF_CHECK(forward(n, x, B, s, &w));
   const Views v = views(n);
+  if (fused(n)) {
+    PF_CHECK(ensure_work(n, B, &w));
+    PF_CHECK(run_rows(n, x, t, B, nullptr, w, s));
+    WArgs A{};
+    const int H = n->H;
+    auto tiles = [](int r, int c) { return ((r + 31) / 32) * ((c + 31) / 32); };
+    A.m[0] = WMat{w.dz2, w.a1, H, H, (int)(v.W2 - n->params), (int)(v.b2 - n->params), 0};
+    A.m[1] = WMat{w.dz1, w.xs, n->d_in, H, (int)(v.W1 - n->params), (int)(v.b1 - n->params), tiles(H, H)};
+    A.m[2] = WMat{w.dy, w.a2, H, n->d_out, (int)(v.W3 - n->params), (int)(v.b3 - n->params),
+                  A.m[1].tile0 + tiles(H, n->d_in)};
+    A.B = B;
+    A.rows = ((B + w.splits - 1) / w.splits + 31) & ~31;
+    A.n_params = n->n_params;
+    A.part = w.part;
+    const int splits = (B + A.rows - 1) / A.rows;
+    k_mlp_wgrad_tiles<<<dim3(A.m[2].tile0 + tiles(n->d_out, H), splits), 256, 0, s>>>(A);
+    k_mlp_combine<<<nblk(n->n_params) + 1, 256, 0, s>>>(w.part, splits, n->n_params, n->grad, d_grad, w.lossp,
+                                                         (B + w.tb - 1) / w.tb, w.loss, n->params, n->m, n->v, ad.lr,
+                                                         ad.b1, ad.b2, ad.eps, ad.c1, ad.c2);
+    PF_CUDA(cudaGetLastError());
+    count_launch(2);
+    if (loss_host) PF_CUDA(cudaMemcpyAsync(loss_host, w.loss, sizeof(float), cudaMemcpyDeviceToHost, s));
+    return POLFED_OK;
+  }
+  PF_CHECK(forward(n, x, B, s, &w));
   k_mlp_out_delta<<<nblk(B * n->d_out), 256, 0, s>>>(w.y, t, v.ym, v.ysd, B, n->d_out, w.dy, w.dz1);
   k_mlp_sum<<<1, 256, 0, s>>>(w.dz1, B * n->d_out, w.loss);
   k_mlp_wgrad<<<nblk(n->d_out * n->H + n->d_out), 256, 0, s>>>(w.dy, w.a2, B, n->H, n->d_out, v.gW3, v.gb3);
@@ -238,6 +559,14 @@ int backward(polfed_mlp* n, const float* x, const float* t, int B, cudaStream_t 
   k_mlp_wgrad<<<nblk(n->H * n->d_in + n->H), 256, 0, s>>>(w.dz1, w.xs, B, n->d_in, n->H, v.gW1, v.gb1);
   PF_CUDA(cudaGetLastError());
   count_launch(7);
+  if (ad.lr > 0.f) {
+    k_mlp_adam<<<nblk(n->n_params), 256, 0, s>>>(n->params, n->m, n->v, n->grad, n->n_params, ad.lr, ad.b1, ad.b2,
+                                                  ad.eps, ad.c1, ad.c2);
+    PF_CUDA(cudaGetLastError());
+    count_launch();
+  }
+  if (d_grad)
+    PF_CUDA(cudaMemcpyAsync(d_grad, n->grad, (size_t)n->n_params * sizeof(float), cudaMemcpyDeviceToDevice, s));
   if (loss_host) PF_CUDA(cudaMemcpyAsync(loss_host, w.loss, sizeof(float), cudaMemcpyDeviceToHost, s));
   return POLFED_OK;
 }
@@ -360,6 +689,12 @@ int polfed_mlp_forward(polfed_mlp* n, const float* d_x, int32_t B, float* d_y, p
   DeviceGuard g(n->device);
   cudaStream_t s = (cudaStream_t)stream;
   Work w;
+  if (fused(n)) {
+    PF_CHECK(ensure_work(n, B, &w));
+    PF_CHECK(run_rows(n, d_x, nullptr, B, d_y, w, s));
+    PF_CUDA(cudaStreamSynchronize(s));
+    return POLFED_OK;
+  }
   PF_CHECK(forward(n, d_x, B, s, &w));
   const Views v = views(n);
   k_mlp_unscale<<<nblk(B * n->d_out), 256, 0, s>>>(w.y, v.ym, v.ysd, B, n->d_out, d_y);
@@ -374,9 +709,7 @@ int polfed_mlp_grad(polfed_mlp* n, const float* d_x, const float* d_t, int32_t B
   if (!n || !d_x || !d_t || B < 1 || B > (1 << 20)) return fail(POLFED_EINVAL, "bad MLP gradient arguments");
   DeviceGuard g(n->device);
   cudaStream_t s = (cudaStream_t)stream;
-  PF_CHECK(backward(n, d_x, d_t, B, s, loss));
-  if (d_grad)
-    PF_CUDA(cudaMemcpyAsync(d_grad, n->grad, (size_t)n->n_params * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  PF_CHECK(backward(n, d_x, d_t, B, s, d_grad, AdamStep(), loss));
   PF_CUDA(cudaStreamSynchronize(s));
   return POLFED_OK;
 }
@@ -387,14 +720,16 @@ int polfed_mlp_train_step(polfed_mlp* n, const float* d_x, const float* d_t, int
     return fail(POLFED_EINVAL, "bad MLP training arguments");
   DeviceGuard g(n->device);
   cudaStream_t s = (cudaStream_t)stream;
-  PF_CHECK(backward(n, d_x, d_t, B, s, loss));
   n->t++;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.f - std::pow(b1, (float)n->t), c2 = 1.f - std::pow(b2, (float)n->t);
-  k_mlp_adam<<<nblk(n->n_params), 256, 0, s>>>(n->params, n->m, n->v, n->grad, n->n_params, lr, b1, b2, 1e-8f, c1,
-                                                c2);
-  PF_CUDA(cudaGetLastError());
-  count_launch();
+  AdamStep ad;
+  ad.lr = lr;
+  ad.c1 = 1.f - std::pow(ad.b1, (float)n->t);
+  ad.c2 = 1.f - std::pow(ad.b2, (float)n->t);
+  const int rc = backward(n, d_x, d_t, B, s, nullptr, ad, loss);
+  if (rc != POLFED_OK) {
+    n->t--;
+    return rc;
+  }
   PF_CUDA(cudaStreamSynchronize(s));
   return POLFED_OK;
 }
