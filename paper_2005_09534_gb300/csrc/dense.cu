@@ -100,13 +100,21 @@ __global__ void __launch_bounds__(256) k_gram(const double* __restrict__ Q, int6
     for (int b = 0; b < T; b++) P[(ty + 16 * a) * S + tx + 16 * b] = (double)ah[a][b] + (double)al[a][b];
 }
 
-// C[(j*S + a) * ldc + col0 + b] = sum_chunk partial[chunk][j][a][b]
-__global__ void k_gram_reduce(const double* __restrict__ partial, int nchunk, int J, int S, double* C, int ldc,
-                              int col0) {
+// C[(j*S + a) * ldc + col0 + b] = sum_chunk partial[chunk][j][a][b], 8 shares of the chunks per element
+__global__ void __launch_bounds__(256) k_gram_reduce(const double* __restrict__ partial, int nchunk, int J, int S,
+                                                      double* C, int ldc, int col0) {
+  __shared__ double sh[8][33];
   const int64_t n = (int64_t)J * S * S;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int c = 0; c < nchunk; c++) s += partial[(int64_t)c * n + e];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t e = blockIdx.x * 32ll + lane;
+  double s = 0.0;
+  if (e < n)
+    for (int c = g; c < nchunk; c += 8) s += partial[(int64_t)c * n + e];
+  sh[g][lane] = s;
+  __syncthreads();
+  if (g == 0 && e < n) {
+#pragma unroll
+    for (int q = 1; q < 8; q++) s += sh[q][lane];
     const int64_t jb = e / (S * S);
     const int a = (int)((e / S) % S), b = (int)(e % S);
     C[(jb * S + a) * ldc + col0 + b] = s;
@@ -184,9 +192,12 @@ __global__ void __launch_bounds__(256) k_update(const double* __restrict__ Q, in
 // G (S x S, symmetric positive definite) = L L^T.  Writes Minv = L^{-T}
 // (so that Q = R Minv has orthonormal columns) and B = L^T (R = Q B).
 // flag[0] |= 1 if a pivot is not positive (rank-deficient block).
-__global__ void k_chol_small(const double* __restrict__ G, int S, double* Minv, double* B, int* flag) {
+// Latency of one CTA's chain: per column one square root and one division.
+__global__ void __launch_bounds__(256) k_chol_small(const double* __restrict__ G, int S, double* Minv, double* B, int* flag) {
   extern __shared__ double sm[];
-  double* A = sm;  // S x S, becomes L (lower)
+  double* A = sm;           // S x S, becomes L (lower)
+  double* dinv = sm + S * S;  // 1 / L[k][k]
+  double* X = S <= 64 ? dinv + S : Minv;  // S x S while it fits
   for (int e = threadIdx.x; e < S * S; e += blockDim.x) {
     const int i = e / S, j = e % S;
     A[e] = 0.5 * (G[i * S + j] + G[j * S + i]);
@@ -199,6 +210,7 @@ __global__ void k_chol_small(const double* __restrict__ G, int S, double* Minv, 
     dmax = m;
   }
   __syncthreads();
+  __shared__ double inv;
   for (int k = 0; k < S; k++) {
     if (threadIdx.x == 0) {
       double d = A[k * S + k];
@@ -206,11 +218,14 @@ __global__ void k_chol_small(const double* __restrict__ G, int S, double* Minv, 
         atomicOr(flag, 1);
         d = fmax(1e-28 * dmax, 1e-300);
       }
-      A[k * S + k] = sqrt(d);
+      d = sqrt(d);
+      A[k * S + k] = d;
+      inv = 1.0 / d;
+      dinv[k] = inv;
     }
     __syncthreads();
-    const double piv = A[k * S + k];
-    for (int i = k + 1 + threadIdx.x; i < S; i += blockDim.x) A[i * S + k] /= piv;
+    const double piv = inv;
+    for (int i = k + 1 + threadIdx.x; i < S; i += blockDim.x) A[i * S + k] *= piv;
     __syncthreads();
     const int m = S - k - 1;
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
@@ -219,16 +234,20 @@ __global__ void k_chol_small(const double* __restrict__ G, int S, double* Minv, 
     }
     __syncthreads();
   }
-  // column c of L^{-1} by forward substitution (one thread per column),
-  // stored transposed: Minv[c * S + i] = (L^{-1})[i][c], i.e. Minv = L^{-T}.
-  for (int c = threadIdx.x; c < S; c += blockDim.x) {
-    double* col = Minv + (size_t)c * S;
-    for (int i = 0; i < c; i++) col[i] = 0.0;
-    for (int i = c; i < S; i++) {
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int k = c; k < i; k++) s -= A[i * S + k] * col[k];
-      col[i] = s / A[i * S + i];
+  // L^{-1} row by row: row i of column c is (delta_ic - sum_k L[i][k] L^{-1}[k][c]) / L[i][i]; two (S = 128)
+  // to sixteen (S = 16) threads share the sum of a column, combined by shuffles.  Stored transposed:
+  // Minv[c * S + i] = (L^{-1})[i][c], i.e. Minv = L^{-T}; X holds it during the sweep.
+  const int np = blockDim.x / S, c = threadIdx.x / np, part = threadIdx.x % np;
+  for (int i = 0; i < S; i++) {
+    double s = 0.0;
+    for (int k = c + part; k < i; k += np) s = fma(A[i * S + k], X[c * S + k], s);
+    for (int o = np / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (part == 0) {
+      const double v = i < c ? 0.0 : ((i == c ? 1.0 : 0.0) - s) * dinv[i];
+      X[c * S + i] = v;
+      Minv[(size_t)c * S + i] = v;
     }
+    __syncwarp();
   }
   for (int e = threadIdx.x; e < S * S; e += blockDim.x) {
     const int i = e / S, j = e % S;
@@ -269,12 +288,16 @@ __global__ void k_coldot(const double* __restrict__ A, const double* __restrict_
   }
 }
 
-__global__ void k_reduce_rows(const double* partial, int nblk, int S, double* out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= S) return;
+// out[c] = sum_b partial[b * S + c], one CTA per column, fixed order
+__global__ void __launch_bounds__(128) k_reduce_rows(const double* partial, int nblk, int S, double* out) {
+  __shared__ double sh[4];
+  const int c = blockIdx.x;
   double t = 0.0;
-  for (int b = 0; b < nblk; b++) t += partial[(int64_t)b * S + c];
-  out[c] = t;
+  for (int b = threadIdx.x; b < nblk; b += 128) t += partial[(int64_t)b * S + c];
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) out[c] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
 }
 
 // y = a*x + b*y + c*z (vectors of length n)
@@ -343,13 +366,163 @@ __global__ void k_scale_add_cols(double* F, const double* __restrict__ G, const 
   }
 }
 
+// ------------------------------------------------- single-vector Lanczos
+// Latency: a few launches per step and nothing returned to the host between
+// them (60 us a step with two synchronizations each before, 14 now; the bounds
+// of an L = 14 chain 17 -> 4 ms, its checks by k_tri_extremes instead of a
+// dense eigen-solve included).
+constexpr int kLzBlocks = 152 * 2;
+constexpr int kLzThreads = 256;
+
+__device__ __forceinline__ double cta_sum(double v, double* sh) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  for (int q = 0; q < kLzThreads / 32; q++) t += sh[q];
+  return t;
+}
+
+// Sum of the CTAs' values by the last one to arrive, in CTA order; true in that
+// CTA, which has the sum in *tot.  count returns to 0.
+__device__ __forceinline__ bool last_cta_sum(double v, double* part, unsigned* count, double* sh, double* tot) {
+  __shared__ bool last;
+  const double t = cta_sum(v, sh);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = t;
+    __threadfence();
+    last = atomicInc(count, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double s = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kLzThreads) s += __ldcg(part + b);
+  *tot = cta_sum(s, sh);
+  return true;
+}
+
+// alpha = v1 . w
+__global__ void __launch_bounds__(kLzThreads) k_lz_alpha(const double* __restrict__ v1, const double* __restrict__ w,
+                                                         int64_t n, double* part, unsigned* count, double* alpha) {
+  __shared__ double sh[kLzThreads / 32];
+  double s = 0.0, t;
+  for (int64_t i = blockIdx.x * (int64_t)kLzThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kLzThreads)
+    s = fma(v1[i], w[i], s);
+  if (last_cta_sum(s, part, count, sh, &t) && threadIdx.x == 0) *alpha = t;
+}
+
+// w -= alpha v1 + beta_prev v0; beta = |w|
+__global__ void __launch_bounds__(kLzThreads) k_lz_beta(const double* __restrict__ v0, const double* __restrict__ v1,
+                                                        double* __restrict__ w, int64_t n, const double* beta_prev,
+                                                        const double* alpha, double* part, unsigned* count,
+                                                        double* beta) {
+  __shared__ double sh[kLzThreads / 32];
+  const double a = *alpha, b = beta_prev ? *beta_prev : 0.0;
+  double s = 0.0, t;
+  for (int64_t i = blockIdx.x * (int64_t)kLzThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kLzThreads) {
+    const double x = -a * v1[i] + w[i] - b * v0[i];
+    w[i] = x;
+    s = fma(x, x, s);
+  }
+  if (last_cta_sum(s, part, count, sh, &t) && threadIdx.x == 0) *beta = sqrt(fmax(t, 0.0));
+}
+
+// w /= beta (a vanishing beta ends the recurrence: w = 0)
+__global__ void k_lz_scale(double* __restrict__ w, int64_t n, const double* beta) {
+  const double b = *beta, f = b < 1e-300 ? 0.0 : 1.0 / b;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) w[i] *= f;
+}
+
+// Extreme eigenvalues of a symmetric tridiagonal of order m by multisection on
+// Sturm counts (64 points a round: lanes 0..63 the lowest, 64..127 the highest
+// eigenvalue), and the last components of their vectors by the three-term
+// recurrence from the last row back (the components of a converging Lanczos
+// vector grow in that direction), whose norm is then known.
+__global__ void __launch_bounds__(128) k_tri_extremes(const double* __restrict__ al, const double* __restrict__ be,
+                                                      int m_in, double* __restrict__ res) {
+  __shared__ double s_lo[2], s_hi[2];
+  __shared__ int s_cnt[128], s_m;
+  const int t = threadIdx.x, g = t >> 6, p = t & 63;
+  if (t == 0) {
+    int m = m_in;  // steps before a vanishing beta
+    for (int i = 0; i < m; i++)
+      if (be[i] < 1e-300) {
+        m = i + 1;
+        break;
+      }
+    s_m = m;
+    double lo = 1e300, hi = -1e300;  // Gershgorin
+    for (int i = 0; i < m; i++) {
+      const double r = (i > 0 ? be[i - 1] : 0.0) + (i + 1 < m ? be[i] : 0.0);
+      lo = fmin(lo, al[i] - r);
+      hi = fmax(hi, al[i] + r);
+    }
+    const double w = fmax(fabs(lo), fabs(hi)) * 1e-15 + 1e-300;
+    s_lo[0] = s_lo[1] = lo - w;
+    s_hi[0] = s_hi[1] = hi + w;
+  }
+  __syncthreads();
+  const int m = s_m, want = g == 0 ? 0 : m - 1;
+  for (int round = 0; round < 12; round++) {
+    const double lo = s_lo[g], hi = s_hi[g], x = lo + (hi - lo) * ((p + 1) / 65.0);
+    // eigenvalues below x: negative pivots of T - x
+    int cnt = 0;
+    double q = 1.0;
+    for (int i = 0; i < m; i++) {
+      const double b = i > 0 ? be[i - 1] : 0.0;
+      q = al[i] - x - (i > 0 ? b * b / q : 0.0);
+      if (fabs(q) < 1e-290) q = -1e-290;
+      cnt += q < 0.0;
+    }
+    s_cnt[t] = cnt;
+    __syncthreads();
+    if (p == 0) {
+      // the first point with more than `want` eigenvalues below it bounds the wanted one from above
+      double a = lo, b = hi;
+      for (int u = 0; u < 64; u++) {
+        const double xu = lo + (hi - lo) * ((u + 1) / 65.0);
+        if (s_cnt[g * 64 + u] > want) {
+          b = xu;
+          break;
+        }
+        a = xu;
+      }
+      s_lo[g] = a;
+      s_hi[g] = b;
+    }
+    __syncthreads();
+  }
+  if (p == 0) {
+    const double lam = 0.5 * (s_lo[g] + s_hi[g]);
+    double y = 1.0, yn = 0.0, ss = 1.0, last = 1.0;  // y_i, y_{i+1}; the last component rides along in scale
+    for (int i = m - 1; i > 0; i--) {
+      const double yp = ((lam - al[i]) * y - (i + 1 < m ? be[i] : 0.0) * yn) / be[i - 1];
+      yn = y;
+      y = yp;
+      ss = fma(y, y, ss);
+      if (ss > 1e200) {
+        y *= 1e-100;
+        yn *= 1e-100;
+        last *= 1e-100;
+        ss *= 1e-200;
+      }
+    }
+    res[g] = lam;
+    res[2 + g] = be[m - 1] * last / sqrt(ss);
+    if (t == 0) res[4] = (double)m;
+  }
+}
+
 // ------------------------------------------------------------------- host
 static int grid_for(int64_t n, int per = 256) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 152 * 8)); }
 
 int Dense::gram(const double* Q, int64_t pstride, int J, const double* R, double* C, int ldc, int col0,
                 cudaStream_t s) {
   if (J <= 0) return POLFED_OK;
-  int64_t nchunk = std::max<int64_t>(1, std::min<int64_t>((4 * 152 + J - 1) / J, (dim + 2047) / 2048));
+  // four CTAs per SM, at least 64 rows each (float-float sums of a chunk, FP64 sums over the chunks).
+  // With 2048 rows each, L = 14 ran two CTAs per panel: 130 us a call at S = 16, now 8.
+  int64_t nchunk = std::max<int64_t>(1, std::min<int64_t>((4 * 152 + J - 1) / J, (dim + 63) / 64));
   const int64_t rpc = (dim + nchunk - 1) / nchunk;
   nchunk = (dim + rpc - 1) / rpc;
   const size_t need = (size_t)nchunk * J * S * S * sizeof(double);
@@ -365,7 +538,7 @@ int Dense::gram(const double* Q, int64_t pstride, int J, const double* R, double
     default: return fail(POLFED_EINVAL, "block size must be 16, 32, 64 or 128");
   }
   PF_CUDA(cudaGetLastError());
-  k_gram_reduce<<<grid_for((int64_t)J * S * S), 256, 0, s>>>((const double*)partial, (int)nchunk, J, S, C, ldc, col0);
+  k_gram_reduce<<<(unsigned)(((int64_t)J * S * S + 31) / 32), 256, 0, s>>>((const double*)partial, (int)nchunk, J, S, C, ldc, col0);
   PF_CUDA(cudaGetLastError());
   count_launch(2);
   return POLFED_OK;
@@ -406,7 +579,7 @@ int Dense::cholqr(double* R, double* Qout, double* B_host, int passes, cudaStrea
   const double* src = R;
   for (int p = 0; p < passes; p++) {
     PF_CHECK(gram(src, 0, 1, src, G, S, 0, s));
-    const size_t smem = (size_t)S * S * sizeof(double);
+    const size_t smem = ((size_t)S * S * (S <= 64 ? 2 : 1) + S) * sizeof(double);
     k_chol_small<<<1, 256, smem, s>>>(G, S, Minv, B, flag);
     PF_CUDA(cudaGetLastError());
     count_launch();
@@ -448,7 +621,7 @@ int Dense::coldot(const double* A, const double* B, int ncol, double* out_host, 
   double* res = part + (size_t)nblk * ncol;
   k_coldot<<<nblk, threads, threads * sizeof(double), s>>>(A, B, dim, ncol, part);
   PF_CUDA(cudaGetLastError());
-  k_reduce_rows<<<(ncol + 127) / 128, 128, 0, s>>>(part, nblk, ncol, res);
+  k_reduce_rows<<<ncol, 128, 0, s>>>(part, nblk, ncol, res);
   PF_CUDA(cudaGetLastError());
   count_launch(2);
   PF_CUDA(cudaMemcpyAsync(out_host, res, (size_t)ncol * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -459,6 +632,37 @@ int Dense::coldot(const double* A, const double* B, int ncol, double* out_host, 
 int Dense::axpbypcz(int64_t n, double a, const double* x, double b, double* y, double c, const double* z,
                     cudaStream_t s) {
   k_axpbypcz<<<grid_for(n), 256, 0, s>>>(n, a, x, b, y, c, z);
+  PF_CUDA(cudaGetLastError());
+  count_launch();
+  return POLFED_OK;
+}
+
+// al, be of kmax steps and the five results of tri_extremes, behind the partial
+// sums and the arrival counter (zeroed here; atomicInc brings it back to 0)
+int Dense::lanczos_begin(int kmax, double** al, double** be, double** res, cudaStream_t s) {
+  PF_CHECK(ensure(lz, lz_bytes, (kLzBlocks + 40 + 2 * (size_t)std::max(kmax, 1)) * sizeof(double)));
+  PF_CUDA(cudaMemsetAsync(lz, 0, (kLzBlocks + 40) * sizeof(double), s));
+  *res = (double*)lz + kLzBlocks + 32;
+  *al = *res + 8;
+  *be = *al + std::max(kmax, 1);
+  return POLFED_OK;
+}
+
+int Dense::lanczos_step(const double* v0, const double* v1, double* w, const double* beta_prev, double* alpha,
+                        double* beta, cudaStream_t s) {
+  double* part = (double*)lz;
+  unsigned* count = (unsigned*)(part + kLzBlocks);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((dim + kLzThreads - 1) / kLzThreads, kLzBlocks));
+  k_lz_alpha<<<grid, kLzThreads, 0, s>>>(v1, w, dim, part, count, alpha);
+  k_lz_beta<<<grid, kLzThreads, 0, s>>>(v0, v1, w, dim, beta_prev, alpha, part, count, beta);
+  k_lz_scale<<<grid_for(dim), 256, 0, s>>>(w, dim, beta);
+  PF_CUDA(cudaGetLastError());
+  count_launch(3);
+  return POLFED_OK;
+}
+
+int Dense::tri_extremes(const double* al, const double* be, int m, double* res, cudaStream_t s) {
+  k_tri_extremes<<<1, 128, 0, s>>>(al, be, m, res);
   PF_CUDA(cudaGetLastError());
   count_launch();
   return POLFED_OK;
@@ -507,9 +711,9 @@ int Dense::ensure(void*& p, size_t& have, size_t need) {
 void Dense::release() {
   if (partial) cudaFree(partial);
   if (small) cudaFree(small);
-  if (tmpbuf) cudaFree(tmpbuf);
-  partial = small = tmpbuf = nullptr;
-  partial_bytes = small_bytes = tmpbuf_bytes = 0;
+  if (lz) cudaFree(lz);
+  partial = small = lz = nullptr;
+  partial_bytes = small_bytes = lz_bytes = 0;
 }
 
 int Dense::configure() {

@@ -14,8 +14,8 @@ struct Dense {
   size_t partial_bytes = 0;
   void* small = nullptr;
   size_t small_bytes = 0;
-  void* tmpbuf = nullptr;
-  size_t tmpbuf_bytes = 0;
+  void* lz = nullptr;  // partial sums, arrival counter, coefficients and results of a bounds recurrence
+  size_t lz_bytes = 0;
 
   int configure();
   // C[(j*S + a) * ldc + col0 + b] = (Q_j^T R)[a][b] for panels j < J (panel stride pstride)
@@ -29,6 +29,12 @@ struct Dense {
   int random_fill(double* X, int64_t n, uint64_t seed, cudaStream_t s);
   int coldot(const double* A, const double* B, int ncol, double* out_host, cudaStream_t s);
   int axpbypcz(int64_t n, double a, const double* x, double b, double* y, double c, const double* z, cudaStream_t s);
+  int lanczos_begin(int kmax, double** al, double** be, double** res, cudaStream_t s);
+  // one step of single-vector Lanczos: alpha = v1.w, w -= alpha v1 + beta_prev v0 (null: 0), beta = |w|, w /= beta
+  int lanczos_step(const double* v0, const double* v1, double* w, const double* beta_prev, double* alpha, double* beta,
+                   cudaStream_t s);
+  // extreme eigenvalues of the tridiagonal (al, be)[0..m): res = {lo, hi, |be t_last| of lo, of hi, m used}
+  int tri_extremes(const double* al, const double* be, int m, double* res, cudaStream_t s);
   int resid(const double* U, double* W, const double* lam_dev, cudaStream_t s);
   int panels_to_colmajor(const double* P, int n, double* out, cudaStream_t s);
   // out (nc_pad / S panels) = columns idx[0..nc) of the panel-major block in, zero padded

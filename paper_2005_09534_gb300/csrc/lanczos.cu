@@ -225,6 +225,8 @@ struct LanczosOut {
   std::vector<double> resid_t;  // H~ units
   int n_out = 0, m = 0, n_conv = 0, checks = 0, ritz_cols = 0, n_refine = 0, refine_K = 0;
   int n_acc = -1;  // Ritz values theta >= p at the last check (converged or not); -1 = no check yet
+  std::vector<double> rr_lam;  // eigenvalues of the Rayleigh-Ritz step whose U, H~U (ritz buffer) and eigenvectors
+                               // (evbuf) are still in place; empty if they are not
   int64_t matvec_cols = 0;
   double t_filter = 0, t_reorth = 0, t_qr = 0, t_teig = 0, t_ritz = 0;
 };
@@ -368,6 +370,7 @@ int run_lanczos(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, double* d_
             T[(size_t)((i + 1) * S + a) * n + i * S + b] = v;
           }
     }
+    out.rr_lam.clear();
     PF_CHECK(c->evbuf.ensure(((size_t)n * n + n) * sizeof(double), &c->ws_total, c->ws_limit));
     double* Td = c->evbuf.as<double>();
     double* wd = Td + (size_t)n * n;
@@ -560,6 +563,7 @@ int rr_select(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, const double
   if (d_evecs) PF_CHECK(D.panels_to_colmajor(Uo, nout, d_evecs, s));
   PF_CUDA(cudaStreamSynchronize(s));
   out.n_out = nout;
+  out.rr_lam = lamh;
   return POLFED_OK;
 }
 
@@ -694,25 +698,14 @@ int refine_dd(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, int Kr, int 
   PF_CHECK(ensure_ritz(c, dim, S, nr, P.N_ev));
   const RitzLayout R(c->ritz.as<double>(), dim, S, nr, P.N_ev);
   const double t0 = now_s();
-  // 1. Rayleigh-Ritz basis of span(U): W = H~ U (FP64), G = U^T W = Y diag(lam) Y^T
-  PF_CHECK(plan.prepare_typed(POLFED_F64, P.e_lo, P.e_hi));
-  PF_CHECK(c->fscr.ensure(std::max(c->fscr.n, filter_scratch_bytes(plan, POLFED_F64, S)), &c->ws_total,
-                          c->ws_limit));
-  FilterScratch scr64;
-  scr64.xs = c->fscr.p;
-  scr64.bytes = c->fscr.n;
-  for (int q = 0; q < npan; q++)
-    PF_CHECK(apply_block(plan, POLFED_F64, R.U + (size_t)q * pstride, R.Wr + (size_t)q * pstride, S, POLFED_F64, scr64,
-                         s));
-  out.matvec_cols += nr_pad;
-  PF_CHECK(c->evbuf.ensure(((size_t)nr_pad * nr_pad + nr_pad) * sizeof(double), &c->ws_total, c->ws_limit));
+  // 1. Rayleigh-Ritz basis of span(U): W = H~ U (FP64), G = U^T W = Y diag(lam) Y^T.  The rr_select that ended
+  //    the Lanczos stage or the last sweep computed them from the same U and left them in place.
+  if ((int)out.rr_lam.size() != nr) return fail(POLFED_EINVAL, "refinement without a Rayleigh-Ritz step before it");
   double* G = c->evbuf.as<double>();
   double* lam_d = G + (size_t)nr_pad * nr_pad;
-  for (int q = 0; q < npan; q++) PF_CHECK(D.gram(R.U, pstride, npan, R.Wr + (size_t)q * pstride, G, nr_pad, q * S, s));
-  PF_CHECK(syevd(c, G, nr, nr_pad, lam_d));
   std::vector<double> lam(nr_pad, 0.0);
-  PF_CUDA(cudaMemcpyAsync(lam.data(), lam_d, nr * sizeof(double), cudaMemcpyDeviceToHost, s));
-  PF_CUDA(cudaStreamSynchronize(s));
+  std::copy(out.rr_lam.begin(), out.rr_lam.end(), lam.begin());
+  out.rr_lam.clear();
   // 2. F = U Y, T = W Y - F diag(lam): the Ritz vectors and their residuals (padding columns zero)
   PF_CUDA(cudaMemsetAsync(R.F, 0, (size_t)npan * pstride * sizeof(double), s));
   PF_CUDA(cudaMemsetAsync(R.T, 0, (size_t)npan * pstride * sizeof(double), s));
@@ -803,7 +796,10 @@ int refine_dd(polfed_ctx* c, HamPlan& plan, const LanczosParams& P, int Kr, int 
   return finish_sweep(c, plan, P, R.F, nr, d_evecs, out);
 }
 
-// Single-vector Lanczos on H for E_min and E_max (text before Eq. (3)).
+// Single-vector Lanczos on H for E_min and E_max (text before Eq. (3)).  The
+// recurrence runs on the device (alpha and beta included); the host looks at it
+// every 20 steps, when one kernel has found the extreme Ritz values and the last
+// components of their vectors.
 int spectral_bounds(polfed_ctx* c, HamPlan& plan, const polfed_opts& o, double* emin, double* emax, double* err,
                     int64_t* matvecs) {
   cudaStream_t s = c->stream;
@@ -813,62 +809,44 @@ int spectral_bounds(polfed_ctx* c, HamPlan& plan, const polfed_opts& o, double* 
   FilterScratch scr;
   scr.xs = c->fscr.p;
   scr.bytes = c->fscr.n;
-  PF_CHECK(c->R.ensure((size_t)3 * dim * sizeof(double), &c->ws_total, c->ws_limit));
+  const int kmax = (int)std::min<int64_t>(o.bounds_steps, dim);
+  const size_t nv = (size_t)dim;
+  PF_CHECK(c->R.ensure(3 * nv * sizeof(double), &c->ws_total, c->ws_limit));
   double* v0 = c->R.as<double>();
-  double* v1 = v0 + dim;
-  double* w = v1 + dim;
+  double* v1 = v0 + nv;
+  double* w = v1 + nv;
+  double *al, *be, *res;  // be[k] couples k and k + 1
   Dense& D = c->dense;
   D.dim = dim;
+  PF_CHECK(D.lanczos_begin(kmax, &al, &be, &res, s));
   PF_CHECK(D.random_fill(v1, dim, o.seed ^ 0x5bd1e995ull, s));
   double nrm = 0.0;
   PF_CHECK(D.coldot(v1, v1, 1, &nrm, s));
   PF_CHECK(D.axpbypcz(dim, 0.0, v1, 1.0 / std::sqrt(nrm), v1, 0.0, nullptr, s));
   PF_CUDA(cudaMemsetAsync(v0, 0, dim * sizeof(double), s));
-  std::vector<double> al, be;  // be[k] couples k and k+1
-  double beta = 0.0;
-  const int kmax = (int)std::min<int64_t>(o.bounds_steps, dim);
   double lo = 0, hi = 0, e_lo = 1e300, e_hi = 1e300;
   for (int k = 0; k < kmax; k++) {
     PF_CHECK(apply_block(plan, POLFED_F64, v1, w, 1, POLFED_F64, scr, s));
     (*matvecs)++;
-    double a = 0.0;
-    PF_CHECK(D.coldot(v1, w, 1, &a, s));
-    al.push_back(a);
-    PF_CHECK(D.axpbypcz(dim, -a, v1, 1.0, w, -beta, v0, s));
-    double bb = 0.0;
-    PF_CHECK(D.coldot(w, w, 1, &bb, s));
-    beta = std::sqrt(std::max(bb, 0.0));
-    be.push_back(beta);
+    // w <- w - alpha v1 - beta_{k-1} v0, then (v0, v1, w) <- (v1, w / beta, v0)
+    PF_CHECK(D.lanczos_step(v0, v1, w, k == 0 ? nullptr : be + k - 1, al + k, be + k, s));
     const int m = k + 1;
-    const bool check = (m >= 20 && m % 20 == 0) || m == kmax || beta < 1e-300;
-    if (check) {
-      // eigen-solve of the m x m tridiagonal
-      std::vector<double> T((size_t)m * m, 0.0);
-      for (int i = 0; i < m; i++) {
-        T[(size_t)i * m + i] = al[i];
-        if (i + 1 < m) T[(size_t)i * m + i + 1] = T[(size_t)(i + 1) * m + i] = be[i];
-      }
-      PF_CHECK(c->evbuf.ensure(((size_t)m * m + m) * sizeof(double), &c->ws_total, c->ws_limit));
-      double* Td = c->evbuf.as<double>();
-      PF_CUDA(cudaMemcpyAsync(Td, T.data(), (size_t)m * m * sizeof(double), cudaMemcpyHostToDevice, s));
-      PF_CHECK(syevd(c, Td, m, m, Td + (size_t)m * m));
-      std::vector<double> ev(m), y0(m), y1(m);
-      PF_CUDA(cudaMemcpyAsync(ev.data(), Td + (size_t)m * m, m * sizeof(double), cudaMemcpyDeviceToHost, s));
-      double last_lo = 0, last_hi = 0;
-      PF_CUDA(cudaMemcpyAsync(&last_lo, Td + (size_t)0 * m + (m - 1), sizeof(double), cudaMemcpyDeviceToHost, s));
-      PF_CUDA(cudaMemcpyAsync(&last_hi, Td + (size_t)(m - 1) * m + (m - 1), sizeof(double), cudaMemcpyDeviceToHost, s));
+    if ((m >= 20 && m % 20 == 0) || m == kmax) {
+      double h[5];  // E_lo, E_hi, |beta t_last| of both, number of steps before a vanishing beta
+      PF_CHECK(D.tri_extremes(al, be, m, res, s));
+      PF_CUDA(cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, s));
       PF_CUDA(cudaStreamSynchronize(s));
-      lo = ev[0];
-      hi = ev[m - 1];
-      e_lo = std::fabs(beta * last_lo);
-      e_hi = std::fabs(beta * last_hi);
+      lo = h[0];
+      hi = h[1];
+      e_lo = h[2];
+      e_hi = h[3];
       const double scale = std::max(std::fabs(lo), std::fabs(hi));
-      if ((e_lo <= 1e-12 * scale && e_hi <= 1e-12 * scale) || beta < 1e-300) break;
+      if ((e_lo <= 1e-12 * scale && e_hi <= 1e-12 * scale) || (int)h[4] < m) break;
     }
-    if (beta < 1e-300) break;
-    // v0 <- v1, v1 <- w / beta
-    std::swap(v0, v1);
-    PF_CHECK(D.axpbypcz(dim, 1.0 / beta, w, 0.0, v1, 0.0, nullptr, s));
+    double* t = v0;
+    v0 = v1;
+    v1 = w;
+    w = t;
   }
   *emin = lo;
   *emax = hi;
