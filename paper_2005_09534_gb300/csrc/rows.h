@@ -543,13 +543,18 @@ struct GroupStep {
 
 // Grid barrier of a cooperative launch: arrivals are counted on one monotone
 // counter; waits are bounded (cap polls), a wait that runs out sets *err and
-// every CTA leaves at its next barrier.
-__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int* err, uint32_t cap) {
+// every CTA leaves at its next barrier.  What needs no other CTA's result goes
+// between the two halves.
+__device__ __forceinline__ void grid_arrive(unsigned* count) {
   __syncthreads();
-  int ok = 1;
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(count, 1u);
+  }
+}
+__device__ __forceinline__ bool grid_wait(unsigned* count, unsigned target, int* err, uint32_t cap) {
+  int ok = 1;
+  if (threadIdx.x == 0) {
     uint32_t it = 0;
     while ((int)(*(volatile unsigned*)count - target) < 0) {
       if (++it > cap) {
@@ -606,51 +611,51 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
   const int me = team * gridDim.x + blockIdx.x;  // neighbouring items go to different SMs
   if (tt < LPR) *reinterpret_cast<int4*>(tile + tt * 16) = make_int4(0, 0, 0, 0);  // the zero row
   unsigned target = R.bar_base;
-  for (int st = R.st0; st < R.st1; st++) {
-    int j = 0, base = 0, r = 0;
-    // fetch the r-th item of this team into items[r & 1]; false if there is none
-    auto fetch = [&]() -> bool {
-      const int item = r * n_teams + ((r & 1) ? n_teams - 1 - me : me);
-      const StepJob* J = nullptr;
-      for (; j < R.n_jobs; j++) {
-        J = R.jobs ? R.jobs + j : &R.one;
-        const int ng = st < J->K ? J->n_groups : 0;
-        if (item < base + ng) break;
-        base += ng;
-      }
-      if (j >= R.n_jobs) return false;
-      Item* I = items + (r & 1);
-      const int gidx = item - base;
-      constexpr int NG = sizeof(GroupRec) / 16;
-      if (tt < NG) cp_async16(reinterpret_cast<char*>(&I->g) + tt * 16, reinterpret_cast<const char*>(J->grec + gidx) + tt * 16);
-      if (tt == NG)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(&I->fhi)),
-                     "l"(reinterpret_cast<const C*>(J->Fhi) + gidx), "n"(sizeof(C))
-                     : "memory");
-      cp_async_commit();
-      if (tt == 32) {
-        const size_t so = R.jobs ? 0 : (size_t)j * R.stride;
-        I->b1 = ((st & 1) ? J->bb : J->ba) + so;
-        I->out = ((st & 1) ? J->ba : J->bb) + so;
-        I->x = J->xs + so;
-        I->rec = reinterpret_cast<const char*>(J->rec);
-        I->fc = reinterpret_cast<const char*>(J->Fc);
-        I->cxt = reinterpret_cast<const char*>(J->Cx);
-        I->n_cross = J->n_cross;
-        I->c2mask = J->c2mask;
-        const int kk = J->K - 1 - st;
-        C cx = C();
-        if constexpr (COLS)
-          I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * (4 * LPR));
-        else
-          cx = R.jobs ? __ldg(reinterpret_cast<const C*>(J->cx) + st) : *reinterpret_cast<const C*>(&R.cx[st - R.st0]);
-        const typename NT::Coef k = NT::make(J->con, kk == 0, st == 0, cx);
-        I->k = k;
-        I->flags = (COLS || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
-      }
-      return true;
-    };
-    bool more = fetch();
+  int st = R.st0, j = 0, base = 0, r = 0;
+  // fetch the r-th item of this team into items[r & 1]; false if there is none
+  auto fetch = [&]() -> bool {
+    const int item = r * n_teams + ((r & 1) ? n_teams - 1 - me : me);
+    const StepJob* J = nullptr;
+    for (; j < R.n_jobs; j++) {
+      J = R.jobs ? R.jobs + j : &R.one;
+      const int ng = st < J->K ? J->n_groups : 0;
+      if (item < base + ng) break;
+      base += ng;
+    }
+    if (j >= R.n_jobs) return false;
+    Item* I = items + (r & 1);
+    const int gidx = item - base;
+    constexpr int NG = sizeof(GroupRec) / 16;
+    if (tt < NG) cp_async16(reinterpret_cast<char*>(&I->g) + tt * 16, reinterpret_cast<const char*>(J->grec + gidx) + tt * 16);
+    if (tt == NG)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(&I->fhi)),
+                   "l"(reinterpret_cast<const C*>(J->Fhi) + gidx), "n"(sizeof(C))
+                   : "memory");
+    cp_async_commit();
+    if (tt == 32) {
+      const size_t so = R.jobs ? 0 : (size_t)j * R.stride;
+      I->b1 = ((st & 1) ? J->bb : J->ba) + so;
+      I->out = ((st & 1) ? J->ba : J->bb) + so;
+      I->x = J->xs + so;
+      I->rec = reinterpret_cast<const char*>(J->rec);
+      I->fc = reinterpret_cast<const char*>(J->Fc);
+      I->cxt = reinterpret_cast<const char*>(J->Cx);
+      I->n_cross = J->n_cross;
+      I->c2mask = J->c2mask;
+      const int kk = J->K - 1 - st;
+      C cx = C();
+      if constexpr (COLS)
+        I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * (4 * LPR));
+      else
+        cx = R.jobs ? __ldg(reinterpret_cast<const C*>(J->cx) + st) : *reinterpret_cast<const C*>(&R.cx[st - R.st0]);
+      const typename NT::Coef k = NT::make(J->con, kk == 0, st == 0, cx);
+      I->k = k;
+      I->flags = (COLS || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
+    }
+    return true;
+  };
+  bool more = fetch();
+  for (;;) {
     while (more) {
       cp_async_wait();
       team_sync(team);  // the item is complete, the previous group's tile is no longer read
@@ -659,11 +664,14 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       more = fetch();
       GroupStep<NT, LPR, J2, COLS, RMAX>::run(I, tile, team, tt >> 5);
     }
-    if (st + 1 < R.st1) {
-      target += gridDim.x;
-      if (!grid_barrier(R.bar, target, R.err, R.cap)) return;
-    }
+    if (++st == R.st1) break;
+    grid_arrive(R.bar);
+    j = base = r = 0;
+    more = fetch();  // the first item of the next step, while the others arrive
+    target += gridDim.x;
+    if (!grid_wait(R.bar, target, R.err, R.cap)) break;
   }
+  cp_async_wait();
 }
 
 }  // namespace polfed
