@@ -712,79 +712,15 @@ static int check_operator(const HamPlan& p, int kind) {
   return POLFED_OK;
 }
 
-// Per-kernel, per-device launch configuration, filled once under its mutex.
-struct LaunchCache {
-  static constexpr int kDevices = 64;
-  std::mutex mu;
-  struct {
-    bool set = false;
-    int nsm = 0, maxdyn = 0;
-  } d[kDevices];
-};
-
-template <class NT, int LPR, bool J2, bool COLS>
-static int launch_rows_t(const StepRun& run, int max_group, int64_t items, bool cooperative, int max_teams,
-                         cudaStream_t s) {
-  auto kern = k_step_rows<NT, LPR, J2, COLS>;
-  static LaunchCache cache;  // the batched runner's worker threads launch concurrently
-  int dev = 0;
-  PF_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= LaunchCache::kDevices) return fail(POLFED_EINVAL, "device ordinal beyond the launch cache");
-  {
-    std::lock_guard<std::mutex> lk(cache.mu);
-    auto& c = cache.d[dev];
-    if (!c.set) {
-      int optin = 0;
-      PF_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-      cudaFuncAttributes fa;
-      PF_CUDA(cudaFuncGetAttributes(&fa, kern));
-      c.maxdyn = optin - (int)fa.sharedSizeBytes;
-      PF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, c.maxdyn));
-      PF_CUDA(cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev));
-      c.set = true;
-    }
-  }
-  const int nsm = cache.d[dev].nsm;
-  int tile = ((max_group + 1) * 16 * LPR + 15) & ~15;
-  const int per_team = tile + 2 * (int)sizeof(WorkItem<NT>);
-  int teams = std::min(max_teams, cache.d[dev].maxdyn / per_team);
-  if (teams < 1) return fail(POLFED_EINVAL, "slice tile does not fit in shared memory");
-  // one CTA per SM; as many teams as there are work items for them
-  const int grid = (int)std::min<int64_t>(nsm, items);
-  teams = (int)std::min<int64_t>(teams, (items + grid - 1) / grid);
-  StepRun r = run;
-  void* args[] = {(void*)&r, (void*)&tile};
-  if (cooperative)
-    PF_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kTeam * teams), args, (size_t)per_team * teams, s));
-  else
-    PF_CUDA(cudaLaunchKernel((const void*)kern, dim3(grid), dim3(kTeam * teams), args, (size_t)per_team * teams, s));
-  return grid;
-}
-
 // Launch the steps of `run`: the grid size (> 0), or a negative status.
-static int launch_rows(const StepRun& run, int kind, int lpr, bool j2, bool cols, int max_group, int64_t items,
+static int launch_rows(const StepRun& run, int kind, int lpr, bool j2, StepMode mode, int max_group, int64_t items,
                        bool cooperative, cudaStream_t s, int max_teams = kMaxTeams) {
-#define PF_L(NT_, L_)                                                                          \
-  case L_:                                                                                     \
-    return j2 ? launch_rows_t<NT_, L_, true, false>(run, max_group, items, cooperative, max_teams, s)     \
-              : launch_rows_t<NT_, L_, false, false>(run, max_group, items, cooperative, max_teams, s);
-#define PF_C(L_)                                                                               \
-  case L_:                                                                                     \
-    return j2 ? launch_rows_t<RF32, L_, true, true>(run, max_group, items, cooperative, max_teams, s)     \
-              : launch_rows_t<RF32, L_, false, true>(run, max_group, items, cooperative, max_teams, s);
-  if (cols) {
-    if (kind != POLFED_F32) return fail(POLFED_EINVAL, "per-column coefficients need FP32 storage");
-    switch (lpr) { PF_C(1) PF_C(2) PF_C(4) PF_C(8) }
-  } else if (kind == POLFED_F32) {
-    switch (lpr) { PF_L(RF32, 1) PF_L(RF32, 2) PF_L(RF32, 4) PF_L(RF32, 8) }
-  } else if (kind == POLFED_F64) {
-    switch (lpr) { PF_L(RF64, 1) PF_L(RF64, 2) PF_L(RF64, 4) PF_L(RF64, 8) }
-  } else if (kind == POLFED_DF64) {
-    switch (lpr) { PF_L(RDF, 1) PF_L(RDF, 2) PF_L(RDF, 4) PF_L(RDF, 8) }
+  switch (kind) {
+    case POLFED_F32: return launch_rows_f32(run, lpr, j2, mode, max_group, items, cooperative, max_teams, s);
+    case POLFED_F64: return launch_rows_f64(run, lpr, j2, mode, max_group, items, cooperative, max_teams, s);
+    case POLFED_DF64: return launch_rows_df(run, lpr, j2, mode, max_group, items, cooperative, max_teams, s);
   }
-#undef PF_L
-#undef PF_C
-  return fail(POLFED_EINVAL, "unsupported lanes-per-row");
+  return fail(POLFED_EINVAL, "bad dtype");
 }
 
 // A cooperative grid fills the GPU and its CTAs wait for one another, so only
@@ -974,6 +910,29 @@ static int check_timeout(HamPlan& plan, cudaStream_t s) {
   return POLFED_OK;
 }
 
+// The parts of a cooperative run over `ns` slices that its mode does not change.
+static int cooperative_run(HamPlan& plan, int kind, const FilterShape& f, int ns, double invD, const SliceBufs& b,
+                           cudaStream_t s, StepRun* run) {
+  PF_CHECK(check_operator(plan, kind));
+  PF_CHECK(plan.prepare_rec(f.lpr, s));
+  *run = StepRun{};
+  run->one = make_job(plan, kind, f.lpr, invD);
+  run->one.xs = b.xs;
+  run->one.ba = b.ba;
+  run->one.bb = b.bb;
+  run->n_jobs = ns;
+  run->stride = (int64_t)f.slice;
+  run->bar = (unsigned*)(plan.err_flag + 16);
+  run->err = plan.err_flag;
+  run->cap = wait_cap(kBarrierWaitPolls);
+  return POLFED_OK;
+}
+
+// steps of a launch: it stays under about a quarter of a second, and its coefficients fit the parameters
+static int steps_per_launch(double row_bytes) {
+  return std::min(kParamSteps, std::max(2, (int)(0.25 * 3e12 / (4.0 * row_bytes) + 1)));
+}
+
 // The Clenshaw steps k = K-1..1 and the final step of Eq. (2) of `ns` slices
 // (b_K in ba, X in xs), several steps to a cooperative launch: K = 200 at
 // L = 14 costs one launch instead of 200.  coef(n) gives c_n; col (device) the
@@ -981,26 +940,15 @@ static int check_timeout(HamPlan& plan, cudaStream_t s) {
 template <class Coef>
 static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, const Coef& coef, int K, double invD,
                      const float* col, int64_t colstride, const SliceBufs& b, cudaStream_t s, char** res) {
-  PF_CHECK(check_operator(plan, kind));
-  PF_CHECK(plan.prepare_rec(f.lpr, s));
+  StepRun run;
+  PF_CHECK(cooperative_run(plan, kind, f, ns, invD, b, s, &run));
   const bool j2 = plan.geo.rec_stride == 32;
-  StepRun run{};
-  run.one = make_job(plan, kind, f.lpr, invD);
-  run.one.xs = b.xs;
-  run.one.ba = b.ba;
-  run.one.bb = b.bb;
   run.one.K = K;
   run.one.colcx = col;
-  run.n_jobs = ns;
-  run.stride = (int64_t)f.slice;
   run.colstride = colstride;
-  run.bar = (unsigned*)(plan.err_flag + 16);
-  run.err = plan.err_flag;
-  run.cap = wait_cap(kBarrierWaitPolls);
   const int64_t items = (int64_t)plan.geo.n_groups * ns;
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
-  // a launch stays under about a quarter of a second, and its coefficients fit the parameters
-  const int chunk = std::min(kParamSteps, std::max(2, (int)(0.25 * 3e12 / (4.0 * row) + 1)));
+  const int chunk = steps_per_launch(row);
   std::lock_guard<std::mutex> lk(coop_mutex());
   for (int st = 0; st < K; st += chunk) {
     run.st0 = st;
@@ -1016,7 +964,7 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
       }
       alg += row * (3.0 + (c != 0.0 ? 1.0 : 0.0));
     }
-    const int grid = launch_rows(run, kind, f.lpr, j2, col != nullptr, plan.geo.max_group, items, true, s);
+    const int grid = launch_rows(run, kind, f.lpr, j2, col ? kFilterCols : kFilter, plan.geo.max_group, items, true, s);
     if (grid < 0) return grid;
     plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
     count_step(kind, alg);
@@ -1069,6 +1017,76 @@ int filter_block_cols(HamPlan& plan, const float* d_coef, int K, const void* in,
   return filter_slices(plan, POLFED_F32, f, [](int) { return 1.0; }, K, 1.0, d_coef, in, out, n_b, abi_kind, scr, s);
 }
 
+size_t moment_scratch_bytes(const HamPlan& plan, int kind, int n_b) {
+  if (kind != POLFED_DF64) return 0;
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  return f.ns * f.slice;
+}
+
+// mu[2 st + {0, 1}] += the sums of step st0 + st, in CTA order (one warp a step)
+__global__ void k_moment_sums(const double2* __restrict__ part, int n_cta, double* __restrict__ mu) {
+  double2 v = make_double2(0.0, 0.0);
+  for (int i = threadIdx.x; i < n_cta; i += 32) {
+    const double2 u = part[(size_t)blockIdx.x * n_cta + i];
+    v.x += u.x;
+    v.y += u.y;
+  }
+  for (int o = 16; o; o >>= 1) {
+    v.x += __shfl_xor_sync(~0u, v.x, o);
+    v.y += __shfl_xor_sync(~0u, v.y, o);
+  }
+  if (threadIdx.x == 0) {
+    mu[2 * blockIdx.x] += v.x;
+    mu[2 * blockIdx.x + 1] += v.y;
+  }
+}
+
+// The recurrence stays in slice layout from its first step to its last.
+// L = 18, 16 columns, float-float with t_n in FP64: a pair of moments took 53 us
+// as five launches (slice copies in and out, H~, update, sum), now 26, of which
+// about half is the FP64 pipe (conversions, update and sums of 778k elements).
+int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
+                 double* mu, FilterScratch& scr, cudaStream_t s) {
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  PF_CHECK(carve_scratch(scr, f));
+  const SliceBufs b(scr, f);
+  const int64_t dim = plan.geo.dim;
+  const int abi = kind == POLFED_F32 ? POLFED_F32 : POLFED_F64;
+  const bool j2 = plan.geo.rec_stride == 32;
+  PF_CUDA(cudaMemsetAsync(mu, 0, (size_t)2 * half * sizeof(double), s));
+  std::lock_guard<std::mutex> lk(coop_mutex());
+  for (int s0 = 0; s0 < f.nsl; s0 += f.ns) {
+    const int ns = std::min(f.ns, f.nsl - s0), col0 = s0 * f.W, ncols = std::min(ns * f.W, n_b - col0);
+    PF_CHECK(slice_in(kind, abi, in, dim, n_b, col0, ncols, f, ns, b.ba, nullptr, 0.0, nullptr, s));
+    if (kind == POLFED_DF64)
+      PF_CHECK(slice_in(POLFED_F64, abi, in, dim, n_b, col0, ncols, f, ns, b.xs, nullptr, 0.0, nullptr, s));
+    StepRun run;
+    PF_CHECK(cooperative_run(plan, kind, f, ns, 1.0, b, s, &run));
+    run.one.K = half;
+    run.one.ta = b.xs;
+    run.one.tb = (char*)t_odd;
+    run.part = (double2*)part;
+    const int64_t items = (int64_t)plan.geo.n_groups * ns;
+    const double row = (double)dim * f.W * elem_bytes(kind) * ns;
+    const int64_t per_step = std::min<int64_t>(items, kMaxMomentCtas) * sizeof(double2);
+    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(steps_per_launch(row), (int64_t)part_bytes / per_step));
+    for (int st = 0; st < half; st += chunk) {
+      run.st0 = st;
+      run.st1 = std::min(half, st + chunk);
+      run.bar_base = plan.bar_base;
+      const int n = run.st1 - run.st0;
+      const int grid = launch_rows(run, kind, f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
+      if (grid < 0) return grid;
+      plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
+      count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
+      k_moment_sums<<<n, 32, 0, s>>>((const double2*)part, grid, mu + 2 * st);
+      PF_CUDA(cudaGetLastError());
+      count_launch();
+    }
+  }
+  return check_timeout(plan, s);
+}
+
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                 cudaStream_t s) {
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
@@ -1090,7 +1108,7 @@ int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int
     const int ns = std::min(f.ns, f.nsl - s0), col0 = s0 * f.W, ncols = std::min(ns * f.W, n_b - col0);
     PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, col0, ncols, f, ns, b.xs, nullptr, 0.0, nullptr, s));
     run.n_jobs = ns;
-    const int grid = launch_rows(run, kind, f.lpr, plan.geo.rec_stride == 32, false, plan.geo.max_group,
+    const int grid = launch_rows(run, kind, f.lpr, plan.geo.rec_stride == 32, kFilter, plan.geo.max_group,
                                  (int64_t)plan.geo.n_groups * ns, false, s);
     if (grid < 0) return grid;
     count_step(kind, (double)dim * f.W * elem_bytes(kind) * ns * 3.0);
@@ -1220,7 +1238,7 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
     const double g0 = counters().step_gpu_s;
     {
       std::lock_guard<std::mutex> lk(coop_mutex());
-      grid = launch_rows(run, kind, kBatchLpr, j2, false, max_group, groups, true, s,
+      grid = launch_rows(run, kind, kBatchLpr, j2, kFilter, max_group, groups, true, s,
                          ctas_per_sm == 1 ? kMaxTeams / 2 : kMaxTeams);
       if (grid < 0) return grid;
       count_step(kind, alg);  // one launch carrying every job's steps

@@ -868,12 +868,11 @@ int kpm_rho(polfed_ctx* c, HamPlan& plan, double e_lo, double e_hi, double sigma
   scr.xs = c->fscr.p;
   scr.bytes = c->fscr.n;
   const size_t vb = ((size_t)dim * R * sizeof(double) + 255) & ~(size_t)255;
-  PF_CHECK(c->kpm.ensure(vb + kpm_buffer_bytes(dim, R, POLFED_F64), &c->ws_total, c->ws_limit));
+  PF_CHECK(c->kpm.ensure(vb + kpm_buffer_bytes(plan, kind, R), &c->ws_total, c->ws_limit));
   double* r = c->kpm.as<double>();
   PF_CHECK(c->dense.random_fill(r, dim * R, seed ^ 0x6b706d5f646f73ull, s));
-  const KpmBuffers b = kpm_carve((char*)c->kpm.p + vb, dim, R, POLFED_F64);
   std::vector<double> mu(n_mom);
-  PF_CHECK(kpm_moments(plan, kind, r, R, n_mom, mu.data(), b, scr, s));
+  PF_CHECK(kpm_moments(plan, kind, r, R, n_mom, mu.data(), (char*)c->kpm.p + vb, scr, s));
   *matvecs += (int64_t)R * ((n_mom + 1) / 2);
   const double d = std::max(0.01, 8.0 / n_mom);
   const double xa = std::max(-1.0, sigma - d), xb = std::min(1.0, sigma + d);

@@ -173,6 +173,13 @@ int filter_block_cols(HamPlan& plan, const float* d_coef, int K, const void* in,
                       FilterScratch& scr, cudaStream_t s);
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                 cudaStream_t s);
+// mu[2k] = t_k . t_k, mu[2k + 1] = t_{k+1} . t_k summed over n_b columns, t_{k+1} = 2 H~ t_k - t_{k-1}, k < half
+// (device, overwritten).  t_odd: moment_scratch_bytes (float-float keeps t_n in FP64); part: room for the sums of
+// kMaxMomentCtas CTAs of one step at least, more steps to a launch with more.  Synchronizes.
+constexpr int kMaxMomentCtas = 304;  // one per SM
+int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
+                 double* mu, FilterScratch& scr, cudaStream_t s);
+size_t moment_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 int choose_lpr(int kind, int n_b);
 
@@ -226,20 +233,13 @@ void cheb_coeffs(double sigma, int K, std::vector<double>& c, double& D);
 // Kernel polynomial method: stochastic Chebyshev moments of H~ and the
 // Jackson-damped fraction of the spectrum inside an interval.
 constexpr int kMaxKpmMoments = 65536;
-struct KpmBuffers {
-  void* t0;
-  void* t1;
-  void* y;       // three dim x R blocks of the ABI element type
-  double* part;  // per-block partial sums
-  double* mu;    // raw moment pairs
-};
 void jackson_coeffs(int N, std::vector<double>& g);
-size_t kpm_buffer_bytes(int64_t dim, int R, int abi_kind);
-KpmBuffers kpm_carve(void* base, int64_t dim, int R, int abi_kind);
+size_t kpm_buffer_bytes(const HamPlan& plan, int kind, int R);
 // mu[n] = (1/R) sum_r r^T T_n(H~) r, n < n_mom (host out); r is row-major dim x R
-// of float (kind POLFED_F32) or double.  Needs plan.prepare_typed(kind, ...).
-int kpm_moments(HamPlan& plan, int kind, const void* r, int R, int n_mom, double* mu, const KpmBuffers& b,
-                FilterScratch& scr, cudaStream_t s);
+// of float (kind POLFED_F32) or double.  Needs plan.prepare_typed(kind, ...), a
+// buffer of kpm_buffer_bytes and filter scratch for R columns.
+int kpm_moments(HamPlan& plan, int kind, const void* r, int R, int n_mom, double* mu, void* buf, FilterScratch& scr,
+                cudaStream_t s);
 double kpm_count_fraction(const double* mu, int n_mom, double x_a, double x_b);
 
 // Basis kernel (polfed_basis_build).

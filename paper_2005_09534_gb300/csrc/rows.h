@@ -1,5 +1,5 @@
 // Device code of the Clenshaw / H~ step: number policies, the group routine and
-// the step kernel (included by hamiltonian.cu only).
+// the step kernel (one translation unit per storage type instantiates it).
 #pragma once
 
 #include <type_traits>
@@ -128,6 +128,18 @@ struct RF32 {
     if (hb) fma<J2>(a, k.cB, b);
     return make_int4(__float_as_int(a.p.x), __float_as_int(a.p.y), __float_as_int(a.q.x), __float_as_int(a.q.y));
   }
+  // dot += (t . t, t' . t)
+  static __device__ __forceinline__ void dots(const int4& t, const int4& n, double2& dot) {
+    auto one = [&](int a, int b) {
+      const double c = (double)__int_as_float(a);
+      dot.x = ::fma(c, c, dot.x);
+      dot.y = ::fma((double)__int_as_float(b), c, dot.y);
+    };
+    one(t.x, n.x);
+    one(t.y, n.y);
+    one(t.z, n.z);
+    one(t.w, n.w);
+  }
 };
 
 struct RF64 {
@@ -186,6 +198,11 @@ struct RF64 {
     if (hx) fma<J2>(a, k.cX, x);
     if (hb) fma<J2>(a, k.cB, b);
     return make_int4(__double2loint(a.p), __double2hiint(a.p), __double2loint(a.q), __double2hiint(a.q));
+  }
+  static __device__ __forceinline__ void dots(const int4& t, const int4& n, double2& dot) {
+    const double c0 = __hiloint2double(t.y, t.x), c1 = __hiloint2double(t.w, t.z);
+    dot.x = ::fma(c1, c1, ::fma(c0, c0, dot.x));
+    dot.y = ::fma(__hiloint2double(n.w, n.z), c1, ::fma(__hiloint2double(n.y, n.x), c0, dot.y));
   }
 };
 
@@ -267,6 +284,25 @@ struct RDF {
     const float2 r1 = one<J2>(a.a[1], a.c[J2 ? 1 : 0], k, d, hi(own), hi(x), hi(b), hx, hb);
     return make_int4(__float_as_int(r0.x), __float_as_int(r0.y), __float_as_int(r1.x), __float_as_int(r1.y));
   }
+  // y = H~ t_n (two elements): t_{n+1} = 2 y - t_{n-1} in FP64 (y itself for n = 0), its split in r
+  static __device__ __forceinline__ double2 moment(const int4& y, const int4& t, const int4& prev, bool hb, double2& dot,
+                                                   bool live, int4& r) {
+    double v0 = (double)__int_as_float(y.x) + (double)__int_as_float(y.y);
+    double v1 = (double)__int_as_float(y.z) + (double)__int_as_float(y.w);
+    if (hb) {
+      v0 = ::fma(2.0, v0, -__hiloint2double(prev.y, prev.x));
+      v1 = ::fma(2.0, v1, -__hiloint2double(prev.w, prev.z));
+    }
+    if (live) {
+      const double c0 = __hiloint2double(t.y, t.x), c1 = __hiloint2double(t.w, t.z);
+      dot.x = ::fma(c1, c1, ::fma(c0, c0, dot.x));
+      dot.y = ::fma(v1, c1, ::fma(v0, c0, dot.y));
+    }
+    const float h0 = (float)v0, h1 = (float)v1;
+    r = make_int4(__float_as_int(h0), __float_as_int((float)(v0 - (double)h0)), __float_as_int(h1),
+                  __float_as_int((float)(v1 - (double)h1)));
+    return make_double2(v0, v1);
+  }
 };
 
 // ------------------------------------------------------------------- jobs
@@ -280,11 +316,16 @@ struct StepJob {
   const void* cx;       // typed cX in step order (a job of StepRun::jobs)
   const float* colcx;   // FP32: per-column cX, row n = order n (W floats each), or null
   char *xs, *ba, *bb;   // x, b_{k+1}, b_{k+2} (overwritten by b_k)
+  char *ta, *tb;        // moments in float-float: t_n (even n, odd n) in FP64
   double con[kConN];    // typed constants (each in its own 8 bytes)
   int K, n_groups, n_cross, c2mask;
 };
 
 constexpr int kParamSteps = 448;  // step coefficients that travel in the kernel parameters
+
+// What a step computes: the filter's recurrence, with a scalar or a per-column
+// c_n, or t_{n+1} = 2 H~ t_n - t_{n-1} with the sums t_n . t_n and t_{n+1} . t_n.
+enum StepMode { kFilter, kFilterCols, kMoments };
 
 struct StepRun {
   StepJob one;            // jobs == nullptr: n_jobs slices of this operator, buffers `stride` bytes apart
@@ -296,6 +337,7 @@ struct StepRun {
   unsigned bar_base;
   uint32_t cap;
   int* err;
+  double2* part;          // moments: the two sums of each CTA, gridDim.x entries per step from st0 on
   double cx[kParamSteps]; // jobs == nullptr: cX of the steps from st0 on, each in its own 8 bytes
 };
 
@@ -339,6 +381,7 @@ struct alignas(16) WorkItem {
   typename NT::C fhi;
   int64_t pad;
   const char *b1, *x, *rec, *fc, *cxt, *col;  // col: the step's per-column cX
+  char* t;                                    // moments in float-float: t_{n-1} in FP64 (x: t_n)
   char* out;                                  // and b2
   typename NT::Coef k;
   int n_cross, c2mask, flags;                 // flags: 1 = reads x, 2 = reads b2
@@ -346,7 +389,7 @@ struct alignas(16) WorkItem {
 
 // One step of one group (the rows sharing s_hi) by a team:
 //   out = cX x + cH (H~ b1) + cB b2,  out in place of b2.
-template <class NT, int LPR, bool J2, bool COLS, int RMAX>
+template <class NT, int LPR, bool J2, StepMode MODE, int RMAX>
 struct GroupStep {
   using C = typename NT::C;
   using Acc = typename NT::template Acc<J2>;
@@ -360,10 +403,11 @@ struct GroupStep {
   static constexpr int RSB = 2 * RS;
   static constexpr int HU = 2;                     // high neighbours in flight per row
   static constexpr int STEP = kTeam * 16;          // bytes between a thread's consecutive rows
+  static constexpr bool T64 = MODE == kMoments && std::is_same<NT, RDF>::value;  // t_n kept in FP64 beside its split
 
   template <int R>
   static __device__ __forceinline__ void pass(const Item* I, int blk, int n_g, const unsigned char* tile, bool& ready,
-                                              int team) {
+                                              int team, double2& dot) {
     const int l32 = threadIdx.x & 31, lane16 = (l32 % LPR) * 16;
     int row = blk * RPW + l32 / LPR;
     bool live = true;
@@ -383,10 +427,10 @@ struct GroupStep {
     if (hx) {
       const char* p = (const char*)lds64(&I->x) + goff;
 #pragma unroll
-      for (int i = 0; i < R; i++) xv[i] = ld_stream(p + i * STEP);
+      for (int i = 0; i < R; i++) xv[i] = T64 ? ld_l2(p + i * STEP) : ld_stream(p + i * STEP);
     }
     if (hb) {
-      const char* p = (const char*)lds64(&I->out) + goff;
+      const char* p = (const char*)lds64(T64 ? (const void*)&I->t : (const void*)&I->out) + goff;
 #pragma unroll
       for (int i = 0; i < R; i++) bv[i] = ld_l2(p + i * STEP);
     }
@@ -507,20 +551,29 @@ struct GroupStep {
       const C* cxt = (const C*)lds64(&I->cxt);
       char* out = (char*)lds64(&I->out) + goff;
       float4 cxv = make_float4(0.f, 0.f, 0.f, 0.f);
-      if constexpr (COLS) cxv = __ldg(reinterpret_cast<const float4*>((const char*)lds64(&I->col) + lane16));
+      if constexpr (MODE == kFilterCols) cxv = __ldg(reinterpret_cast<const float4*>((const char*)lds64(&I->col) + lane16));
       const C fhi = I->fhi;
       const Coef kf = NT::load_fin(&I->k);
 #pragma unroll
       for (int i = 0; i < R; i++) {
         const C d = NT::add3(__ldg(fc + i * (kTeam / LPR)), fhi, __ldg(cxt + pat[i]));
         const int4 own = *reinterpret_cast<const int4*>(tile + ROWB + ro + i * STEP);
-        const int4 r = NT::template fin<J2>(acc[i], kf, d, own, xv[i], bv[i], hx, hb, COLS, cxv);
+        int4 r;
+        if constexpr (T64) {
+          const int4 y = NT::template fin<J2>(acc[i], kf, d, own, xv[i], bv[i], false, false, false, cxv);
+          const double2 v = NT::moment(y, xv[i], bv[i], hb, dot, R > 1 || live, r);
+          if (R > 1 || live) __stcg(reinterpret_cast<double2*>((char*)lds64(&I->t) + goff + i * STEP), v);
+        } else {
+          r = NT::template fin<J2>(acc[i], kf, d, own, xv[i], bv[i], hx, hb, MODE == kFilterCols, cxv);
+          if constexpr (MODE == kMoments)
+            if (R > 1 || live) NT::dots(own, r, dot);
+        }
         if (R > 1 || live) __stcg(reinterpret_cast<int4*>(out + i * STEP), r);
       }
     }
   }
 
-  static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w) {
+  static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w, double2& dot) {
     const int n_g = lds32(&I->g.n_g);
     {
       const char* src = (const char*)lds64(&I->b1) + (size_t)(uint32_t)lds32(&I->g.r0) * ROWB;
@@ -532,8 +585,8 @@ struct GroupStep {
     const int nblk = (n_g + RPW - 1) / RPW, nfull = n_g / RPW;
     int blk = w;
     if constexpr (RMAX >= 2)
-      for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team);
-    for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team);
+      for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team, dot);
+    for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team, dot);
     if (!ready) {
       cp_async_wait();
       team_sync(team);
@@ -598,7 +651,7 @@ __device__ __forceinline__ bool grid_wait(unsigned* count, unsigned target, int*
 // L = 14 FP64 37 -> 6.3, L = 18 float-float 28 -> 9, L = 20 J1-J2 float-float
 // 91 -> 66, L = 20 J1-J2 FP32 71 -> 40, L = 22 FP32 128 -> 111, L = 24 J1-J2
 // FP32 1183 -> 800.
-template <class NT, int LPR, bool J2, bool COLS>
+template <class NT, int LPR, bool J2, StepMode MODE>
 __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_constant__ StepRun R, int tile_bytes) {
   using C = typename NT::C;
   using Item = WorkItem<NT>;
@@ -643,18 +696,28 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       I->n_cross = J->n_cross;
       I->c2mask = J->c2mask;
       const int kk = J->K - 1 - st;
+      bool last = kk == 0, first = st == 0;
       C cx = C();
-      if constexpr (COLS)
+      if constexpr (MODE == kMoments) {  // t_1 = H~ t_0, then 2 H~ t_n - t_{n-1}; float-float always takes H~ t_n
+        last = first = first || std::is_same<NT, RDF>::value;
+        I->x = (st & 1) ? J->tb + so : J->ta + so;
+        I->t = (st & 1) ? J->ta + so : J->tb + so;
+      } else if constexpr (MODE == kFilterCols) {
         I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * (4 * LPR));
-      else
+      } else {
         cx = R.jobs ? __ldg(reinterpret_cast<const C*>(J->cx) + st) : *reinterpret_cast<const C*>(&R.cx[st - R.st0]);
-      const typename NT::Coef k = NT::make(J->con, kk == 0, st == 0, cx);
+      }
+      const typename NT::Coef k = NT::make(J->con, last, first, cx);
       I->k = k;
-      I->flags = (COLS || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
+      if constexpr (MODE == kMoments)
+        I->flags = (std::is_same<NT, RDF>::value ? 1 : 0) | (st > 0 ? 2 : 0);
+      else
+        I->flags = (MODE == kFilterCols || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
     }
     return true;
   };
   bool more = fetch();
+  double2 dot = make_double2(0.0, 0.0);
   for (;;) {
     while (more) {
       cp_async_wait();
@@ -662,7 +725,22 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       const Item* I = items + (r & 1);
       r++;
       more = fetch();
-      GroupStep<NT, LPR, J2, COLS, RMAX>::run(I, tile, team, tt >> 5);
+      GroupStep<NT, LPR, J2, MODE, RMAX>::run(I, tile, team, tt >> 5, dot);
+    }
+    if constexpr (MODE == kMoments) {
+      __shared__ double2 wsum[kTeam * kMaxTeams / 32];
+      for (int o = 16; o; o >>= 1) {
+        dot.x += __shfl_xor_sync(~0u, dot.x, o);
+        dot.y += __shfl_xor_sync(~0u, dot.y, o);
+      }
+      if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = dot;
+      __syncthreads();
+      if (threadIdx.x == 32) {
+        for (int w = 0; w < (int)blockDim.x / 32; w++)
+          if (w != 1) dot = make_double2(dot.x + wsum[w].x, dot.y + wsum[w].y);
+        R.part[(size_t)(st - R.st0) * gridDim.x + blockIdx.x] = dot;
+      }
+      dot = make_double2(0.0, 0.0);
     }
     if (++st == R.st1) break;
     grid_arrive(R.bar);
@@ -673,5 +751,13 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
   }
   cp_async_wait();
 }
+
+// Launch the steps of `run` on up to max_teams teams per SM: the grid size (> 0), or a negative status.
+int launch_rows_f32(const StepRun& run, int lpr, bool j2, StepMode mode, int max_group, int64_t items, bool cooperative,
+                    int max_teams, cudaStream_t s);
+int launch_rows_f64(const StepRun& run, int lpr, bool j2, StepMode mode, int max_group, int64_t items, bool cooperative,
+                    int max_teams, cudaStream_t s);
+int launch_rows_df(const StepRun& run, int lpr, bool j2, StepMode mode, int max_group, int64_t items, bool cooperative,
+                   int max_teams, cudaStream_t s);
 
 }  // namespace polfed
