@@ -377,6 +377,13 @@ union V16 {
   S s[16 / sizeof(S)];
 };
 
+// a chunk's elements as they are stored (float-float: both hi, then both lo)
+template <class NT>
+__device__ __forceinline__ int4 stored(const int4& v) {
+  if constexpr (std::is_same<NT, RDF>::value) return make_int4(v.x, v.z, v.y, v.w);
+  return v;
+}
+
 template <class NT>
 __device__ __forceinline__ typename NT::C col_cx_scale(const float* colscale, int c, typename NT::C cscale) {
   if constexpr (std::is_same<NT, RF32>::value) {
@@ -430,8 +437,8 @@ __global__ void k_slice_in(const In* __restrict__ in, int64_t dim, int ld, int c
         a.s[v] = Conv<NT>::mul(col_cx_scale<NT>(colscale ? colscale + sl * colstride : nullptr, c + v, cscale), o.s[v]);
     }
     const int64_t d = sl * stride + r * W + c;
-    if (xs) *reinterpret_cast<int4*>(xs + d) = o.i;
-    if (a_scaled) *reinterpret_cast<int4*>(a_scaled + d) = a.i;
+    if (xs) *reinterpret_cast<int4*>(xs + d) = stored<NT>(o.i);
+    if (a_scaled) *reinterpret_cast<int4*>(a_scaled + d) = stored<NT>(a.i);
   }
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0 && flag) atomicMax(reinterpret_cast<int*>(flag), __float_as_int(mx));
@@ -453,7 +460,7 @@ __global__ void k_slice_out(const typename NT::S* __restrict__ ys, int64_t dim, 
     const int q = (int)(e - r * cpr), sl = q / cps, c = (q - sl * cps) * VEC, cc = sl * W + c;
     if (cc >= ncols) continue;
     V16<S> u;
-    u.i = *reinterpret_cast<const int4*>(ys + sl * stride + r * W + c);
+    u.i = stored<NT>(*reinterpret_cast<const int4*>(ys + sl * stride + r * W + c));  // its own inverse
     Out o[VEC];
 #pragma unroll
     for (int v = 0; v < VEC; v++) {

@@ -50,6 +50,36 @@ __device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
   return fast_two_sum(p, e);
 }
 
+// The same on two values at once, each in one half of a pair (packed FP32
+// instructions; rounding and order are those of the scalar forms).  The
+// float-float step issues 2.2 instructions a clock with scalar ones: L = 20,
+// J1-J2, 32 columns took 65 us a step and slice, packed 60, and with two rows
+// of a thread in flight, which their registers then allow, 56.
+struct DF2 {
+  float2 h, l;
+};
+__device__ __forceinline__ float2 pair(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, pair(-1.f), a); }
+__device__ __forceinline__ DF2 fast_two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  return DF2{s, __fadd2_rn(b, sub2(a, s))};
+}
+__device__ __forceinline__ DF2 two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b), t = sub2(a, s);  // t = -(s - a)
+  return DF2{s, __fadd2_rn(sub2(a, __fadd2_rn(s, t)), __fadd2_rn(b, t))};
+}
+__device__ __forceinline__ DF2 df_add(const DF2& a, const DF2& b) {
+  const DF2 s = two_sum(a.h, b.h);
+  return fast_two_sum(s.h, __fadd2_rn(s.l, __fadd2_rn(a.l, b.l)));
+}
+__device__ __forceinline__ DF2 df_mul(float2 c, const DF2& b) {  // c: one (hi, lo) for both
+  const float2 p = __fmul2_rn(pair(c.x), b.h);
+  float2 e = __ffma2_rn(pair(c.x), b.h, make_float2(-p.x, -p.y));
+  e = __ffma2_rn(pair(c.x), b.l, e);
+  e = __ffma2_rn(pair(c.y), b.h, e);
+  return fast_two_sum(p, e);
+}
+
 // A policy works on 16-byte chunks of a row (int4 as loaded):
 //   S, C         storage element and constant type
 //   Acc          running sums over a row's neighbours (zero / add1 / add2: coupling class 1 / 2)
@@ -207,7 +237,7 @@ struct RF64 {
 };
 
 struct RDF {
-  using S = float2;  // (hi, lo)
+  using S = float2;  // (hi, lo); two neighbouring elements are stored as (hi, hi, lo, lo)
   using C = float2;
   struct Coef {
     float2 o1, o2, cH, cX, cB;
@@ -218,9 +248,11 @@ struct RDF {
   static __device__ __forceinline__ Coef load_fin(const Coef* k) { return *k; }
   template <bool J2>
   struct Acc {
-    float2 a[2];  // per element (running hi sum, accumulated low parts and rounding errors)
-    float2 c[J2 ? 2 : 1];
+    DF2 a, c;  // running hi sums, accumulated low parts and rounding errors; c: coupling class 2
   };
+  static __device__ __forceinline__ DF2 chunk(const int4& v) {
+    return DF2{make_float2(__int_as_float(v.x), __int_as_float(v.y)), make_float2(__int_as_float(v.z), __int_as_float(v.w))};
+  }
   static __device__ __forceinline__ bool pow2(float2 v) {
     return v.y == 0.f && (__float_as_uint(v.x) & 0x7FFFFFu) == 0;
   }
@@ -240,55 +272,54 @@ struct RDF {
   static __device__ __forceinline__ bool has_b(const Coef& k) { return k.cB.x != 0.f; }
   template <bool J2>
   static __device__ __forceinline__ void zero(Acc<J2>& a) {
-    a.a[0] = a.a[1] = make_float2(0.f, 0.f);
-    if constexpr (J2) a.c[0] = a.c[1] = make_float2(0.f, 0.f);
+    a.a = DF2{pair(0.f), pair(0.f)};
+    if constexpr (J2) a.c = a.a;
   }
-  static __device__ __forceinline__ void acc(float2& a, int hi, int lo) {
-    const float2 s = two_sum(a.x, __int_as_float(hi));
-    a.x = s.x;
-    a.y += s.y + __int_as_float(lo);
+  static __device__ __forceinline__ void acc(DF2& a, const int4& u) {
+    const DF2 v = chunk(u), s = two_sum(a.h, v.h);
+    a.h = s.h;
+    a.l = __fadd2_rn(a.l, __fadd2_rn(s.l, v.l));
   }
   template <bool J2>
   static __device__ __forceinline__ void add1(Acc<J2>& a, const Sum&, const int4& u) {
-    acc(a.a[0], u.x, u.y);
-    acc(a.a[1], u.z, u.w);
+    acc(a.a, u);
   }
   template <bool J2>
   static __device__ __forceinline__ void add2(Acc<J2>& a, const Sum&, const int4& u) {
-    acc(a.c[0], u.x, u.y);
-    acc(a.c[J2 ? 1 : 0], u.z, u.w);
+    acc(a.c, u);
   }
   static __device__ __forceinline__ float2 add3(float2 a, float2 b, float2 c) { return df_add(df_add(a, b), c); }
   template <bool J2>
-  static __device__ __forceinline__ float2 one(float2 s1, float2 s2, const Coef& k, float2 d, float2 own, float2 x,
-                                               float2 b, bool hx, bool hb) {
-    float2 y = df_add(df_mul(d, own), df_mul(k.o1, fast_two_sum(s1.x, s1.y)));
-    if constexpr (J2) y = df_add(y, df_mul(k.o2, fast_two_sum(s2.x, s2.y)));
-    if (k.exact) {
-      float2 r = make_float2(k.cH.x * y.x, k.cH.x * y.y);
-      if (hx) r = df_add(r, make_float2(k.cX.x * x.x, k.cX.x * x.y));
-      if (hb) r = df_add(r, make_float2(k.cB.x * b.x, k.cB.x * b.y));
-      return r;
-    }
-    float2 r = df_mul(k.cH, y);
-    if (hx) r = df_add(r, df_mul(k.cX, x));
-    if (hb) r = df_add(r, df_mul(k.cB, b));
-    return r;
-  }
-  template <bool J2>
   static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, float2 d, const int4& own, const int4& x,
                                              const int4& b, bool hx, bool hb, bool, const float4&) {
-    auto lo = [](const int4& v) { return make_float2(__int_as_float(v.x), __int_as_float(v.y)); };
-    auto hi = [](const int4& v) { return make_float2(__int_as_float(v.z), __int_as_float(v.w)); };
-    const float2 r0 = one<J2>(a.a[0], a.c[0], k, d, lo(own), lo(x), lo(b), hx, hb);
-    const float2 r1 = one<J2>(a.a[1], a.c[J2 ? 1 : 0], k, d, hi(own), hi(x), hi(b), hx, hb);
-    return make_int4(__float_as_int(r0.x), __float_as_int(r0.y), __float_as_int(r1.x), __float_as_int(r1.y));
+    DF2 y = df_add(df_mul(d, chunk(own)), df_mul(k.o1, fast_two_sum(a.a.h, a.a.l)));
+    if constexpr (J2) y = df_add(y, df_mul(k.o2, fast_two_sum(a.c.h, a.c.l)));
+    auto scaled = [](float c, const DF2& v) { return DF2{__fmul2_rn(pair(c), v.h), __fmul2_rn(pair(c), v.l)}; };
+    DF2 r;
+    if (k.exact) {
+      r = scaled(k.cH.x, y);
+      if (hx) r = df_add(r, scaled(k.cX.x, chunk(x)));
+      if (hb) r = df_add(r, scaled(k.cB.x, chunk(b)));
+    } else {
+      r = df_mul(k.cH, y);
+      if (hx) r = df_add(r, df_mul(k.cX, chunk(x)));
+      if (hb) r = df_add(r, df_mul(k.cB, chunk(b)));
+    }
+    return make_int4(__float_as_int(r.h.x), __float_as_int(r.h.y), __float_as_int(r.l.x), __float_as_int(r.l.y));
+  }
+  // (double)v of a float by integer operations: with the FP64 pipe's conversions
+  // (2 a clock and SM) a pair of moments at L = 18, 16 columns takes 26 us, so 23
+  static __device__ __forceinline__ double f2d(int b) {
+    const uint32_t a = (uint32_t)b & 0x7FFFFFFFu;
+    if (a - 0x00800000u < 0x7F000000u)
+      return __hiloint2double((int)(((uint32_t)b & 0x80000000u) | ((a >> 3) + 0x38000000u)), b << 29);
+    return a == 0 ? __hiloint2double(b, 0) : (double)__int_as_float(b);
   }
   // y = H~ t_n (two elements): t_{n+1} = 2 y - t_{n-1} in FP64 (y itself for n = 0), its split in r
   static __device__ __forceinline__ double2 moment(const int4& y, const int4& t, const int4& prev, bool hb, double2& dot,
                                                    bool live, int4& r) {
-    double v0 = (double)__int_as_float(y.x) + (double)__int_as_float(y.y);
-    double v1 = (double)__int_as_float(y.z) + (double)__int_as_float(y.w);
+    double v0 = f2d(y.x) + f2d(y.z);
+    double v1 = f2d(y.y) + f2d(y.w);
     if (hb) {
       v0 = ::fma(2.0, v0, -__hiloint2double(prev.y, prev.x));
       v1 = ::fma(2.0, v1, -__hiloint2double(prev.w, prev.z));
@@ -299,8 +330,8 @@ struct RDF {
       dot.y = ::fma(v1, c1, ::fma(v0, c0, dot.y));
     }
     const float h0 = (float)v0, h1 = (float)v1;
-    r = make_int4(__float_as_int(h0), __float_as_int((float)(v0 - (double)h0)), __float_as_int(h1),
-                  __float_as_int((float)(v1 - (double)h1)));
+    r = make_int4(__float_as_int(h0), __float_as_int(h1), __float_as_int((float)(v0 - f2d(__float_as_int(h0)))),
+                  __float_as_int((float)(v1 - f2d(__float_as_int(h1)))));
     return make_double2(v0, v1);
   }
 };
@@ -401,13 +432,13 @@ struct GroupStep {
   static constexpr int MAXCR = J2 ? 6 : 2;
   static constexpr int RS = J2 ? 32 : 16;          // uint16 entries of a record
   static constexpr int RSB = 2 * RS;
-  static constexpr int HU = 2;                     // high neighbours in flight per row
   static constexpr int STEP = kTeam * 16;          // bytes between a thread's consecutive rows
   static constexpr bool T64 = MODE == kMoments && std::is_same<NT, RDF>::value;  // t_n kept in FP64 beside its split
 
   template <int R>
   static __device__ __forceinline__ void pass(const Item* I, int blk, int n_g, const unsigned char* tile, bool& ready,
                                               int team, double2& dot) {
+    constexpr int HU = R == 1 ? 4 : 2;  // high neighbours in flight per row
     const int l32 = threadIdx.x & 31, lane16 = (l32 % LPR) * 16;
     int row = blk * RPW + l32 / LPR;
     bool live = true;
@@ -655,7 +686,8 @@ template <class NT, int LPR, bool J2, StepMode MODE>
 __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_constant__ StepRun R, int tile_bytes) {
   using C = typename NT::C;
   using Item = WorkItem<NT>;
-  constexpr int RMAX = (std::is_same<NT, RDF>::value) ? 1 : 2;
+  // rows of a thread in flight (float-float moments hold t_n and t_{n-1} too: 22.6 us a pair with one, 23.8 with two)
+  constexpr int RMAX = (std::is_same<NT, RDF>::value && MODE == kMoments) ? 1 : 2;
   extern __shared__ __align__(128) unsigned char smem[];
   const int team = threadIdx.x / kTeam, tt = threadIdx.x % kTeam;
   unsigned char* tile = smem + (size_t)team * tile_bytes;
