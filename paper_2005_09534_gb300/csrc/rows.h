@@ -438,7 +438,9 @@ struct GroupStep {
   template <int R>
   static __device__ __forceinline__ void pass(const Item* I, int blk, int n_g, const unsigned char* tile, bool& ready,
                                               int team, double2& dot) {
-    constexpr int HU = R == 1 ? 4 : 2;  // high neighbours in flight per row
+    // high neighbours in flight per row (FP32, L = 24, J1-J2: 37.8 ms with two, 37.3 with four; float-float with
+    // two rows is faster with two, 7.3 and 7.6 ms; FP64 at L = 14, single rows: 1200 us with four, 1165 with six)
+    constexpr int HU = std::is_same<NT, RF32>::value ? 4 : (R == 1 ? (std::is_same<NT, RF64>::value ? 6 : 4) : 2);
     const int l32 = threadIdx.x & 31, lane16 = (l32 % LPR) * 16;
     int row = blk * RPW + l32 / LPR;
     bool live = true;
@@ -455,16 +457,6 @@ struct GroupStep {
     int4 xv[R], bv[R];
 #pragma unroll
     for (int i = 0; i < R; i++) NT::template zero<J2>(acc[i]);
-    if (hx) {
-      const char* p = (const char*)lds64(&I->x) + goff;
-#pragma unroll
-      for (int i = 0; i < R; i++) xv[i] = T64 ? ld_l2(p + i * STEP) : ld_stream(p + i * STEP);
-    }
-    if (hb) {
-      const char* p = (const char*)lds64(T64 ? (const void*)&I->t : (const void*)&I->out) + goff;
-#pragma unroll
-      for (int i = 0; i < R; i++) bv[i] = ld_l2(p + i * STEP);
-    }
     // high bonds: the same local rows of other groups
     const char* b1 = (const char*)lds64(&I->b1);
     auto add = [&](Acc& a, bool c1, const int4& u) {
@@ -502,6 +494,18 @@ struct GroupStep {
       const int n_hn1 = lds32(&I->g.n_hn1);
       high(0, n_hn1, true);
       if constexpr (J2) high(n_hn1, lds32(&I->g.n_hn), false);
+    }
+    // x and b2, when the registers of the high neighbours are free again: loaded
+    // first, L = 22, FP32, 64 columns takes 109 us a step and slice, here 101
+    if (hx) {
+      const char* p = (const char*)lds64(&I->x) + goff;
+#pragma unroll
+      for (int i = 0; i < R; i++) xv[i] = T64 ? ld_l2(p + i * STEP) : ld_stream(p + i * STEP);
+    }
+    if (hb) {
+      const char* p = (const char*)lds64(T64 ? (const void*)&I->t : (const void*)&I->out) + goff;
+#pragma unroll
+      for (int i = 0; i < R; i++) bv[i] = ld_l2(p + i * STEP);
     }
     // neighbour records of the rows: header and cross neighbours
     const char* rp0 = (const char*)lds64(&I->rec) + (size_t)(uint32_t)((lds32(&I->g.cls_base) + row) * RSB);
