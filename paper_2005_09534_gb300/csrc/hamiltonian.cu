@@ -78,14 +78,16 @@ void upload_binomials() {
 // L = 18 float-float 256 moments at b = 7 / 8 / 9: 7.2, 6.9, 7.7 ms; L = 20 J1-J2
 // float-float K = 64 at b = 8 / 9 / 10: 10.1, 8.7, 9.6 ms; L = 22 FP32 K = 200 at
 // b = 8 / 9 / 10: 49.7, 46.0, 45.7 ms.
-static int choose_b(int L) {
-  int b = L <= 14 ? L - 9 : (L <= 20 ? L / 2 - 1 : 10);
+static int clamp_b(int L, int b) {
   if (const char* e = getenv("POLFED_LOWBITS")) b = atoi(e);
   if (b > 10) b = 10;
   if (b < 2) b = 2;
   if (L - b < 2) b = L - 2;
   return b;
 }
+static int choose_b(int L) { return clamp_b(L, L <= 14 ? L - 9 : (L <= 20 ? L / 2 - 1 : 10)); }
+// FP32 moments keep their split too: it decides the order of their sums (policy RF32M).
+int moments_b(int kind, int L) { return kind == POLFED_F32 ? clamp_b(L, L - 10) : 0; }
 
 int build_geometry(const polfed_model* m, int b_override, HamGeometry* g) {
   if (!m) return fail(POLFED_EINVAL, "model is NULL");
@@ -1070,6 +1072,7 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
     StepRun run;
     PF_CHECK(cooperative_run(plan, kind, f, ns, 1.0, b, s, &run));
     run.one.K = half;
+    run.one.low_first = f.lpr == 8 && plan.geo.max_group >= 32;
     run.one.ta = b.xs;
     run.one.tb = (char*)t_odd;
     run.part = (double2*)part;

@@ -179,6 +179,7 @@ int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int
 constexpr int kMaxMomentCtas = 304;  // one per SM
 int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
                  double* mu, FilterScratch& scr, cudaStream_t s);
+int moments_b(int kind, int L);  // low bits of a plan for moments, 0: the plan's own choice
 size_t moment_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 int choose_lpr(int kind, int n_b);

@@ -93,6 +93,7 @@ __device__ __forceinline__ DF2 df_mul(float2 c, const DF2& b) {  // c: one (hi, 
 enum { kConS1, kConS2, kConS1Last, kConS2Last, kConInvD, kConN };
 
 struct RF32 {
+  static constexpr bool kBondOrder = false;
   using S = float;
   using C = float;
   struct Coef {
@@ -173,6 +174,7 @@ struct RF32 {
 };
 
 struct RF64 {
+  static constexpr bool kBondOrder = false;
   using S = double;
   using C = double;
   struct Coef {
@@ -236,7 +238,51 @@ struct RF64 {
   }
 };
 
+// FP32 moments.  They are returned in FP64 though each carries FP32 rounding
+// noise of 1e-8: other sums of the same neighbours would differ from earlier
+// results by that much.  So this policy keeps the sums as they have always been:
+// neighbours by plain addition in bond order, then d own + o1 sum1 + o2 sum2.
+struct RF32M : RF32 {
+  static constexpr bool kBondOrder = true;
+  struct Sum {};
+  static __device__ __forceinline__ Sum load_sum(const Coef*) { return Sum{}; }
+  static __device__ __forceinline__ Coef load_fin(const Coef* k) { return *k; }
+  template <bool J2>
+  struct Acc {
+    float2 p, q, p2, q2;
+  };
+  template <bool J2>
+  static __device__ __forceinline__ void zero(Acc<J2>& a) {
+    a.p = a.q = a.p2 = a.q2 = make_float2(0.f, 0.f);
+  }
+  static __device__ __forceinline__ float2 lo(const int4& u) { return make_float2(__int_as_float(u.x), __int_as_float(u.y)); }
+  static __device__ __forceinline__ float2 hi(const int4& u) { return make_float2(__int_as_float(u.z), __int_as_float(u.w)); }
+  template <bool J2>
+  static __device__ __forceinline__ void add1(Acc<J2>& a, const Sum&, const int4& u) {
+    a.p = __fadd2_rn(a.p, lo(u));
+    a.q = __fadd2_rn(a.q, hi(u));
+  }
+  template <bool J2>
+  static __device__ __forceinline__ void add2(Acc<J2>& a, const Sum&, const int4& u) {
+    a.p2 = __fadd2_rn(a.p2, lo(u));
+    a.q2 = __fadd2_rn(a.q2, hi(u));
+  }
+  template <bool J2>
+  static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, float d, const int4& own, const int4&,
+                                             const int4& b, bool, bool hb, bool, const float4&) {
+    auto one = [&](float2 s1, float2 s2, float2 o, float2 bb) {
+      const float2 dd = make_float2(d, d), o1 = make_float2(k.s1, k.s1), o2 = make_float2(k.s2, k.s2);
+      float2 y = __ffma2_rn(dd, o, __fmul2_rn(o1, s1));
+      if constexpr (J2) y = __ffma2_rn(o2, s2, y);
+      return hb ? __ffma2_rn(make_float2(2.f, 2.f), y, make_float2(-bb.x, -bb.y)) : y;
+    };
+    const float2 x = one(a.p, a.p2, lo(own), lo(b)), y = one(a.q, a.q2, hi(own), hi(b));
+    return make_int4(__float_as_int(x.x), __float_as_int(x.y), __float_as_int(y.x), __float_as_int(y.y));
+  }
+};
+
 struct RDF {
+  static constexpr bool kBondOrder = false;
   using S = float2;  // (hi, lo); two neighbouring elements are stored as (hi, hi, lo, lo)
   using C = float2;
   struct Coef {
@@ -350,6 +396,7 @@ struct StepJob {
   char *ta, *tb;        // moments in float-float: t_n (even n, odd n) in FP64
   double con[kConN];    // typed constants (each in its own 8 bytes)
   int K, n_groups, n_cross, c2mask;
+  int low_first;        // FP32 moments: low bonds before high ones
 };
 
 constexpr int kParamSteps = 448;  // step coefficients that travel in the kernel parameters
@@ -415,7 +462,7 @@ struct alignas(16) WorkItem {
   char* t;                                    // moments in float-float: t_{n-1} in FP64 (x: t_n)
   char* out;                                  // and b2
   typename NT::Coef k;
-  int n_cross, c2mask, flags;                 // flags: 1 = reads x, 2 = reads b2
+  int n_cross, c2mask, flags;                 // flags: 1 = reads x, 2 = reads b2, 4 = low bonds first
 };
 
 // One step of one group (the rows sharing s_hi) by a team:
@@ -608,6 +655,72 @@ struct GroupStep {
     }
   }
 
+  // The same step with the neighbours in bond order (RF32M): high, low, cross
+  // bonds, or low, cross, high where the job says so.
+  static __device__ __forceinline__ void pass_in_order(const Item* I, int blk, int n_g, const unsigned char* tile,
+                                                       bool& ready, int team, double2& dot) {
+    const int l32 = threadIdx.x & 31, lane16 = (l32 % LPR) * 16;
+    const bool live = blk * RPW + l32 / LPR < n_g;
+    const int row = min(blk * RPW + l32 / LPR, n_g - 1);
+    const uint32_t ro = (uint32_t)(row * ROWB + lane16);
+    const size_t goff = (size_t)(uint32_t)lds32(&I->g.r0) * ROWB + ro;
+    const int flags = lds32(&I->flags);
+    const char* b1 = (const char*)lds64(&I->b1);
+    const typename NT::Sum k = NT::load_sum(&I->k);
+    const int4 bv = (flags & 2) ? ld_l2((const char*)lds64(&I->out) + goff) : make_int4(0, 0, 0, 0);
+    Acc acc;
+    NT::template zero<J2>(acc);
+    auto add = [&](bool c1, const int4& u) {
+      if (!J2 || c1)
+        NT::template add1<J2>(acc, k, u);
+      else
+        NT::template add2<J2>(acc, k, u);
+    };
+    const int n_hn = lds32(&I->g.n_hn), n_hn1 = lds32(&I->g.n_hn1), n_cross = lds32(&I->n_cross);
+    const uint16_t* rec = (const uint16_t*)lds64(&I->rec) + (size_t)(uint32_t)(lds32(&I->g.cls_base) + row) * RS;
+    const uint32_t pat = ~((uint32_t)__ldg(rec) ^ (uint32_t)lds32(&I->g.need_mask)) & ((1u << n_cross) - 1u);
+    auto high = [&]() {
+      auto src = [&](int j) { return ld_l2(b1 + ro + (size_t)(uint32_t)lds32(&I->g.hn_base[j]) * ROWB); };
+      int j = 0;
+      for (; j + 4 <= n_hn; j += 4) {
+        int4 u[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) u[q] = src(j + q);
+#pragma unroll
+        for (int q = 0; q < 4; q++) add(j + q < n_hn1, u[q]);
+      }
+      for (; j < n_hn; j++) add(j < n_hn1, src(j));
+    };
+    if (!(flags & 4)) high();
+    if (!ready) {
+      cp_async_wait();
+      team_sync(team);
+      ready = true;
+    }
+    const uint32_t cnt = __ldg(rec + 1);
+    for (int e = 0; e < (int)(cnt & 0xFF); e++)
+      add(true, *reinterpret_cast<const int4*>(tile + lane16 + __ldg(rec + low_entry(e, true))));
+    if constexpr (J2)
+      for (int e = 0; e < (int)(cnt >> 8); e++)
+        add(false, *reinterpret_cast<const int4*>(tile + lane16 + __ldg(rec + low_entry(e, false))));
+    for (int c = 0; c < n_cross; c++)
+      if ((pat >> c) & 1)
+        add(!J2 || !((lds32(&I->c2mask) >> c) & 1),
+            ld_l2(b1 + lane16 + (size_t)(uint32_t)lds32(&I->g.cr_base[c]) * ROWB - ROWB + __ldg(rec + 2 + c)));
+    if (flags & 4) high();
+    const C d = NT::add3(__ldg((const C*)lds64(&I->fc) + lds32(&I->g.cls_base) + row), I->fhi,
+                         __ldg((const C*)lds64(&I->cxt) + pat));
+    const int4 own = *reinterpret_cast<const int4*>(tile + ROWB + ro);
+    const int4 r = NT::template fin<J2>(acc, NT::load_fin(&I->k), d, own, bv, bv, false, flags & 2, false,
+                                        make_float4(0.f, 0.f, 0.f, 0.f));
+    if (live) {
+      NT::dots(own, r, dot);
+      __stcg(reinterpret_cast<int4*>((char*)lds64(&I->out) + goff), r);
+    }
+  }
+  // entry of the e-th low neighbour in a record
+  static __device__ __forceinline__ int low_entry(int e, bool c1) { return J2 ? (c1 ? 8 : 18) + e : 4 + e; }
+
   static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w, double2& dot) {
     const int n_g = lds32(&I->g.n_g);
     {
@@ -619,9 +732,13 @@ struct GroupStep {
     bool ready = false;
     const int nblk = (n_g + RPW - 1) / RPW, nfull = n_g / RPW;
     int blk = w;
-    if constexpr (RMAX >= 2)
-      for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team, dot);
-    for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team, dot);
+    if constexpr (NT::kBondOrder) {
+      for (; blk < nblk; blk += NW) pass_in_order(I, blk, n_g, tile, ready, team, dot);
+    } else {
+      if constexpr (RMAX >= 2)
+        for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team, dot);
+      for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team, dot);
+    }
     if (!ready) {
       cp_async_wait();
       team_sync(team);
@@ -734,8 +851,8 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       const int kk = J->K - 1 - st;
       bool last = kk == 0, first = st == 0;
       C cx = C();
-      if constexpr (MODE == kMoments) {  // t_1 = H~ t_0, then 2 H~ t_n - t_{n-1}; float-float always takes H~ t_n
-        last = first = first || std::is_same<NT, RDF>::value;
+      if constexpr (MODE == kMoments) {  // t_1 = H~ t_0, then 2 H~ t_n - t_{n-1}; FP32 and float-float take H~ t_n and finish it
+        last = first = first || !std::is_same<NT, RF64>::value;
         I->x = (st & 1) ? J->tb + so : J->ta + so;
         I->t = (st & 1) ? J->ta + so : J->tb + so;
       } else if constexpr (MODE == kFilterCols) {
@@ -746,7 +863,7 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       const typename NT::Coef k = NT::make(J->con, last, first, cx);
       I->k = k;
       if constexpr (MODE == kMoments)
-        I->flags = (std::is_same<NT, RDF>::value ? 1 : 0) | (st > 0 ? 2 : 0);
+        I->flags = (std::is_same<NT, RDF>::value ? 1 : 0) | (st > 0 ? 2 : 0) | (J->low_first ? 4 : 0);
       else
         I->flags = (MODE == kFilterCols || NT::has_x(k) ? 1 : 0) | (NT::has_b(k) ? 2 : 0);
     }
