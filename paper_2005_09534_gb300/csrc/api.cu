@@ -114,8 +114,7 @@ int polfed_h_apply(const polfed_model* model, const uint32_t* d_states, int64_t 
   PF_CHECK(check_bounds(e_lo, e_hi));
   cudaStream_t s = (cudaStream_t)stream;
   HamPlan plan;
-  PF_CHECK(plan.init(model, s, true));
-  PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
+  PF_CHECK(plan.init(model, s, true, -1, dtype, e_lo, e_hi));
   StreamScratch mem;
   mem.s = s;
   FilterScratch scr;
@@ -150,8 +149,7 @@ int polfed_cheb_filter(const polfed_model* model, const uint32_t* d_states, int6
   for (double v : c) csum += std::fabs(v);
   cudaStream_t s = (cudaStream_t)stream;
   HamPlan plan;
-  PF_CHECK(plan.init(model, s, true));
-  PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
+  PF_CHECK(plan.init(model, s, true, -1, dtype, e_lo, e_hi));
   StreamScratch mem;
   mem.s = s;
   FilterScratch scr;
@@ -191,8 +189,7 @@ int polfed_cheb_filter_cols(const polfed_model* model, const uint32_t* d_states,
     }
   cudaStream_t s = (cudaStream_t)stream;
   HamPlan plan;
-  PF_CHECK(plan.init(model, s, true));
-  PF_CHECK(plan.prepare_typed(POLFED_F32, e_lo, e_hi));
+  PF_CHECK(plan.init(model, s, true, -1, POLFED_F32, e_lo, e_hi));
   StreamScratch mem, cmem;
   mem.s = s;
   cmem.s = s;

@@ -101,7 +101,6 @@ class Rendezvous : public FilterHook {
     r.in.assign(in, in + npan);
     r.out.assign(out, out + npan);
     r.S = S;
-    PF_CHECK(plan.prepare_rec(kBatchLpr, s));
     if (cudaEventCreateWithFlags(&r.ready, cudaEventDisableTiming) != cudaSuccess)
       return fail(POLFED_ECUDA, "cudaEventCreate failed");
     cudaEventRecord(r.ready, s);
@@ -248,7 +247,6 @@ int autotune(const std::vector<polfed_model>& models, const std::vector<int>& N_
     PF_CHECK(plans[i].init(&models[i], s, false, batch_b(models[i].L)));
     const double b = norm_bound(models[i]);
     PF_CHECK(plans[i].prepare_typed(kind, -b, b));
-    PF_CHECK(plans[i].prepare_rec(kBatchLpr, s));
     vec_bytes += (size_t)plans[i].geo.dim * 64 * sizeof(double);
   }
   DeviceBuffer X, Y, scr;
@@ -331,9 +329,7 @@ int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const
     if (!(sigma[i] > -1.0 && sigma[i] < 1.0)) return fail(POLFED_EINVAL, "sigma must be in (-1, 1)");
     if (K[i] < 0 || K[i] > 10000000) return fail(POLFED_EINVAL, "K must be in 0..1e7");
     if (!d_X[i] || !d_Y[i] || d_X[i] == d_Y[i]) return fail(POLFED_EINVAL, "bad X / Y pointers");
-    PF_CHECK(plans[i].init(&models[i], s, true, batch_b(models[i].L)));
-    PF_CHECK(plans[i].prepare_typed(dtype, e_lo[i], e_hi[i]));
-    PF_CHECK(plans[i].prepare_rec(kBatchLpr, s));
+    PF_CHECK(plans[i].init(&models[i], s, true, batch_b(models[i].L), dtype, e_lo[i], e_hi[i]));
     double D = 1.0;
     cheb_coeffs(sigma[i], K[i], coefs[i], D);
     items.push_back(BatchFilterItem{&plans[i], coefs[i].data(), K[i], 1.0 / D, d_X[i], d_Y[i], n_b, false});

@@ -39,6 +39,7 @@ namespace polfed {
 
 // ------------------------------------------------------------- binomials
 __constant__ uint32_t c_binom[33][33];
+__device__ uint32_t d_binom[33][33];  // for divergent reads
 static uint32_t h_binom[33][33];
 static std::once_flag h_binom_once;
 
@@ -67,6 +68,7 @@ void upload_binomials() {
   std::lock_guard<std::mutex> lk(mu);
   if (dev < 64 && (done >> dev) & 1) return;
   cudaMemcpyToSymbol(c_binom, h_binom, sizeof(h_binom));
+  cudaMemcpyToSymbol(d_binom, h_binom, sizeof(h_binom));
   if (dev < 64) done |= (1ull << dev);
 }
 
@@ -205,47 +207,147 @@ static ClassStart class_starts(const HamGeometry& g) {
   return cs;
 }
 
-// Everything that needs no other table: low part (T_lo, U_lo, F_lo), high part
-// (T_hi, F_hi, the group schedule) and the cross-bond diagonal.
-__global__ void k_tables(const HamGeometry g, const ClassStart cs, HamTables t) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < (1 << g.b)) {
+// alpha- and beta-scaled diagonals of one storage type: low part by cls_off +
+// local index, then the groups in schedule order (alpha * (F_hi - beta)), then
+// the cross patterns.  kind < 0: none.
+struct TypedOut {
+  int kind;
+  double alpha, beta;
+  void* out;
+  __device__ __forceinline__ void put(int i, double v) const {
+    if (kind == POLFED_F32)
+      reinterpret_cast<float*>(out)[i] = (float)v;
+    else if (kind == POLFED_F64)
+      reinterpret_cast<double*>(out)[i] = v;
+    else
+      reinterpret_cast<float2*>(out)[i] = make_float2((float)v, (float)(v - (double)(float)v));
+  }
+};
+
+// All tables of a plan in one launch: thread i < n_main does low state i (rank,
+// diagonal), high state i (rank, diagonal, its group's place in the schedule and
+// its record) and cross pattern i; the threads after them one entry of a
+// neighbour record each.  A state's neighbours are ranked again instead of being
+// read from another launch's table, with the binomials in shared memory (as
+// divergent reads of constant memory they are serialized).  Bound by launches and
+// latency: the four kernels this replaces took 21 us and three more launches at
+// L = 22, this one 17; an L = 12 call with one column took 52 us, now 42.
+constexpr int kTableThreads = 128;
+__global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, const ClassStart cs, HamTables t, int* err,
+                                                          TypedOut ty, int n_main) {
+  __shared__ uint32_t B[33][33];
+  for (int e = threadIdx.x; e < 33 * 33; e += kTableThreads) (&B[0][0])[e] = (&d_binom[0][0])[e];
+  __syncthreads();
+  const int i = blockIdx.x * kTableThreads + threadIdx.x;
+  auto rank_lo = [&](uint32_t a) {
     uint32_t r = 0;
-    int k = 0;
-    for (int p = 0; p < g.b; p++)
-      if ((i >> p) & 1) r += c_binom[p][++k];
+    for (int k = 1; a; a &= a - 1, k++) r += B[__ffs(a) - 1][k];
+    return r;
+  };
+  const int RS = g.rec_stride, j = i - n_main;
+  if (j >= 0) {  // neighbour records (layout in HamTables::rec): one entry, for every row size
+    if (j >= RS << g.b) return;
+    const uint32_t a = (uint32_t)(j / RS);
+    const int e = j % RS, l1 = RS == 32 ? 8 : 4;  // l1: first low entry, after the cross neighbours
+    auto active = [&](int q0, int n, int want, int* cnt) {  // the want-th active low bond of a class
+      uint32_t m = 0;
+      *cnt = 0;
+      for (int q = q0; q < q0 + n; q++)
+        if (__popc(a & g.low_mask[q]) == 1 && (*cnt)++ == want) m = g.low_mask[q];
+      return m;
+    };
+    uint32_t flip = 0, v = 0;
+    int n1, n2;
+    if (e == 0) {
+      for (int q = 0; q < g.n_cross; q++) v |= ((a >> g.cross_lo[q]) & 1u) << q;
+    } else if (e == 1) {
+      active(0, g.n_low1, -1, &n1);
+      active(g.n_low1, g.n_low2, -1, &n2);
+      v = (uint32_t)(n1 | (n2 << 8));
+    } else if (e < l1) {
+      if (e - 2 < g.n_cross) flip = 1u << g.cross_lo[e - 2];
+    } else if (e < l1 + 10 || RS == 16) {
+      flip = active(0, g.n_low1, e - l1, &n1);
+    } else {
+      flip = active(g.n_low1, g.n_low2, e - l1 - 10, &n2);
+    }
+    const uint32_t row = flip ? rank_lo(a ^ flip) + 1 : 0;
+    const size_t o = ((size_t)g.cls_off[__popc(a)] + rank_lo(a)) * RS + e;
+    for (int q = 0; q < 4; q++) t.rec[q][o] = (uint16_t)(e < 2 ? v : row * (16u << q));
+    return;
+  }
+  if (i < 64) err[i] = 0;
+  if (i < (1 << g.b)) {
+    const uint32_t a = (uint32_t)i, r = rank_lo(a);
+    const int pos = g.cls_off[__popc(a)] + (int)r;
     t.T_lo[i] = (uint16_t)r;
-    t.U_lo[g.cls_off[k] + r] = (uint16_t)i;
+    t.U_lo[pos] = (uint16_t)i;
     double d = 0.0;
-    const int nl = g.n_low1 + g.n_low2;
-    for (int q = 0; q < nl; q++) {
+    for (int q = 0; q < g.n_low1 + g.n_low2; q++) {
       const double J = q < g.n_low1 ? g.J1 : g.J2;
-      d += J * g.Delta * (__popc(i & g.low_mask[q]) == 1 ? -0.25 : 0.25);
+      d += J * g.Delta * (__popc(a & g.low_mask[q]) == 1 ? -0.25 : 0.25);
     }
     for (int q = 0; q < g.b; q++) d += g.h[q] * (((i >> q) & 1) ? 0.5 : -0.5);
     t.F_lo[i] = d;
+    if (ty.kind >= 0) ty.put(pos, ty.alpha * d);
   }
   if (i < (1 << g.nh)) {
-    const int pc = __popc(i), n_lo = g.n_up - pc;
+    const uint32_t grp = (uint32_t)i;
+    const int pc = __popc(grp), n_lo = g.n_up - pc;
+    // first row of the group: its bits sit above n_lo low ones
+    auto rank_hi = [&](uint32_t a) {
+      uint32_t r = 0;
+      for (int k = g.n_up - __popc(a) + 1; a; a &= a - 1, k++) r += B[g.b + __ffs(a) - 1][k];
+      return (int)r;
+    };
+    auto valid = [&](uint32_t a) {
+      const int n = g.n_up - __popc(a);
+      return n >= 0 && n <= g.b;
+    };
     int T = -1;
     double d = 0.0;
-    if (n_lo >= 0 && n_lo <= g.b) {
-      uint32_t r = 0, ro = 0;
-      int k = 0;
-      for (int q = 0; q < g.nh; q++)
-        if ((i >> q) & 1) {
-          ++k;
-          r += c_binom[g.b + q][n_lo + k];
-          ro += c_binom[q][k];  // rank among nh-bit strings of popcount pc
-        }
-      T = (int)r;
+    if (valid(grp)) {
+      T = rank_hi(grp);
       const int nhb = g.n_high1 + g.n_high2;
       for (int q = 0; q < nhb; q++) {
         const double J = q < g.n_high1 ? g.J1 : g.J2;
-        d += J * g.Delta * (__popc(i & g.high_mask[q]) == 1 ? -0.25 : 0.25);
+        d += J * g.Delta * (__popc(grp & g.high_mask[q]) == 1 ? -0.25 : 0.25);
       }
       for (int q = 0; q < g.nh; q++) d += g.h[g.b + q] * (((i >> q) & 1) ? 0.5 : -0.5);
-      t.order[cs.v[pc] + (int)ro] = i;
+      const int pos = cs.v[pc] + (int)rank_lo(grp);  // among the nh-bit strings of its popcount
+      t.order[pos] = i;
+      GroupRec* r = t.grec + pos;
+      r->r0 = T;
+      r->n_g = (int)B[g.b][n_lo];
+      r->cls_base = g.cls_off[n_lo];
+      int cnt = 0, cnt1 = 0;
+      for (int k = 0; k < nhb; k++) {
+        const uint32_t m = g.high_mask[k];
+        if (__popc(grp & m) != 1) continue;
+        r->hn_base[cnt++] = rank_hi(grp ^ m);
+        if (k < g.n_high1) cnt1++;
+      }
+      for (int k = cnt; k < kMaxHigh; k++) r->hn_base[k] = 0;
+      r->n_hn = cnt;
+      r->n_hn1 = cnt1;
+      int need = 0;
+      for (int k = 0; k < 8; k++) {
+        int base = 0, n = 0;
+        if (k < g.n_cross) {
+          if (!((grp >> g.cross_hi[k]) & 1)) need |= 1 << k;  // the low bit must differ from the high bit
+          const uint32_t g2 = grp ^ (1u << g.cross_hi[k]);
+          // rows with the bond antiparallel exist only if the neighbouring class is valid
+          if (valid(g2)) {
+            base = rank_hi(g2);
+            n = (int)B[g.b][g.n_up - __popc(g2)];
+          }
+        }
+        r->cr_base[k] = base;
+        r->cr_n[k] = n;
+      }
+      r->need_mask = need;
+      r->pad0 = r->pad1 = 0;
+      if (ty.kind >= 0) ty.put((1 << g.b) + pos, ty.alpha * (d - ty.beta));
     }
     t.T_hi[i] = T;
     t.F_hi[i] = d;
@@ -257,75 +359,8 @@ __global__ void k_tables(const HamGeometry g, const ClassStart cs, HamTables t) 
       d += J * g.Delta * (((i >> k) & 1) ? -0.25 : 0.25);
     }
     t.C_x[i] = d;
+    if (ty.kind >= 0) ty.put((1 << g.b) + g.n_groups + i, ty.alpha * d);
   }
-}
-
-// Per-group constants in schedule order.
-__global__ void k_tables_groups(const HamGeometry g, const int32_t* T_hi, const int32_t* order, GroupRec* gr) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= g.n_groups) return;
-  const int grp = order[idx];
-  GroupRec r;
-  const int n_lo = g.n_up - __popc(grp);
-  r.r0 = T_hi[grp];
-  r.n_g = (int)c_binom[g.b][n_lo];
-  r.cls_base = g.cls_off[n_lo];
-  int cnt = 0, cnt1 = 0;
-  for (int k = 0; k < g.n_high1 + g.n_high2; k++) {
-    const uint32_t m = g.high_mask[k];
-    if (__popc((uint32_t)grp & m) == 1 && cnt < kMaxHigh) {
-      r.hn_base[cnt++] = T_hi[grp ^ m];
-      if (k < g.n_high1) cnt1++;
-    }
-  }
-  for (int k = cnt; k < kMaxHigh; k++) r.hn_base[k] = 0;
-  r.n_hn = cnt;
-  r.n_hn1 = cnt1;
-  int need = 0;
-  for (int k = 0; k < 8; k++) {
-    r.cr_base[k] = 0;
-    r.cr_n[k] = 0;
-    if (k < g.n_cross) {
-      const int hb = (grp >> g.cross_hi[k]) & 1;
-      if (!hb) need |= 1 << k;  // the low bit must differ from the high bit
-      const int g2 = grp ^ (1 << g.cross_hi[k]);
-      const int n_lo2 = g.n_up - __popc(g2);
-      // rows with the bond antiparallel exist only if the neighbouring class is valid
-      if (T_hi[g2] >= 0 && n_lo2 >= 0 && n_lo2 <= g.b) {
-        r.cr_base[k] = T_hi[g2];
-        r.cr_n[k] = (int)c_binom[g.b][n_lo2];
-      }
-    }
-  }
-  r.need_mask = need;
-  r.pad0 = r.pad1 = 0;
-  gr[idx] = r;
-}
-
-// Neighbour records for rows of `rowb` bytes (layout in HamTables::rec).
-__global__ void k_tables_rec(const HamGeometry g, const uint16_t* T_lo, uint16_t* rec, int rowb) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= (1 << g.b)) return;
-  const int RS = g.rec_stride;
-  uint16_t* r = rec + (size_t)(g.cls_off[__popc(a)] + T_lo[a]) * RS;
-  for (int e = 0; e < RS; e++) r[e] = 0;
-  int n1 = 0, n2 = 0;
-  uint32_t pat = 0;
-  const int l1 = RS == 32 ? 8 : 4;  // first low entry, after the cross neighbours
-  for (int k = 0; k < g.n_low1; k++) {
-    const uint32_t m = g.low_mask[k];
-    if (__popc((uint32_t)a & m) == 1) r[l1 + n1++] = (uint16_t)((T_lo[a ^ m] + 1) * rowb);
-  }
-  for (int k = g.n_low1; k < g.n_low1 + g.n_low2; k++) {
-    const uint32_t m = g.low_mask[k];
-    if (__popc((uint32_t)a & m) == 1) r[l1 + 10 + n2++] = (uint16_t)((T_lo[a ^ m] + 1) * rowb);
-  }
-  for (int k = 0; k < g.n_cross; k++) {
-    pat |= (uint32_t)((a >> g.cross_lo[k]) & 1) << k;
-    r[2 + k] = (uint16_t)((T_lo[a ^ (1 << g.cross_lo[k])] + 1) * rowb);
-  }
-  r[0] = (uint16_t)pat;
-  r[1] = (uint16_t)(n1 | (n2 << 8));
 }
 
 // -------------------------------------------------------- bounded waits
@@ -505,19 +540,17 @@ __global__ void k_slice_out(const typename NT::S* __restrict__ ys, int64_t dim, 
 
 // Typed, alpha/beta-scaled diagonal tables: F_lo by class order | F_hi in
 // schedule order | C_x.
-template <class NT>
-__global__ void k_typed(const HamTables t, int nlo, int ngr, int ncx, double alpha, double beta,
-                        typename NT::C* out) {
+__global__ void k_typed(const HamTables t, int nlo, int ngr, int ncx, TypedOut ty) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nlo + ngr + ncx) return;
   double v;
   if (i < nlo)
-    v = alpha * t.F_lo[t.U_lo[i]];
+    v = ty.alpha * t.F_lo[t.U_lo[i]];
   else if (i < nlo + ngr)
-    v = alpha * (t.F_hi[t.order[i - nlo]] - beta);
+    v = ty.alpha * (t.F_hi[t.order[i - nlo]] - ty.beta);
   else
-    v = alpha * t.C_x[i - nlo - ngr];
-  out[i] = Conv<NT>::from_d(v);
+    v = ty.alpha * t.C_x[i - nlo - ngr];
+  ty.put(i, v);
 }
 
 // --------------------------------------------------------------- host side
@@ -559,8 +592,19 @@ struct PlanLayout {
   }
 };
 
+static int typed_out(int kind, double e_lo, double e_hi, void* dst, TypedOut* ty) {
+  if (kind < 0 || kind > 2) return fail(POLFED_EINVAL, "bad dtype");
+  *ty = TypedOut{kind, 1.0, 0.0, dst};
+  if (!(e_lo == 0.0 && e_hi == 0.0)) {
+    if (!(e_hi > e_lo)) return fail(POLFED_EINVAL, "need e_lo < e_hi");
+    ty->alpha = 2.0 / (e_hi - e_lo);
+    ty->beta = 0.5 * (e_hi + e_lo);
+  }
+  return POLFED_OK;
+}
+
 // Point the plan's tables into `base` and enqueue the kernels that fill them.
-int HamPlan::bind(char* base, cudaStream_t s) {
+int HamPlan::bind(char* base, cudaStream_t s, int kind, double e_lo, double e_hi, void* typed_dst) {
   const PlanLayout lay(geo);
   tab.T_lo = (uint16_t*)(base + lay.Tlo);
   tab.U_lo = (uint16_t*)(base + lay.Ulo);
@@ -570,53 +614,42 @@ int HamPlan::bind(char* base, cudaStream_t s) {
   tab.F_hi = (double*)(base + lay.Fhi);
   tab.C_x = (double*)(base + lay.Cx);
   tab.grec = (GroupRec*)(base + lay.Grp);
-  for (int i = 0; i < 4; i++) {
-    tab.rec[i] = (uint16_t*)(base + lay.Rec + i * lay.rec1);
-    rec_ok[i] = false;
-  }
+  for (int i = 0; i < 4; i++) tab.rec[i] = (uint16_t*)(base + lay.Rec + i * lay.rec1);
   err_flag = (int*)(base + lay.Err);
   bar_base = 0;
-  PF_CUDA(cudaMemsetAsync(err_flag, 0, 256, s));
-  const int n = std::max(std::max(1 << geo.b, 1 << geo.nh), 1 << geo.n_cross);
-  k_tables<<<(n + 255) / 256, 256, 0, s>>>(geo, class_starts(geo), tab);
-  k_tables_groups<<<(unsigned)((geo.n_groups + 127) / 128), 128, 0, s>>>(geo, tab.T_hi, tab.order, tab.grec);
+  TypedOut ty{-1, 1.0, 0.0, nullptr};
+  if (kind >= 0) {
+    PF_CHECK(typed_out(kind, e_lo, e_hi, typed_dst, &ty));
+    typed[kind] = typed_dst;
+    typed_ok[kind] = true;
+    typed_lo[kind] = e_lo;
+    typed_hi[kind] = e_hi;
+  }
+  const int n_main = (std::max({64, 1 << geo.b, 1 << geo.nh, 1 << geo.n_cross}) + kTableThreads - 1) / kTableThreads;
+  const int n_rec = ((geo.rec_stride << geo.b) + kTableThreads - 1) / kTableThreads;
+  k_tables<<<n_main + n_rec, kTableThreads, 0, s>>>(geo, class_starts(geo), tab, err_flag, ty, n_main * kTableThreads);
   PF_CUDA(cudaGetLastError());
   return POLFED_OK;
-}
-
-int HamPlan::init(const polfed_model* m, cudaStream_t s, bool stream_ordered, int b_override) {
-  release();
-  upload_binomials();
-  PF_CHECK(build_geometry(m, b_override, &geo));
-  stream = s;
-  stream_alloc = stream_ordered;
-  const size_t bytes = PlanLayout(geo).total;
-  if (stream_ordered)
-    PF_CUDA(cudaMallocAsync(&dev, bytes, s));
-  else
-    PF_CUDA(cudaMalloc(&dev, bytes));
-  return bind((char*)dev, s);
 }
 
 static size_t typed_bytes_of(const HamGeometry& g) {
   return (((size_t)1 << g.b) + ((size_t)1 << g.n_cross) + (size_t)g.n_groups) * 8 + 512;
 }
 
-static int fill_typed(const HamPlan& p, int kind, double e_lo, double e_hi, void* dst, cudaStream_t s) {
-  double alpha = 1.0, beta = 0.0;
-  if (!(e_lo == 0.0 && e_hi == 0.0)) {
-    if (!(e_hi > e_lo)) return fail(POLFED_EINVAL, "need e_lo < e_hi");
-    alpha = 2.0 / (e_hi - e_lo);
-    beta = 0.5 * (e_hi + e_lo);
-  }
-  const int nlo = 1 << p.geo.b, ncx = 1 << p.geo.n_cross, ngr = p.geo.n_groups, n = nlo + ncx + ngr;
-  switch (kind) {
-    case POLFED_F32: k_typed<RF32><<<(n + 255) / 256, 256, 0, s>>>(p.tab, nlo, ngr, ncx, alpha, beta, (float*)dst); break;
-    case POLFED_F64: k_typed<RF64><<<(n + 255) / 256, 256, 0, s>>>(p.tab, nlo, ngr, ncx, alpha, beta, (double*)dst); break;
-    default: k_typed<RDF><<<(n + 255) / 256, 256, 0, s>>>(p.tab, nlo, ngr, ncx, alpha, beta, (float2*)dst); break;
-  }
-  PF_CUDA(cudaGetLastError());
-  return POLFED_OK;
+int HamPlan::init(const polfed_model* m, cudaStream_t s, bool stream_ordered, int b_override, int kind, double e_lo,
+                  double e_hi) {
+  release();
+  upload_binomials();
+  PF_CHECK(build_geometry(m, b_override, &geo));
+  stream = s;
+  stream_alloc = stream_ordered;
+  const size_t bytes = PlanLayout(geo).total, all = bytes + (kind >= 0 ? typed_bytes_of(geo) : 0);
+  if (stream_ordered)
+    PF_CUDA(cudaMallocAsync(&dev, all, s));
+  else
+    PF_CUDA(cudaMalloc(&dev, all));
+  dev_end = (char*)dev + all;
+  return bind((char*)dev, s, kind, e_lo, e_hi, (char*)dev + bytes);
 }
 
 int HamPlan::prepare_typed(int kind, double e_lo, double e_hi) {
@@ -629,20 +662,14 @@ int HamPlan::prepare_typed(int kind, double e_lo, double e_hi) {
       PF_CUDA(cudaMalloc(&typed[kind], typed_bytes_of(geo)));
   }
   typed_ok[kind] = false;
-  PF_CHECK(fill_typed(*this, kind, e_lo, e_hi, typed[kind], stream));
+  TypedOut ty;
+  PF_CHECK(typed_out(kind, e_lo, e_hi, typed[kind], &ty));
+  const int nlo = 1 << geo.b, ncx = 1 << geo.n_cross, n = nlo + geo.n_groups + ncx;
+  k_typed<<<(n + 255) / 256, 256, 0, stream>>>(tab, nlo, geo.n_groups, ncx, ty);
+  PF_CUDA(cudaGetLastError());
   typed_ok[kind] = true;
   typed_lo[kind] = e_lo;
   typed_hi[kind] = e_hi;
-  return POLFED_OK;
-}
-
-int HamPlan::prepare_rec(int lpr, cudaStream_t s) {
-  const int i = lpr_index(lpr);
-  if (rec_ok[i]) return POLFED_OK;
-  const int nlo = 1 << geo.b;
-  k_tables_rec<<<(nlo + 255) / 256, 256, 0, s>>>(geo, tab.T_lo, tab.rec[i], 16 * lpr);
-  PF_CUDA(cudaGetLastError());
-  rec_ok[i] = true;
   return POLFED_OK;
 }
 
@@ -654,7 +681,7 @@ void HamPlan::release() {
       cudaFree(dev);
   }
   for (int k = 0; k < 3; k++) {
-    if (typed[k]) {
+    if (typed[k] && !(typed[k] >= dev && typed[k] < dev_end)) {  // not part of dev
       if (stream_alloc)
         cudaFreeAsync(typed[k], stream);
       else
@@ -923,7 +950,6 @@ static int check_timeout(HamPlan& plan, cudaStream_t s) {
 static int cooperative_run(HamPlan& plan, int kind, const FilterShape& f, int ns, double invD, const SliceBufs& b,
                            cudaStream_t s, StepRun* run) {
   PF_CHECK(check_operator(plan, kind));
-  PF_CHECK(plan.prepare_rec(f.lpr, s));
   *run = StepRun{};
   run->one = make_job(plan, kind, f.lpr, invD);
   run->one.xs = b.xs;
@@ -1102,7 +1128,6 @@ int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
   PF_CHECK(carve_scratch(scr, f));
   PF_CHECK(check_operator(plan, kind));
-  PF_CHECK(plan.prepare_rec(f.lpr, s));
   const SliceBufs b(scr, f);
   const int64_t dim = plan.geo.dim;
   StepRun run{};
@@ -1191,7 +1216,6 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
     const HamGeometry& g = p.geo;
     if ((g.rec_stride == 32) != j2) return fail(POLFED_EINVAL, "batched filter: all jobs must agree on J2 = 0 or not");
     PF_CHECK(check_operator(p, kind));
-    if (!p.rec_ok[lpr_index(kBatchLpr)]) return fail(POLFED_EINVAL, "batched filter: record tables not prepared");
     const FilterShape f = batch_shape(g, kind, it.n_b);
     float* flag = (float*)(base + Lo.flags_off + 16 * q);
     char* xs = base + pos;
@@ -1415,12 +1439,7 @@ static int static_filter(const polfed_model* model, double e_lo, double e_hi, co
   char* d = (char*)base;
   plan.stream = s;
   plan.stream_alloc = false;
-  PF_CHECK(plan.bind(d, s));
-  PF_CHECK(fill_typed(plan, dtype, e_lo, e_hi, d + tab, s));
-  plan.typed[dtype] = d + tab;
-  plan.typed_ok[dtype] = true;
-  plan.typed_lo[dtype] = e_lo;
-  plan.typed_hi[dtype] = e_hi;
+  PF_CHECK(plan.bind(d, s, dtype, e_lo, e_hi, d + tab));
   FilterScratch scr;
   scr.xs = d + tab + typ;
   scr.bytes = bytes - tab - typ;

@@ -93,8 +93,7 @@ int polfed_kpm_moments(const polfed_model* model, const uint32_t* d_states, int6
   if (!std::isfinite(e_lo) || !std::isfinite(e_hi) || !(e_lo < e_hi)) return fail(POLFED_EINVAL, "need e_lo < e_hi");
   cudaStream_t s = (cudaStream_t)stream;
   HamPlan plan;
-  PF_CHECK(plan.init(model, s, true, moments_b(dtype, model->L)));
-  PF_CHECK(plan.prepare_typed(dtype, e_lo, e_hi));
+  PF_CHECK(plan.init(model, s, true, moments_b(dtype, model->L), dtype, e_lo, e_hi));
   const size_t fb = (filter_scratch_bytes(plan, dtype, R) + 255) & ~(size_t)255;
   void* mem = nullptr;
   PF_CUDA(cudaMallocAsync(&mem, fb + kpm_buffer_bytes(plan, dtype, R), s));

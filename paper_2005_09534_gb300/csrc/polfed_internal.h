@@ -133,21 +133,23 @@ class HamPlan {
   HamGeometry geo;
   HamTables tab{};
   void* dev = nullptr;       // one allocation for all tables
+  void* dev_end = nullptr;
   int* err_flag = nullptr;   // set by a kernel whose bounded wait expired
   unsigned bar_base = 0;     // arrivals counted so far on the grid barrier (err_flag + 16)
   // per-precision alpha/beta-scaled tables (k_typed), indexed by dtype
   void* typed[3] = {nullptr, nullptr, nullptr};
   bool typed_ok[3] = {false, false, false};
   double typed_lo[3] = {0, 0, 0}, typed_hi[3] = {0, 0, 0};
-  bool rec_ok[4] = {false, false, false, false};
   cudaStream_t stream = nullptr;
   bool stream_alloc = false;  // tables from cudaMallocAsync
 
   // All of these only enqueue work on the stream.
-  int init(const polfed_model* m, cudaStream_t s, bool stream_ordered, int b_override = -1);
-  int bind(char* base, cudaStream_t s);                   // tables in caller memory (geo already set)
+  // kind >= 0: with the scaled tables of that storage type (prepare_typed in the same launch)
+  int init(const polfed_model* m, cudaStream_t s, bool stream_ordered, int b_override = -1, int kind = -1,
+           double e_lo = 0.0, double e_hi = 0.0);
+  // tables (and typed_dst, kind >= 0) in caller memory, geo already set
+  int bind(char* base, cudaStream_t s, int kind = -1, double e_lo = 0.0, double e_hi = 0.0, void* typed_dst = nullptr);
   int prepare_typed(int kind, double e_lo, double e_hi);  // alpha/beta-scaled tables
-  int prepare_rec(int lpr, cudaStream_t s);               // neighbour records for this lanes-per-row
   void release();
   ~HamPlan() { release(); }
 };
@@ -189,7 +191,7 @@ int choose_lpr(int kind, int n_b);
 // order and coefficients (F32 or DF64 storage; all jobs J2 == 0 or all not).
 constexpr int kBatchLpr = 8;  // 128-byte slices
 struct BatchFilterItem {
-  HamPlan* plan;          // prepare_typed(kind, ...) and prepare_rec(kBatchLpr, ...) done
+  HamPlan* plan;          // prepare_typed(kind, ...) done
   const double* coef;     // host, K + 1 coefficients: Y = invD * sum_n coef[n] T_n(H~) X
   int K;
   double invD;

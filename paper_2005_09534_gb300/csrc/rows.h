@@ -385,7 +385,7 @@ struct RDF {
 // ------------------------------------------------------------------- jobs
 // One column slice of one operator going through its Clenshaw steps.
 struct StepJob {
-  const uint16_t* rec;  // neighbour records (k_tables_rec)
+  const uint16_t* rec;  // neighbour records (HamTables::rec)
   const GroupRec* grec;
   const void* Fc;       // typed, alpha-scaled diagonal of the low part, by cls_off + local index
   const void* Fhi;      // of the high part (schedule order, includes -alpha*beta)
