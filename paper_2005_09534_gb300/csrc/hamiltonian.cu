@@ -790,6 +790,32 @@ static FilterShape filter_shape(const HamGeometry& g, int kind, int n_b, size_t 
 
 constexpr size_t kSliceSet = (size_t)96 << 20;  // of the 126 MB L2
 
+// The launches of a block: sets of ns slices, and the columns that do not fill
+// the last slice by themselves in a narrower one.  Small problems, whose slices
+// all run together, keep the padded slice: it shares their launch.  L = 20,
+// J1-J2, FP32, 37 columns, K = 48: 4.33 ms as two slices of 32, 3.19 as one and
+// one of 8 (2.05 and 0.92 in the steps).
+struct SlicePart {
+  FilterShape f;
+  int ns, s0, col0, ncols;  // slices s0.. of columns col0..
+};
+
+static std::vector<SlicePart> slice_parts(const HamGeometry& g, int kind, const FilterShape& f, int n_b) {
+  std::vector<SlicePart> parts;
+  const int rem = n_b % f.W;
+  const bool split = f.nsl > f.ns && rem > 0 && choose_lpr(kind, rem) < f.lpr;
+  const int nfull = f.nsl - (split ? 1 : 0);
+  for (int s0 = 0; s0 < nfull; s0 += f.ns) {
+    const int ns = std::min(f.ns, nfull - s0), col0 = s0 * f.W;
+    parts.push_back(SlicePart{f, ns, s0, col0, std::min(ns * f.W, n_b - col0)});
+  }
+  if (split) {
+    FilterShape t = filter_shape(g, kind, rem, 0);
+    parts.push_back(SlicePart{t, 1, nfull, nfull * f.W, rem});
+  }
+  return parts;
+}
+
 size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b) {
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
   return 3 * (size_t)f.ns * f.slice + 256;
@@ -974,13 +1000,14 @@ static int steps_per_launch(double row_bytes) {
 // per-column rows instead.  The result is in *res.
 template <class Coef>
 static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, const Coef& coef, int K, double invD,
-                     const float* col, int64_t colstride, const SliceBufs& b, cudaStream_t s, char** res) {
+                     const float* col, int64_t colstride, int colw, const SliceBufs& b, cudaStream_t s, char** res) {
   StepRun run;
   PF_CHECK(cooperative_run(plan, kind, f, ns, invD, b, s, &run));
   const bool j2 = plan.geo.rec_stride == 32;
   run.one.K = K;
   run.one.colcx = col;
   run.colstride = colstride;
+  run.one.colw = colw;
   const int64_t items = (int64_t)plan.geo.n_groups * ns;
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
   const int chunk = steps_per_launch(row);
@@ -1014,27 +1041,26 @@ static int filter_slices(HamPlan& plan, int kind, const FilterShape& f, const Co
                          const float* d_col, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                          cudaStream_t s) {
   PF_CHECK(carve_scratch(scr, f));
-  const SliceBufs b(scr, f);
   const int64_t dim = plan.geo.dim;
   const int64_t colstride = d_col ? (int64_t)(K + 1) * f.W : 0;
   PF_CUDA(cudaMemsetAsync(scr.flag, 0, 16, s));
-  for (int s0 = 0; s0 < f.nsl; s0 += f.ns) {
-    const int ns = std::min(f.ns, f.nsl - s0), col0 = s0 * f.W, ncols = std::min(ns * f.W, n_b - col0);
+  for (const SlicePart& p : slice_parts(plan.geo, kind, f, n_b)) {
+    const SliceBufs b(scr, p.f);
     if (K == 0) {
-      PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, col0, ncols, f, ns, nullptr, b.ba, coef(0) * invD, scr.flag, s));
-      PF_CHECK(slice_out(kind, abi_kind, b.ba, dim, f, ns, ncols, out, n_b, col0, scr.flag, s));
+      PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, nullptr, b.ba, coef(0) * invD, scr.flag, s));
+      PF_CHECK(slice_out(kind, abi_kind, b.ba, dim, p.f, p.ns, p.ncols, out, n_b, p.col0, scr.flag, s));
       continue;
     }
-    const float* col = d_col ? d_col + s0 * colstride : nullptr;
+    const float* col = d_col ? d_col + p.s0 * colstride : nullptr;
     // b_K = c_K X (in ba); b_{K+1} = 0 is not read by the first step
-    PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, col0, ncols, f, ns, b.xs, b.ba, col ? 1.0 : coef(K), scr.flag, s,
-                      col ? col + (size_t)K * f.W : nullptr, colstride));
+    PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.xs, b.ba, col ? 1.0 : coef(K), scr.flag,
+                      s, col ? col + (size_t)K * f.W : nullptr, colstride));
     char* res = nullptr;
     StepTimer tm(s, kind);
-    PF_CHECK(run_steps(plan, kind, f, ns, coef, K, invD, col, colstride, b, s, &res));
+    PF_CHECK(run_steps(plan, kind, p.f, p.ns, coef, K, invD, col, colstride, f.W, b, s, &res));
     PF_CHECK(tm.stop());
     PF_CHECK(check_timeout(plan, s));
-    PF_CHECK(slice_out(kind, abi_kind, res, dim, f, ns, ncols, out, n_b, col0, scr.flag, s));
+    PF_CHECK(slice_out(kind, abi_kind, res, dim, p.f, p.ns, p.ncols, out, n_b, p.col0, scr.flag, s));
   }
   return POLFED_OK;
 }
@@ -1084,26 +1110,25 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
                  double* mu, FilterScratch& scr, cudaStream_t s) {
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
   PF_CHECK(carve_scratch(scr, f));
-  const SliceBufs b(scr, f);
   const int64_t dim = plan.geo.dim;
   const int abi = kind == POLFED_F32 ? POLFED_F32 : POLFED_F64;
   const bool j2 = plan.geo.rec_stride == 32;
   PF_CUDA(cudaMemsetAsync(mu, 0, (size_t)2 * half * sizeof(double), s));
   std::lock_guard<std::mutex> lk(coop_mutex());
-  for (int s0 = 0; s0 < f.nsl; s0 += f.ns) {
-    const int ns = std::min(f.ns, f.nsl - s0), col0 = s0 * f.W, ncols = std::min(ns * f.W, n_b - col0);
-    PF_CHECK(slice_in(kind, abi, in, dim, n_b, col0, ncols, f, ns, b.ba, nullptr, 0.0, nullptr, s));
+  for (const SlicePart& p : slice_parts(plan.geo, kind, f, n_b)) {
+    const SliceBufs b(scr, p.f);
+    PF_CHECK(slice_in(kind, abi, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.ba, nullptr, 0.0, nullptr, s));
     if (kind == POLFED_DF64)
-      PF_CHECK(slice_in(POLFED_F64, abi, in, dim, n_b, col0, ncols, f, ns, b.xs, nullptr, 0.0, nullptr, s));
+      PF_CHECK(slice_in(POLFED_F64, abi, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.xs, nullptr, 0.0, nullptr, s));
     StepRun run;
-    PF_CHECK(cooperative_run(plan, kind, f, ns, 1.0, b, s, &run));
+    PF_CHECK(cooperative_run(plan, kind, p.f, p.ns, 1.0, b, s, &run));
     run.one.K = half;
     run.one.low_first = f.lpr == 8 && plan.geo.max_group >= 32;
     run.one.ta = b.xs;
     run.one.tb = (char*)t_odd;
     run.part = (double2*)part;
-    const int64_t items = (int64_t)plan.geo.n_groups * ns;
-    const double row = (double)dim * f.W * elem_bytes(kind) * ns;
+    const int64_t items = (int64_t)plan.geo.n_groups * p.ns;
+    const double row = (double)dim * p.f.W * elem_bytes(kind) * p.ns;
     const int64_t per_step = std::min<int64_t>(items, kMaxMomentCtas) * sizeof(double2);
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(steps_per_launch(row), (int64_t)part_bytes / per_step));
     for (int st = 0; st < half; st += chunk) {
@@ -1111,7 +1136,7 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
       run.st1 = std::min(half, st + chunk);
       run.bar_base = plan.bar_base;
       const int n = run.st1 - run.st0;
-      const int grid = launch_rows(run, kind, f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
+      const int grid = launch_rows(run, kind, p.f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
       if (grid < 0) return grid;
       plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
       count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
@@ -1128,26 +1153,25 @@ int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
   PF_CHECK(carve_scratch(scr, f));
   PF_CHECK(check_operator(plan, kind));
-  const SliceBufs b(scr, f);
   const int64_t dim = plan.geo.dim;
-  StepRun run{};
-  // one step of order K = 1 with c_0 = 0: out = H~ in, no barrier
-  run.one = make_job(plan, kind, f.lpr, 1.0);
-  run.one.xs = run.one.ba = b.xs;
-  run.one.bb = b.bb;
-  run.one.K = 1;
-  run.st1 = 1;
-  run.stride = (int64_t)f.slice;
-  run.err = plan.err_flag;
-  for (int s0 = 0; s0 < f.nsl; s0 += f.ns) {
-    const int ns = std::min(f.ns, f.nsl - s0), col0 = s0 * f.W, ncols = std::min(ns * f.W, n_b - col0);
-    PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, col0, ncols, f, ns, b.xs, nullptr, 0.0, nullptr, s));
-    run.n_jobs = ns;
-    const int grid = launch_rows(run, kind, f.lpr, plan.geo.rec_stride == 32, kFilter, plan.geo.max_group,
-                                 (int64_t)plan.geo.n_groups * ns, false, s);
+  for (const SlicePart& p : slice_parts(plan.geo, kind, f, n_b)) {
+    const SliceBufs b(scr, p.f);
+    PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.xs, nullptr, 0.0, nullptr, s));
+    StepRun run{};
+    // one step of order K = 1 with c_0 = 0: out = H~ in, no barrier
+    run.one = make_job(plan, kind, p.f.lpr, 1.0);
+    run.one.xs = run.one.ba = b.xs;
+    run.one.bb = b.bb;
+    run.one.K = 1;
+    run.st1 = 1;
+    run.stride = (int64_t)p.f.slice;
+    run.err = plan.err_flag;
+    run.n_jobs = p.ns;
+    const int grid = launch_rows(run, kind, p.f.lpr, plan.geo.rec_stride == 32, kFilter, plan.geo.max_group,
+                                 (int64_t)plan.geo.n_groups * p.ns, false, s);
     if (grid < 0) return grid;
-    count_step(kind, (double)dim * f.W * elem_bytes(kind) * ns * 3.0);
-    PF_CHECK(slice_out(kind, abi_kind, b.bb, dim, f, ns, ncols, out, n_b, col0, nullptr, s));
+    count_step(kind, (double)dim * p.f.W * elem_bytes(kind) * p.ns * 3.0);
+    PF_CHECK(slice_out(kind, abi_kind, b.bb, dim, p.f, p.ns, p.ncols, out, n_b, p.col0, nullptr, s));
   }
   return POLFED_OK;
 }

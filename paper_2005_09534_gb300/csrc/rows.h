@@ -391,11 +391,12 @@ struct StepJob {
   const void* Fhi;      // of the high part (schedule order, includes -alpha*beta)
   const void* Cx;       // of the cross bonds, by pattern
   const void* cx;       // typed cX in step order (a job of StepRun::jobs)
-  const float* colcx;   // FP32: per-column cX, row n = order n (W floats each), or null
+  const float* colcx;   // FP32: per-column cX, row n = order n (colw floats each), or null
   char *xs, *ba, *bb;   // x, b_{k+1}, b_{k+2} (overwritten by b_k)
   char *ta, *tb;        // moments in float-float: t_n (even n, odd n) in FP64
   double con[kConN];    // typed constants (each in its own 8 bytes)
   int K, n_groups, n_cross, c2mask;
+  int colw;
   int low_first;        // FP32 moments: low bonds before high ones
 };
 
@@ -856,7 +857,7 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
         I->x = (st & 1) ? J->tb + so : J->ta + so;
         I->t = (st & 1) ? J->ta + so : J->tb + so;
       } else if constexpr (MODE == kFilterCols) {
-        I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * (4 * LPR));
+        I->col = reinterpret_cast<const char*>(J->colcx + (R.jobs ? 0 : j * R.colstride) + (size_t)kk * J->colw);
       } else {
         cx = R.jobs ? __ldg(reinterpret_cast<const C*>(J->cx) + st) : *reinterpret_cast<const C*>(&R.cx[st - R.st0]);
       }
