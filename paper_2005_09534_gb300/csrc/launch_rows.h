@@ -43,7 +43,8 @@ int launch_rows_t(const StepRun& run, int max_group, int64_t items, bool coopera
   }
   const int nsm = cache.d[dev].nsm;
   int tile = ((max_group + 1) * 16 * LPR + 15) & ~15;
-  const int per_team = tile + 2 * (int)sizeof(WorkItem<NT>);
+  const int rowd = std::is_same<NT, RF64>::value ? (tile / (16 * LPR)) * (int)sizeof(double) : 0;
+  const int per_team = tile + 2 * (int)sizeof(WorkItem<NT>) + rowd;
   int teams = std::min(max_teams, cache.d[dev].maxdyn / per_team);
   if (teams < 1) return fail(POLFED_EINVAL, "slice tile does not fit in shared memory");
   // one CTA per SM; as many teams as there are work items for them

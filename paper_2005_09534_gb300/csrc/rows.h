@@ -226,7 +226,7 @@ struct RF64 {
   template <bool J2>
   static __device__ __forceinline__ int4 fin(Acc<J2>& a, const Coef& k, double d, const int4& own, const int4& x,
                                              const int4& b, bool hx, bool hb, bool, const float4&) {
-    fma<J2>(a, k.cH * d, own);
+    fma<J2>(a, d, own);  // d: cH times the diagonal
     if (hx) fma<J2>(a, k.cX, x);
     if (hb) fma<J2>(a, k.cB, b);
     return make_int4(__double2loint(a.p), __double2hiint(a.p), __double2loint(a.q), __double2hiint(a.q));
@@ -481,11 +481,13 @@ struct GroupStep {
   static constexpr int RS = J2 ? 32 : 16;          // uint16 entries of a record
   static constexpr int RSB = 2 * RS;
   static constexpr int STEP = kTeam * 16;          // bytes between a thread's consecutive rows
+  // FP64: the diagonal of a row is formed once, not by each of its lanes (see run)
+  static constexpr bool ROWD = std::is_same<NT, RF64>::value;
   static constexpr bool T64 = MODE == kMoments && std::is_same<NT, RDF>::value;  // t_n kept in FP64 beside its split
 
   template <int R>
   static __device__ __forceinline__ void pass(const Item* I, int blk, int n_g, const unsigned char* tile, bool& ready,
-                                              int team, double2& dot) {
+                                              int team, double2& dot, const C* dsm) {
     // high neighbours in flight per row (FP32, L = 24, J1-J2: 37.8 ms with two, 37.3 with four; float-float with
     // two rows is faster with two, 7.3 and 7.6 ms; FP64 at L = 14, single rows: 1200 us with four, 1165 with six)
     constexpr int HU = std::is_same<NT, RF32>::value ? 4 : (R == 1 ? (std::is_same<NT, RF64>::value ? 6 : 4) : 2);
@@ -594,10 +596,10 @@ struct GroupStep {
     }
     // low bonds: rows of the staged group; lists are padded with the zero row at tile offset 0
     const unsigned char* tl = tile + lane16;
-    auto low = [&](Acc& a, bool c1, uint32_t e0, uint32_t e1) {
+    auto low = [&](Acc& a, bool c1, uint32_t e0, uint32_t e1, bool second) {
       const int4 u0 = *reinterpret_cast<const int4*>(tl + e0), u1 = *reinterpret_cast<const int4*>(tl + e1);
       add(a, c1, u0);
-      add(a, c1, u1);
+      if (!ROWD || second) add(a, c1, u1);  // FP64: not even a padded entry is free
     };
 #pragma unroll
     for (int i = 0; i < R; i++) {
@@ -607,25 +609,25 @@ struct GroupStep {
       if constexpr (J2) {
         const int n2 = __reduce_max_sync(~0u, cnt >> 8);
         const uint4 q1 = ld_tab(rp + 16), q2 = ld_tab(rp + 32);
-        if (n1 > 0) low(acc[i], true, half(q1, 0), half(q1, 1));
-        if (n1 > 2) low(acc[i], true, half(q1, 2), half(q1, 3));
-        if (n1 > 4) low(acc[i], true, half(q1, 4), half(q1, 5));
-        if (n1 > 6) low(acc[i], true, half(q1, 6), half(q1, 7));
-        if (n1 > 8) low(acc[i], true, half(q2, 0), half(q2, 1));
+        if (n1 > 0) low(acc[i], true, half(q1, 0), half(q1, 1), n1 > 1);
+        if (n1 > 2) low(acc[i], true, half(q1, 2), half(q1, 3), n1 > 3);
+        if (n1 > 4) low(acc[i], true, half(q1, 4), half(q1, 5), n1 > 5);
+        if (n1 > 6) low(acc[i], true, half(q1, 6), half(q1, 7), n1 > 7);
+        if (n1 > 8) low(acc[i], true, half(q2, 0), half(q2, 1), n1 > 9);
         const uint4 q3 = ld_tab(rp + 48);
-        if (n2 > 0) low(acc[i], false, half(q2, 2), half(q2, 3));
-        if (n2 > 2) low(acc[i], false, half(q2, 4), half(q2, 5));
-        if (n2 > 4) low(acc[i], false, half(q2, 6), half(q2, 7));
-        if (n2 > 6) low(acc[i], false, half(q3, 0), half(q3, 1));
-        if (n2 > 8) low(acc[i], false, half(q3, 2), half(q3, 3));
+        if (n2 > 0) low(acc[i], false, half(q2, 2), half(q2, 3), n2 > 1);
+        if (n2 > 2) low(acc[i], false, half(q2, 4), half(q2, 5), n2 > 3);
+        if (n2 > 4) low(acc[i], false, half(q2, 6), half(q2, 7), n2 > 5);
+        if (n2 > 6) low(acc[i], false, half(q3, 0), half(q3, 1), n2 > 7);
+        if (n2 > 8) low(acc[i], false, half(q3, 2), half(q3, 3), n2 > 9);
       } else {
-        if (n1 > 0) low(acc[i], true, half(hd[i], 4), half(hd[i], 5));
-        if (n1 > 2) low(acc[i], true, half(hd[i], 6), half(hd[i], 7));
+        if (n1 > 0) low(acc[i], true, half(hd[i], 4), half(hd[i], 5), n1 > 1);
+        if (n1 > 2) low(acc[i], true, half(hd[i], 6), half(hd[i], 7), n1 > 3);
         if (n1 > 4) {
           const uint4 q1 = ld_tab(rp + 16);
-          low(acc[i], true, half(q1, 0), half(q1, 1));
-          if (n1 > 6) low(acc[i], true, half(q1, 2), half(q1, 3));
-          if (n1 > 8) low(acc[i], true, half(q1, 4), half(q1, 5));
+          low(acc[i], true, half(q1, 0), half(q1, 1), n1 > 5);
+          if (n1 > 6) low(acc[i], true, half(q1, 2), half(q1, 3), n1 > 7);
+          if (n1 > 8) low(acc[i], true, half(q1, 4), half(q1, 5), n1 > 9);
         }
       }
     }
@@ -639,7 +641,11 @@ struct GroupStep {
       const Coef kf = NT::load_fin(&I->k);
 #pragma unroll
       for (int i = 0; i < R; i++) {
-        const C d = NT::add3(__ldg(fc + i * (kTeam / LPR)), fhi, __ldg(cxt + pat[i]));
+        C d;
+        if constexpr (ROWD)
+          d = dsm[row + i * (kTeam / LPR)];
+        else
+          d = NT::add3(__ldg(fc + i * (kTeam / LPR)), fhi, __ldg(cxt + pat[i]));
         const int4 own = *reinterpret_cast<const int4*>(tile + ROWB + ro + i * STEP);
         int4 r;
         if constexpr (T64) {
@@ -722,13 +728,25 @@ struct GroupStep {
   // entry of the e-th low neighbour in a record
   static __device__ __forceinline__ int low_entry(int e, bool c1) { return J2 ? (c1 ? 8 : 18) + e : 4 + e; }
 
-  static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w, double2& dot) {
+  static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w, double2& dot, C* dsm) {
     const int n_g = lds32(&I->g.n_g);
     {
       const char* src = (const char*)lds64(&I->b1) + (size_t)(uint32_t)lds32(&I->g.r0) * ROWB;
       const int nb = n_g * ROWB;
       for (int c = (threadIdx.x % kTeam) * 16; c < nb; c += STEP) cp_async16(tile + ROWB + c, src + c);
       cp_async_commit();
+    }
+    if constexpr (ROWD) {
+      // cH d of the group's rows: 3 FP64 instructions a row instead of 3 for each of its 16-byte chunks, the
+      // FP64 pipe being 89% busy (L = 20, 64 columns, K = 40: 16.4 ms, with this and no padded entries 14.6)
+      const int cls = lds32(&I->g.cls_base), n_cross = lds32(&I->n_cross);
+      const uint32_t need = (uint32_t)lds32(&I->g.need_mask);
+      const C cH = NT::load_fin(&I->k).cH;
+      for (int r = threadIdx.x % kTeam; r < n_g; r += kTeam) {
+        const uint32_t own = __ldg((const uint16_t*)lds64(&I->rec) + (size_t)(cls + r) * RS);
+        const uint32_t pat = ~(own ^ need) & ((1u << n_cross) - 1u);
+        dsm[r] = cH * NT::add3(__ldg((const C*)lds64(&I->fc) + cls + r), I->fhi, __ldg((const C*)lds64(&I->cxt) + pat));
+      }
     }
     bool ready = false;
     const int nblk = (n_g + RPW - 1) / RPW, nfull = n_g / RPW;
@@ -737,8 +755,8 @@ struct GroupStep {
       for (; blk < nblk; blk += NW) pass_in_order(I, blk, n_g, tile, ready, team, dot);
     } else {
       if constexpr (RMAX >= 2)
-        for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team, dot);
-      for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team, dot);
+        for (; blk + NW < nfull; blk += 2 * NW) pass<2>(I, blk, n_g, tile, ready, team, dot, dsm);
+      for (; blk < nblk; blk += NW) pass<1>(I, blk, n_g, tile, ready, team, dot, dsm);
     }
     if (!ready) {
       cp_async_wait();
@@ -814,6 +832,9 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
   const int team = threadIdx.x / kTeam, tt = threadIdx.x % kTeam;
   unsigned char* tile = smem + (size_t)team * tile_bytes;
   Item* items = reinterpret_cast<Item*>(smem + (size_t)(blockDim.x / kTeam) * tile_bytes) + 2 * team;
+  // FP64: cH d of the group's rows, behind the items
+  C* dsm = reinterpret_cast<C*>(smem + (size_t)(blockDim.x / kTeam) * (tile_bytes + 2 * sizeof(Item))) +
+           (size_t)team * (tile_bytes / (16 * LPR));
   const int n_teams = (blockDim.x / kTeam) * gridDim.x;
   const int me = team * gridDim.x + blockIdx.x;  // neighbouring items go to different SMs
   if (tt < LPR) *reinterpret_cast<int4*>(tile + tt * 16) = make_int4(0, 0, 0, 0);  // the zero row
@@ -879,7 +900,7 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       const Item* I = items + (r & 1);
       r++;
       more = fetch();
-      GroupStep<NT, LPR, J2, MODE, RMAX>::run(I, tile, team, tt >> 5, dot);
+      GroupStep<NT, LPR, J2, MODE, RMAX>::run(I, tile, team, tt >> 5, dot, dsm);
     }
     if constexpr (MODE == kMoments) {
       __shared__ double2 wsum[kTeam * kMaxTeams / 32];
