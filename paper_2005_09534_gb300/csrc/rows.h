@@ -397,14 +397,16 @@ struct StepJob {
   double con[kConN];    // typed constants (each in its own 8 bytes)
   int K, n_groups, n_cross, c2mask;
   int colw;
+  int rowmul;           // direct: bytes between rows / bytes of a slice's row
   int low_first;        // FP32 moments: low bonds before high ones
 };
 
 constexpr int kParamSteps = 448;  // step coefficients that travel in the kernel parameters
 
 // What a step computes: the filter's recurrence, with a scalar or a per-column
-// c_n, or t_{n+1} = 2 H~ t_n - t_{n-1} with the sums t_n . t_n and t_{n+1} . t_n.
-enum StepMode { kFilter, kFilterCols, kMoments };
+// c_n, or t_{n+1} = 2 H~ t_n - t_{n-1} with the sums t_n . t_n and t_{n+1} . t_n,
+// or one H~ product on the columns of a row-major block (rows `rowmul` slice rows apart).
+enum StepMode { kFilter, kFilterCols, kMoments, kDirect };
 
 struct StepRun {
   StepJob one;            // jobs == nullptr: n_jobs slices of this operator, buffers `stride` bytes apart
@@ -463,7 +465,7 @@ struct alignas(16) WorkItem {
   char* t;                                    // moments in float-float: t_{n-1} in FP64 (x: t_n)
   char* out;                                  // and b2
   typename NT::Coef k;
-  int n_cross, c2mask, flags;                 // flags: 1 = reads x, 2 = reads b2, 4 = low bonds first
+  int n_cross, c2mask, rowmul, flags;         // flags: 1 = reads x, 2 = reads b2, 4 = low bonds first
 };
 
 // One step of one group (the rows sharing s_hi) by a team:
@@ -498,8 +500,11 @@ struct GroupStep {
       live = row < n_g;
       row = min(row, n_g - 1);
     }
-    const uint32_t ro = (uint32_t)(row * ROWB + lane16);
-    const size_t goff = (size_t)(uint32_t)lds32(&I->g.r0) * ROWB + ro;
+    const uint32_t ro = (uint32_t)(row * ROWB + lane16);  // in the tile
+    const uint32_t mul = MODE == kDirect ? (uint32_t)lds32(&I->rowmul) : 1u;
+    const uint32_t pitch = ROWB * mul, gro = MODE == kDirect ? (uint32_t)(row * pitch + lane16) : ro;
+    const uint32_t step = STEP * mul;
+    const size_t goff = (size_t)(uint32_t)lds32(&I->g.r0) * pitch + gro;
     const int flags = lds32(&I->flags);
     const bool hx = flags & 1, hb = flags & 2;
     const typename NT::Sum k = NT::load_sum(&I->k);
@@ -516,16 +521,16 @@ struct GroupStep {
         NT::template add2<J2>(a, k, u);
     };
     {
-      const char* hp = b1 + ro;
+      const char* hp = b1 + gro;
       auto high = [&](int k0, int k1, bool c1) {
         int kk = k0;
         for (; kk + HU <= k1; kk += HU) {
           int4 u[HU][R];
 #pragma unroll
           for (int j = 0; j < HU; j++) {
-            const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk + j]) * ROWB;
+            const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk + j]) * pitch;
 #pragma unroll
-            for (int i = 0; i < R; i++) u[j][i] = ld_l2(p + i * STEP);
+            for (int i = 0; i < R; i++) u[j][i] = ld_l2(p + i * step);
           }
 #pragma unroll
           for (int j = 0; j < HU; j++)
@@ -534,9 +539,9 @@ struct GroupStep {
         }
         for (; kk < k1; kk++) {
           int4 u[R];
-          const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk]) * ROWB;
+          const char* p = hp + (size_t)(uint32_t)lds32(&I->g.hn_base[kk]) * pitch;
 #pragma unroll
-          for (int i = 0; i < R; i++) u[i] = ld_l2(p + i * STEP);
+          for (int i = 0; i < R; i++) u[i] = ld_l2(p + i * step);
 #pragma unroll
           for (int i = 0; i < R; i++) add(acc[i], c1, u[i]);
         }
@@ -578,12 +583,12 @@ struct GroupStep {
 #pragma unroll
     for (int c = 0; c < MAXCR; c++) {
       if (c < n_cross) {
-        const char* p = b1 + lane16 + (size_t)(uint32_t)lds32(&I->g.cr_base[c]) * ROWB - ROWB;
+        const char* p = b1 + lane16 + (size_t)(uint32_t)lds32(&I->g.cr_base[c]) * pitch - pitch;
         const bool c1 = !J2 || !((lds32(&I->c2mask) >> c) & 1);
         int4 u[R];
 #pragma unroll
         for (int i = 0; i < R; i++)
-          if ((pat[i] >> c) & 1) u[i] = ld_l2(p + half(hd[i], 2 + c));
+          if ((pat[i] >> c) & 1) u[i] = ld_l2(p + half(hd[i], 2 + c) * mul);
 #pragma unroll
         for (int i = 0; i < R; i++)
           if ((pat[i] >> c) & 1) add(acc[i], c1, u[i]);
@@ -657,7 +662,7 @@ struct GroupStep {
           if constexpr (MODE == kMoments)
             if (R > 1 || live) NT::dots(own, r, dot);
         }
-        if (R > 1 || live) __stcg(reinterpret_cast<int4*>(out + i * STEP), r);
+        if (R > 1 || live) __stcg(reinterpret_cast<int4*>(out + i * step), r);
       }
     }
   }
@@ -731,9 +736,11 @@ struct GroupStep {
   static __device__ __forceinline__ void run(const Item* I, unsigned char* tile, int team, int w, double2& dot, C* dsm) {
     const int n_g = lds32(&I->g.n_g);
     {
-      const char* src = (const char*)lds64(&I->b1) + (size_t)(uint32_t)lds32(&I->g.r0) * ROWB;
+      const uint32_t mul = MODE == kDirect ? (uint32_t)lds32(&I->rowmul) : 1u;
+      const char* src = (const char*)lds64(&I->b1) + (size_t)(uint32_t)lds32(&I->g.r0) * (ROWB * mul);
       const int nb = n_g * ROWB;
-      for (int c = (threadIdx.x % kTeam) * 16; c < nb; c += STEP) cp_async16(tile + ROWB + c, src + c);
+      for (int c = (threadIdx.x % kTeam) * 16; c < nb; c += STEP)
+        cp_async16(tile + ROWB + c, src + (MODE == kDirect ? c / ROWB * (ROWB * mul) + c % ROWB : c));
       cp_async_commit();
     }
     if constexpr (ROWD) {
@@ -870,6 +877,7 @@ __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_
       I->cxt = reinterpret_cast<const char*>(J->Cx);
       I->n_cross = J->n_cross;
       I->c2mask = J->c2mask;
+      if constexpr (MODE == kDirect) I->rowmul = J->rowmul;
       const int kk = J->K - 1 - st;
       bool last = kk == 0, first = st == 0;
       C cx = C();

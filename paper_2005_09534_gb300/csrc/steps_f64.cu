@@ -7,6 +7,7 @@ int launch_rows_f64(const StepRun& run, int lpr, bool j2, StepMode mode, int max
                     int max_teams, cudaStream_t s) {
   switch (mode) {
     case kFilter: return launch_rows_mode<RF64, kFilter>(run, lpr, j2, max_group, items, cooperative, max_teams, s);
+    case kDirect: return launch_rows_mode<RF64, kDirect>(run, lpr, j2, max_group, items, cooperative, max_teams, s);
     case kMoments: return launch_rows_mode<RF64, kMoments>(run, lpr, j2, max_group, items, cooperative, max_teams, s);
     default: return fail(POLFED_EINVAL, "per-column coefficients need FP32 storage");
   }
