@@ -1,6 +1,7 @@
 // C ABI entry points: error reporting, basis, H~ application and the filter.
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -42,6 +43,66 @@ static int check_block_args(const polfed_model* model, const uint32_t* d_states,
 static int check_bounds(double e_lo, double e_hi) {
   if (!std::isfinite(e_lo) || !std::isfinite(e_hi)) return fail(POLFED_EINVAL, "non-finite e_lo/e_hi");
   if (!(e_lo == 0.0 && e_hi == 0.0) && !(e_lo < e_hi)) return fail(POLFED_EINVAL, "need e_lo < e_hi");
+  return POLFED_OK;
+}
+
+namespace {
+struct ScratchPools {
+  std::mutex mu;
+  cudaMemPool_t pool[64] = {};
+  bool tried[64] = {};
+};
+ScratchPools g_pools;
+
+// the current device's pool, or null
+cudaMemPool_t scratch_pool(bool create) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lk(g_pools.mu);
+  if (create && !g_pools.tried[dev]) {
+    g_pools.tried[dev] = true;
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    size_t free_b = 0, total = 0;
+    cudaMemPool_t q = nullptr;
+    if (cudaMemGetInfo(&free_b, &total) == cudaSuccess && cudaMemPoolCreate(&q, &props) == cudaSuccess) {
+      uint64_t keep = total / 64;
+      if (cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        g_pools.pool[dev] = q;
+      else
+        cudaMemPoolDestroy(q);
+    }
+    cudaGetLastError();
+  }
+  return g_pools.pool[dev];
+}
+}  // namespace
+
+void pool_trim() {
+  if (cudaMemPool_t q = scratch_pool(false))
+    if (cudaMemPoolTrimTo(q, 0) != cudaSuccess) cudaGetLastError();
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  pool_trim();
+  return cudaMalloc(p, bytes);
+}
+
+int scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  if (cudaMemPool_t q = scratch_pool(true)) {
+    if (cudaMallocFromPoolAsync(p, bytes, q, s) == cudaSuccess) return POLFED_OK;
+    cudaGetLastError();
+    pool_trim();
+    if (cudaMallocFromPoolAsync(p, bytes, q, s) == cudaSuccess) return POLFED_OK;
+    cudaGetLastError();
+  }
+  PF_CUDA(cudaMallocAsync(p, bytes, s));
   return POLFED_OK;
 }
 
@@ -118,10 +179,13 @@ int polfed_h_apply(const polfed_model* model, const uint32_t* d_states, int64_t 
   StreamScratch mem;
   mem.s = s;
   FilterScratch scr;
-  scr.bytes = filter_scratch_bytes(plan, dtype, n_b);
-  PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
-  scr.xs = mem.p;
-  PF_CHECK(apply_block(plan, dtype, d_X, d_Y, n_b, dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64, scr, s));
+  const int abi = dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64;
+  if (!apply_direct(dtype, abi, n_b, d_X, d_Y)) {
+    scr.bytes = filter_scratch_bytes(plan, dtype, n_b);
+    PF_CHECK(scratch_alloc(&mem.p, scr.bytes, s));
+    scr.xs = mem.p;
+  }
+  PF_CHECK(apply_block(plan, dtype, d_X, d_Y, n_b, abi, scr, s));
   PF_CUDA(cudaStreamSynchronize(s));
   return POLFED_OK;
 }
@@ -154,7 +218,7 @@ int polfed_cheb_filter(const polfed_model* model, const uint32_t* d_states, int6
   mem.s = s;
   FilterScratch scr;
   scr.bytes = filter_scratch_bytes(plan, dtype, n_b);
-  PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
+  PF_CHECK(scratch_alloc(&mem.p, scr.bytes, s));
   scr.xs = mem.p;
   PF_CHECK(filter_block(plan, dtype, c.data(), K, invD, d_X, d_Y, n_b, dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64,
                         scr, s));
@@ -195,9 +259,9 @@ int polfed_cheb_filter_cols(const polfed_model* model, const uint32_t* d_states,
   cmem.s = s;
   FilterScratch scr;
   scr.bytes = filter_scratch_bytes(plan, POLFED_F32, n_b);
-  PF_CUDA(cudaMallocAsync(&mem.p, scr.bytes, s));
+  PF_CHECK(scratch_alloc(&mem.p, scr.bytes, s));
   scr.xs = mem.p;
-  PF_CUDA(cudaMallocAsync(&cmem.p, cf.size() * sizeof(float), s));
+  PF_CHECK(scratch_alloc(&cmem.p, cf.size() * sizeof(float), s));
   PF_CUDA(cudaMemcpyAsync(cmem.p, cf.data(), cf.size() * sizeof(float), cudaMemcpyHostToDevice, s));
   PF_CHECK(filter_block_cols(plan, (const float*)cmem.p, K, d_X, d_Y, n_b, POLFED_F32, scr, s));
   float flag[3] = {0, 0, 0};

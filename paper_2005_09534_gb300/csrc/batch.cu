@@ -48,7 +48,7 @@ struct DeviceBuffer {
     if (p) cudaFree(p);
     p = nullptr;
     n = 0;
-    if (cudaMalloc(&p, need) != cudaSuccess) {
+    if (device_malloc(&p, need) != cudaSuccess) {
       cudaGetLastError();
       return fail(POLFED_ENOMEM, "batched runner: cudaMalloc of " + std::to_string(need) + " bytes failed");
     }
@@ -337,7 +337,7 @@ int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const
   const int abi = dtype == POLFED_F32 ? POLFED_F32 : POLFED_F64;
   void* scr = nullptr;
   const size_t bytes = batch_scratch_bytes(items, dtype);
-  PF_CUDA(cudaMallocAsync(&scr, bytes, s));
+  PF_CHECK(scratch_alloc(&scr, bytes, s));
   BatchStats bs;
   int rc = filter_batched(items, dtype, abi, scr, bytes, s, ctas_per_sm, &bs);
   cudaFreeAsync(scr, s);

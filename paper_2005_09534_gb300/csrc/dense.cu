@@ -703,7 +703,7 @@ int Dense::ensure(void*& p, size_t& have, size_t need) {
   if (p) cudaFree(p);
   p = nullptr;
   have = 0;
-  PF_CUDA(cudaMalloc(&p, need));
+  PF_CUDA(device_malloc(&p, need));
   have = need;
   return POLFED_OK;
 }

@@ -645,9 +645,9 @@ int HamPlan::init(const polfed_model* m, cudaStream_t s, bool stream_ordered, in
   stream_alloc = stream_ordered;
   const size_t bytes = PlanLayout(geo).total, all = bytes + (kind >= 0 ? typed_bytes_of(geo) : 0);
   if (stream_ordered)
-    PF_CUDA(cudaMallocAsync(&dev, all, s));
+    PF_CHECK(scratch_alloc(&dev, all, s));
   else
-    PF_CUDA(cudaMalloc(&dev, all));
+    PF_CUDA(device_malloc(&dev, all));
   dev_end = (char*)dev + all;
   return bind((char*)dev, s, kind, e_lo, e_hi, (char*)dev + bytes);
 }
@@ -657,9 +657,9 @@ int HamPlan::prepare_typed(int kind, double e_lo, double e_hi) {
   if (typed_ok[kind] && typed_lo[kind] == e_lo && typed_hi[kind] == e_hi) return POLFED_OK;
   if (!typed[kind]) {
     if (stream_alloc)
-      PF_CUDA(cudaMallocAsync(&typed[kind], typed_bytes_of(geo), stream));
+      PF_CHECK(scratch_alloc(&typed[kind], typed_bytes_of(geo), stream));
     else
-      PF_CUDA(cudaMalloc(&typed[kind], typed_bytes_of(geo)));
+      PF_CUDA(device_malloc(&typed[kind], typed_bytes_of(geo)));
   }
   typed_ok[kind] = false;
   TypedOut ty;
@@ -1148,15 +1148,20 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
   return check_timeout(plan, s);
 }
 
+// Rows that are whole slices of 16-byte chunks are gathered where they lie: 64
+// FP64 columns at L = 22 spent 345 of 1770 us on the copies into slices and out of
+// them; in one launch over the block they take 1340 (FP32: 350 and 247).
+bool apply_direct(int kind, int abi_kind, int n_b, const void* in, const void* out) {
+  const size_t pitch = (size_t)n_b * elem_bytes(kind);
+  return kind == abi_kind && kind != POLFED_DF64 && pitch % (16 * choose_lpr(kind, n_b)) == 0 && (uintptr_t)in % 16 == 0 &&
+         (uintptr_t)out % 16 == 0;
+}
+
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                 cudaStream_t s) {
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
-  // Rows that are whole slices of 16-byte chunks are gathered where they lie: 64
-  // FP64 columns at L = 22 spent 345 of 1770 us on the copies into slices and out of
-  // them; in one launch over the block they take 1340 (FP32: 350 and 247).
-  const size_t es = elem_bytes(kind), pitch = (size_t)n_b * es;
-  if (kind == abi_kind && kind != POLFED_DF64 && pitch % (16 * f.lpr) == 0 && (uintptr_t)in % 16 == 0 &&
-      (uintptr_t)out % 16 == 0) {
+  if (apply_direct(kind, abi_kind, n_b, in, out)) {
+    const size_t pitch = (size_t)n_b * elem_bytes(kind);
     PF_CHECK(check_operator(plan, kind));
     StepRun run{};
     run.one = make_job(plan, kind, f.lpr, 1.0);

@@ -96,7 +96,7 @@ int polfed_kpm_moments(const polfed_model* model, const uint32_t* d_states, int6
   PF_CHECK(plan.init(model, s, true, moments_b(dtype, model->L), dtype, e_lo, e_hi));
   const size_t fb = (filter_scratch_bytes(plan, dtype, R) + 255) & ~(size_t)255;
   void* mem = nullptr;
-  PF_CUDA(cudaMallocAsync(&mem, fb + kpm_buffer_bytes(plan, dtype, R), s));
+  PF_CHECK(scratch_alloc(&mem, fb + kpm_buffer_bytes(plan, dtype, R), s));
   FilterScratch scr;
   scr.xs = mem;
   scr.bytes = fb;

@@ -55,7 +55,7 @@ struct DevBuf {
     p = nullptr;
     n = 0;
     if (limit && total && *total + need > limit) return fail(POLFED_ENOMEM, "context workspace limit exceeded");
-    if (cudaMalloc(&p, need) != cudaSuccess) {
+    if (device_malloc(&p, need) != cudaSuccess) {
       cudaGetLastError();
       return fail(POLFED_ENOMEM, "cudaMalloc of " + std::to_string(need) + " bytes failed");
     }
@@ -947,6 +947,7 @@ void polfed_ctx_destroy(polfed_ctx* c) {
   c->kpm.release();
   c->coefbuf.release();
   c->dense.release();
+  pool_trim();
   if (c->solver) cusolverDnDestroy(c->solver);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;

@@ -463,7 +463,7 @@ int ensure_work(polfed_mlp* n, int B, Work* w) {
     if (n->work) cudaFree(n->work);
     n->work = nullptr;
     n->work_floats = 0;
-    if (cudaMalloc(&n->work, need * sizeof(float)) != cudaSuccess) {
+    if (device_malloc((void**)&n->work, need * sizeof(float)) != cudaSuccess) {
       cudaGetLastError();
       return fail(POLFED_ENOMEM, "MLP work allocation failed");
     }
@@ -612,10 +612,10 @@ int polfed_mlp_create(int32_t d_in, int32_t hidden, int32_t d_out, uint64_t seed
   cudaGetDevice(&n->device);
   const size_t bytes = (size_t)n->n_params * sizeof(float);
   const size_t sbytes = (size_t)(2 * d_in + 2 * d_out) * sizeof(float);
-  if (cudaMalloc(&n->params, bytes) != cudaSuccess || cudaMalloc(&n->m, bytes) != cudaSuccess ||
-      cudaMalloc(&n->v, bytes) != cudaSuccess || cudaMalloc(&n->grad, bytes) != cudaSuccess ||
-      cudaMalloc(&n->scale, sbytes) != cudaSuccess ||
-      cudaMalloc(&n->io, (size_t)(d_in + d_out) * sizeof(float)) != cudaSuccess) {
+  if (device_malloc((void**)&n->params, bytes) != cudaSuccess || device_malloc((void**)&n->m, bytes) != cudaSuccess ||
+      device_malloc((void**)&n->v, bytes) != cudaSuccess || device_malloc((void**)&n->grad, bytes) != cudaSuccess ||
+      device_malloc((void**)&n->scale, sbytes) != cudaSuccess ||
+      device_malloc((void**)&n->io, (size_t)(d_in + d_out) * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();
     polfed_mlp_destroy(n);
     return fail(POLFED_ENOMEM, "MLP allocation failed");

@@ -450,7 +450,7 @@ int entropy_small(int L, const uint32_t* d_states, const double* d_vecs, int64_t
   const size_t bM = up((size_t)nvb * h * dim * 8), bT = up((size_t)nvb * h * tri_doubles(h) * 8), bS = up((size_t)n_vec * h * 8);
   StreamMem mem;
   mem.s = s;
-  if (cudaMallocAsync(&mem.p, bM + bT + bS + 256, s) != cudaSuccess) {
+  if (scratch_alloc(&mem.p, bM + bT + bS + 256, s) != POLFED_OK) {
     cudaGetLastError();
     return fail(POLFED_ENOMEM, "device workspace for the Schmidt blocks");
   }
@@ -510,7 +510,7 @@ int polfed_gap_ratio(const double* d_evals, int32_t n, double* r_mean, double* d
   cudaStream_t s = (cudaStream_t)stream;
   StreamMem mem;
   mem.s = s;
-  PF_CUDA(cudaMallocAsync(&mem.p, 64, s));
+  PF_CHECK(scratch_alloc(&mem.p, 64, s));
   double* sum = (double*)mem.p;
   int* flag = (int*)((char*)mem.p + 32);
   PF_CUDA(cudaMemsetAsync(mem.p, 0, 64, s));
@@ -622,7 +622,7 @@ int polfed_entanglement_entropy(polfed_ctx* ctx, int32_t L, const uint32_t* d_st
   const size_t bInfo = up((size_t)2 * nv_max * 4), bS = up((size_t)n_vec * h * 8), bWs = up(ws_dev + 16);
   StreamMem mem;
   mem.s = s;
-  if (cudaMallocAsync(&mem.p, bM + bG + bW + bOff + bJobs + bSz + bInfo + bS + bWs, s) != cudaSuccess) {
+  if (scratch_alloc(&mem.p, bM + bG + bW + bOff + bJobs + bSz + bInfo + bS + bWs, s) != POLFED_OK) {
     cudaGetLastError();
     return fail(POLFED_ENOMEM, "device workspace for the Schmidt blocks");
   }

@@ -60,6 +60,15 @@ inline void count_step(int kind, double alg_bytes) {
   c.all_alg_bytes[kind] += alg_bytes;
 }
 
+// Stream-ordered scratch of a call (freed with cudaFreeAsync), from a pool of the
+// library's own: the default pool unmaps freed memory at the next synchronization,
+// and mapping it again costs 70 us for a few MB, 2 ms for a GB.  The pool keeps at
+// most 1/64 of the device's memory between calls; pool_trim gives back what is
+// unused, as polfed_ctx_destroy and every allocation that fails do.
+int scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+void pool_trim();
+cudaError_t device_malloc(void** p, size_t bytes);  // cudaMalloc, once more after pool_trim
+
 // -------------------------------------------------------------- binomials
 // C(n, k) for 0 <= n, k <= 32 (C(32,16) < 2^31).
 uint32_t binom_host(int n, int k);
@@ -173,6 +182,8 @@ int filter_block(HamPlan& plan, int kind, const double* coeffs, int K, double in
 // d_coef[(q (K + 1) + n) W + j - q W] = coefficient of column j at order n.  in/out as filter_block.
 int filter_block_cols(HamPlan& plan, const float* d_coef, int K, const void* in, void* out, int n_b, int abi_kind,
                       FilterScratch& scr, cudaStream_t s);
+// H~ of a block: needs no scratch where apply_direct holds
+bool apply_direct(int kind, int abi_kind, int n_b, const void* in, const void* out);
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                 cudaStream_t s);
 // mu[2k] = t_k . t_k, mu[2k + 1] = t_{k+1} . t_k summed over n_b columns, t_{k+1} = 2 H~ t_k - t_{k-1}, k < half
