@@ -226,12 +226,12 @@ struct TypedOut {
 
 // All tables of a plan in one launch: thread i < n_main does low state i (rank,
 // diagonal), high state i (rank, diagonal, its group's place in the schedule and
-// its record) and cross pattern i; the threads after them one entry of a
-// neighbour record each.  A state's neighbours are ranked again instead of being
+// the head of its record) and cross pattern i; the threads after them one entry
+// of a neighbour record or one neighbour of a group each.  A state's neighbours are ranked again instead of being
 // read from another launch's table, with the binomials in shared memory (as
 // divergent reads of constant memory they are serialized).  Bound by launches and
 // latency: the four kernels this replaces took 21 us and three more launches at
-// L = 22, this one 17; an L = 12 call with one column took 52 us, now 42.
+// L = 22, this one 10; an L = 12 call with one column took 52 us, now 40.
 constexpr int kTableThreads = 128;
 __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, const ClassStart cs, HamTables t, int* err,
                                                           TypedOut ty, int n_main) {
@@ -244,9 +244,47 @@ __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, c
     for (int k = 1; a; a &= a - 1, k++) r += B[__ffs(a) - 1][k];
     return r;
   };
-  const int RS = g.rec_stride, j = i - n_main;
+  // first row of a group: its bits sit above n_lo low ones
+  auto rank_hi = [&](uint32_t a) {
+    uint32_t r = 0;
+    for (int k = g.n_up - __popc(a) + 1; a; a &= a - 1, k++) r += B[g.b + __ffs(a) - 1][k];
+    return (int)r;
+  };
+  auto valid = [&](uint32_t a) {
+    const int n = g.n_up - __popc(a);
+    return n >= 0 && n <= g.b;
+  };
+  const int RS = g.rec_stride;
+  int j = i - n_main;
+  if (j >= RS << g.b) {  // one neighbour of a group: kMaxHigh high ones, then 8 cross bonds
+    j -= RS << g.b;
+    const int e = j % (kMaxHigh + 8);
+    const uint32_t grp = (uint32_t)(j / (kMaxHigh + 8));
+    if (grp >> g.nh || !valid(grp)) return;
+    GroupRec* r = t.grec + cs.v[__popc(grp)] + (int)rank_lo(grp);
+    if (e < kMaxHigh) {
+      uint32_t m = 0;
+      int cnt = 0;
+      for (int q = 0; q < g.n_high1 + g.n_high2 && !m; q++)
+        if (__popc(grp & g.high_mask[q]) == 1 && cnt++ == e) m = g.high_mask[q];
+      r->hn_base[e] = m ? rank_hi(grp ^ m) : 0;
+    } else {
+      const int k = e - kMaxHigh;
+      int base = 0, n = 0;
+      if (k < g.n_cross) {
+        const uint32_t g2 = grp ^ (1u << g.cross_hi[k]);
+        // rows with the bond antiparallel exist only if the neighbouring class is valid
+        if (valid(g2)) {
+          base = rank_hi(g2);
+          n = (int)B[g.b][g.n_up - __popc(g2)];
+        }
+      }
+      r->cr_base[k] = base;
+      r->cr_n[k] = n;
+    }
+    return;
+  }
   if (j >= 0) {  // neighbour records (layout in HamTables::rec): one entry, for every row size
-    if (j >= RS << g.b) return;
     const uint32_t a = (uint32_t)(j / RS);
     const int e = j % RS, l1 = RS == 32 ? 8 : 4;  // l1: first low entry, after the cross neighbours
     auto active = [&](int q0, int n, int want, int* cnt) {  // the want-th active low bond of a class
@@ -294,16 +332,6 @@ __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, c
   if (i < (1 << g.nh)) {
     const uint32_t grp = (uint32_t)i;
     const int pc = __popc(grp), n_lo = g.n_up - pc;
-    // first row of the group: its bits sit above n_lo low ones
-    auto rank_hi = [&](uint32_t a) {
-      uint32_t r = 0;
-      for (int k = g.n_up - __popc(a) + 1; a; a &= a - 1, k++) r += B[g.b + __ffs(a) - 1][k];
-      return (int)r;
-    };
-    auto valid = [&](uint32_t a) {
-      const int n = g.n_up - __popc(a);
-      return n >= 0 && n <= g.b;
-    };
     int T = -1;
     double d = 0.0;
     if (valid(grp)) {
@@ -320,31 +348,16 @@ __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, c
       r->r0 = T;
       r->n_g = (int)B[g.b][n_lo];
       r->cls_base = g.cls_off[n_lo];
-      int cnt = 0, cnt1 = 0;
-      for (int k = 0; k < nhb; k++) {
-        const uint32_t m = g.high_mask[k];
-        if (__popc(grp & m) != 1) continue;
-        r->hn_base[cnt++] = rank_hi(grp ^ m);
-        if (k < g.n_high1) cnt1++;
-      }
-      for (int k = cnt; k < kMaxHigh; k++) r->hn_base[k] = 0;
+      int cnt = 0, cnt1 = 0, need = 0;
+      for (int k = 0; k < nhb; k++)
+        if (__popc(grp & g.high_mask[k]) == 1) {
+          cnt++;
+          if (k < g.n_high1) cnt1++;
+        }
       r->n_hn = cnt;
       r->n_hn1 = cnt1;
-      int need = 0;
-      for (int k = 0; k < 8; k++) {
-        int base = 0, n = 0;
-        if (k < g.n_cross) {
-          if (!((grp >> g.cross_hi[k]) & 1)) need |= 1 << k;  // the low bit must differ from the high bit
-          const uint32_t g2 = grp ^ (1u << g.cross_hi[k]);
-          // rows with the bond antiparallel exist only if the neighbouring class is valid
-          if (valid(g2)) {
-            base = rank_hi(g2);
-            n = (int)B[g.b][g.n_up - __popc(g2)];
-          }
-        }
-        r->cr_base[k] = base;
-        r->cr_n[k] = n;
-      }
+      for (int k = 0; k < g.n_cross; k++)
+        if (!((grp >> g.cross_hi[k]) & 1)) need |= 1 << k;  // the low bit must differ from the high bit
       r->need_mask = need;
       r->pad0 = r->pad1 = 0;
       if (ty.kind >= 0) ty.put((1 << g.b) + pos, ty.alpha * (d - ty.beta));
@@ -626,7 +639,7 @@ int HamPlan::bind(char* base, cudaStream_t s, int kind, double e_lo, double e_hi
     typed_hi[kind] = e_hi;
   }
   const int n_main = (std::max({64, 1 << geo.b, 1 << geo.nh, 1 << geo.n_cross}) + kTableThreads - 1) / kTableThreads;
-  const int n_rec = ((geo.rec_stride << geo.b) + kTableThreads - 1) / kTableThreads;
+  const int n_rec = ((geo.rec_stride << geo.b) + ((kMaxHigh + 8) << geo.nh) + kTableThreads - 1) / kTableThreads;
   k_tables<<<n_main + n_rec, kTableThreads, 0, s>>>(geo, class_starts(geo), tab, err_flag, ty, n_main * kTableThreads);
   PF_CUDA(cudaGetLastError());
   return POLFED_OK;
