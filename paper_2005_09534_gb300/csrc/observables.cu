@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "polfed_internal.h"
+#include "rows.h"
 
 namespace polfed {
 
@@ -195,8 +196,9 @@ __global__ void k_gap_ratio(const double* __restrict__ e, int n, double* r_out, 
 // GB300 runs 2 FP64 FMAs per SM and clock, so the FP64 pipe bounds all of this:
 // the work per block is kept to n^3/2 (Gram) + 2 n^3/3 (reduction) FMAs, the
 // square root and the division of a step are taken by one thread only, and
-// eigenvalues come from Sturm counts without divisions (k_schmidt_values).
-// Measured: 50 vectors at L = 14 (2800 blocks of 1 to 35 rows) 28.6 -> 1.1 ms
+// eigenvalues come from Sturm counts without divisions, most of them in float-float
+// (k_schmidt_values).
+// Measured: 50 vectors at L = 14 (2800 blocks of 1 to 35 rows) 28.6 -> 0.85 ms
 // against the batched library solver, whose 42 solves took 900 launches and a
 // synchronization each.  Blocks beyond kTriMax rows do not fit shared memory
 // and stay with the library.
@@ -371,20 +373,54 @@ __device__ __forceinline__ int sturm(const double* __restrict__ d, const double*
   return cnt;
 }
 
+// The same count in float-float arithmetic (2^-46) on the FP32 pipe, for a first
+// bracket; d and e2 as (hi, lo).  A minor below 2^-60 of its predecessor counts as
+// -2^-60 of it.
+__device__ __forceinline__ int sturm_ff(const float2* d, const float2* e2, int n, double x) {
+  constexpr int kTiny = 127 - 60;
+  const float xh = (float)x;
+  const float2 mx = make_float2(-xh, -(float)(x - (double)xh));
+  int cnt = 0;
+  float2 p = make_float2(1.f, 0.f), pm = make_float2(0.f, 0.f), e = pm;
+  for (int i = 0; i < n; i++) {
+    const float2 w = df_mul(e, pm), nx = df_add(df_mul(df_add(d[i], mx), p), make_float2(-w.x, -w.y));
+    e = e2[i];
+    const int hi = __float_as_int(nx.x), ho = __float_as_int(p.x);
+    int ex = (hi >> 23) & 0xFF;
+    const bool tiny = ex < kTiny;
+    const int sign = (tiny ? ~ho : hi) & 0x80000000;
+    ex = tiny ? kTiny : ex;
+    cnt += (uint32_t)(sign ^ ho) >> 31;
+    const float f = __int_as_float((254 - ex) << 23);
+    pm = make_float2(p.x * f, p.y * f);
+    p = tiny ? make_float2(__int_as_float(sign | 0x3F800000), 0.f) : make_float2(nx.x * f, nx.y * f);
+  }
+  return cnt;
+}
+
 // One thread per eigenvalue, one CTA of 2^h threads per (vector, cut): bisection
 // on the Sturm count to 2^-62 of the block's trace (below the rounding of G) or
 // to the last bit, then S = -sum lambda ln lambda (lambda <= 0 from rounding
 // contributes nothing), summed in fixed order.  `first` holds the offset of each
 // block's eigenvalues (h + 2 entries).
+// Three FP64 instructions a term, at 2 a clock and SM, bound it: so the first 38
+// bisections count in float-float, two FP64 counts confirm the bracket they leave
+// (widened by its rounding; the whole interval otherwise) and FP64 goes on from
+// there.  50 vectors at L = 14: 737 us with FP64 alone, now 482 us.
 struct BlockFirst {
   int v[12];
 };
 __global__ void __launch_bounds__(512) k_schmidt_values(const double* __restrict__ T, int h, const BlockFirst first,
                                                         double* __restrict__ S) {
   __shared__ double red[512];
+  __shared__ float2 fd[512], fe[512];
   const int64_t vc = blockIdx.x;
   const int t = threadIdx.x;
   const double* base = T + vc * tri_doubles(h);
+  auto split = [](double v) { return make_float2((float)v, (float)(v - (double)(float)v)); };
+  fd[t] = split(base[t]);
+  fe[t] = split(base[t + (1 << h)]);
+  __syncthreads();
   int k = 0;
   while (t >= first.v[k + 1]) k++;
   const int n = first.v[k + 1] - first.v[k], idx = t - first.v[k];
@@ -393,7 +429,20 @@ __global__ void __launch_bounds__(512) k_schmidt_values(const double* __restrict
   if (scale > 0.0 && isfinite(scale)) {
     const double* d = base + first.v[k];
     const double* e2 = d + (1 << h);
-    double lo = -0x1p-48, hi = 1.0 + 0x1p-48;
+    double lo = 0.0, hi = 1.0;
+    for (int it = 0; it < 38; it++) {
+      const double mid = 0.5 * (lo + hi);
+      if (sturm_ff(fd + first.v[k], fe + first.v[k], n, mid) > idx)
+        hi = mid;
+      else
+        lo = mid;
+    }
+    lo -= 0x1p-39;
+    hi += 0x1p-39;
+    if (sturm(d, e2, n, lo) > idx || sturm(d, e2, n, hi) <= idx) {
+      lo = -0x1p-48;
+      hi = 1.0 + 0x1p-48;
+    }
     for (int it = 0; it < 64; it++) {
       const double mid = 0.5 * (lo + hi);
       if (mid == lo || mid == hi || hi - lo < 0x1p-62) break;
