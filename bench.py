@@ -75,16 +75,17 @@ def step_kernel_source_sha():
 
 
 def step_kernel_traffic(precision, workload):
-    """DRAM traffic of one step-kernel launch from the committed ncu summary of
-    this workload and precision, if it was taken on the current kernel source
-    (else None)."""
+    """DRAM bytes per algorithmic byte of the step kernel from the committed ncu
+    summary of this workload and precision, if it was taken on the current
+    kernel source (else None).  A launch carries many steps, so the summary holds
+    a ratio."""
     try:
         sha = step_kernel_source_sha()
         with open(os.path.join(ROOT, "profiles", "step_kernel_traffic.json")) as f:
             d = json.load(f)
         e = d.get(f"{workload}:{precision}")
         if e and e.get("source_sha") == sha:
-            return {"dram_bytes_per_launch_scaled": e["dram_bytes_per_launch"], "source": e.get("summary")}
+            return {"dram_per_alg_byte": e["dram_per_alg_byte"], "source": e.get("summary")}
     except Exception:
         pass
     return None
@@ -534,7 +535,7 @@ def run_single(args, pf, torch, dev, world, rank, local, dist):
     tr = step_kernel_traffic(dom, args.workload)
     roof = {"bound": "hbm", "achieved": d["achieved_gbs"], "peak": peak, "unit": "GB/s",
             "frac": round(d["achieved_gbs"] / peak, 4),
-            "traffic": (tr or {}).get("dram_bytes_per_launch_scaled"),
+            "traffic": round(tr["dram_per_alg_byte"] * d["alg_bytes_per_launch"]) if tr else None,
             "peak_kind": f"of {peak_kind}",
             "kernel": f"k_step_rows<{dom}> (Clenshaw steps on 128-byte column slices, many steps to a launch)",
             "alg_bytes_per_launch": d["alg_bytes_per_launch"], "avg_launch_us": d["avg_launch_us"],

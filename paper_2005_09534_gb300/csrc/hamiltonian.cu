@@ -75,11 +75,11 @@ void upload_binomials() {
 // -------------------------------------------------------------- geometry
 // Low bits of a plan.  Large L: b = 10, a group block of at most C(10,5) * 128 B
 // = 32 KB (six teams to an SM).  Smaller L: few enough rows per group that the
-// groups feed all 912 teams.  Measured on GB300 (whole filter calls, b one lower /
-// chosen / one higher): L = 14 FP64 K = 200 at b = 5 / 6 / 7: 1.39, 1.58, 2.10 ms;
-// L = 18 float-float 256 moments at b = 7 / 8 / 9: 7.2, 6.9, 7.7 ms; L = 20 J1-J2
-// float-float K = 64 at b = 8 / 9 / 10: 10.1, 8.7, 9.6 ms; L = 22 FP32 K = 200 at
-// b = 8 / 9 / 10: 49.7, 46.0, 45.7 ms.
+// groups feed all 912 teams.  Measured on GB300 (whole calls, b one lower / chosen /
+// one higher): L = 14 FP64 K = 200: 1.20, 1.14, 1.37 ms; L = 18 float-float 256
+// moments: 3.16, 2.85, 3.33 ms; L = 20 J1-J2 float-float K = 64: 7.93, 7.23, 7.48 ms
+// (FP32 per column: 3.74, 3.14, 3.04); L = 22 FP32 K = 200 at b = 8 / 9 / 10: 45.1,
+// 40.6, 40.2 ms.
 static int clamp_b(int L, int b) {
   if (const char* e = getenv("POLFED_LOWBITS")) b = atoi(e);
   if (b > 10) b = 10;
@@ -1117,8 +1117,8 @@ __global__ void k_moment_sums(const double2* __restrict__ part, int n_cta, doubl
 
 // The recurrence stays in slice layout from its first step to its last.
 // L = 18, 16 columns, float-float with t_n in FP64: a pair of moments took 53 us
-// as five launches (slice copies in and out, H~, update, sum), now 26, of which
-// about half is the FP64 pipe (conversions, update and sums of 778k elements).
+// as five launches (slice copies in and out, H~, update, sum), now 22, of which
+// about a third is the FP64 pipe (conversions, update and sums of 778k elements).
 int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
                  double* mu, FilterScratch& scr, cudaStream_t s) {
   const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);

@@ -814,8 +814,8 @@ __device__ __forceinline__ bool grid_wait(unsigned* count, unsigned target, int*
 // What bounds it.  A row reads 9.3 rows of 128 bytes through L2 at L = 22 XXZ
 // (itself 1, high bonds 5.8, cross bonds 1, b2 1, x on half of the steps) and
 // 5 more from the staged group: 0.84 GB per step against the 0.32 GB a step
-// cannot do without, of which 0.40 GB come from DRAM.  The time is the latency
-// of those loads (long-scoreboard stalls; issue slots 30%, L2 28%, DRAM 57%
+// cannot do without, of which 0.34 GB come from DRAM.  The time is the latency
+// of those loads (long-scoreboard stalls; issue slots 30%, L2 35%, DRAM 44%
 // busy), so the kernel holds as many independent warps as its registers allow
 // (six teams of four per SM, each with its own group and barrier), keeps
 // uniform values in shared memory and reads everything but the own group
@@ -825,10 +825,12 @@ __device__ __forceinline__ bool grid_wait(unsigned* count, unsigned target, int*
 // its loads wait for one another).
 // Many steps per launch save a launch of about 5 us each, which at L <= 18 is
 // most of the step: the barrier costs 1.4 us.
+// Items are dealt in advance: handed out by an atomic counter instead, neighbouring
+// groups drift apart and L = 20 float-float takes 8.5 ms for 7.3, L = 22 42.4 for 40.6.
 // Measured, us per step and slice of 128 bytes (one launch per step before):
-// L = 14 FP64 37 -> 6.3, L = 18 float-float 28 -> 9, L = 20 J1-J2 float-float
-// 91 -> 66, L = 20 J1-J2 FP32 71 -> 40, L = 22 FP32 128 -> 111, L = 24 J1-J2
-// FP32 1183 -> 800.
+// L = 14 FP64 37 -> 5.2, L = 18 float-float moments 53 -> 22, L = 20 J1-J2
+// float-float 91 -> 56, L = 20 J1-J2 FP32 71 -> 43, L = 22 FP32 128 -> 99,
+// L = 24 J1-J2 FP32 1183 -> 760.
 template <class NT, int LPR, bool J2, StepMode MODE>
 __global__ void __launch_bounds__(kTeam* kMaxTeams, 1) k_step_rows(const __grid_constant__ StepRun R, int tile_bytes) {
   using C = typename NT::C;
