@@ -791,13 +791,28 @@ struct FilterShape {
   size_t slice;  // bytes of one slice buffer
 };
 
-static FilterShape filter_shape(const HamGeometry& g, int kind, int n_b, size_t limit) {
+static FilterShape slices_of(const HamGeometry& g, int kind, int n_b, size_t limit, int lpr) {
   FilterShape f;
-  f.lpr = choose_lpr(kind, n_b);
+  f.lpr = lpr;
   f.W = slice_width(kind, f.lpr);
   f.nsl = (n_b + f.W - 1) / f.W;
   f.slice = ((size_t)g.dim * f.W * elem_bytes(kind) + 255) & ~(size_t)255;
   f.ns = (int)std::max<size_t>(1, std::min<size_t>((size_t)f.nsl, limit / (3 * f.slice)));
+  return f;
+}
+
+static FilterShape filter_shape(const HamGeometry& g, int kind, int n_b, size_t limit) {
+  return slices_of(g, kind, n_b, limit, choose_lpr(kind, n_b));
+}
+
+// The FP32 filter takes 64-byte rows where a slice of 128-byte ones, the gather
+// source, is beyond L2 (346 MB at L = 24) and rows gather few neighbours: XXZ,
+// 32 columns, K = 40: 18.5 ms with 128 bytes, 17.2 with 64 (21.2 with 32).  Within L2
+// (L = 22) they cost 7%; J1-J2 gains nothing (38.1 and 38.3 ms at L = 24).
+static FilterShape filter_rows(const HamGeometry& g, int kind, int n_b, size_t limit) {
+  const FilterShape f = filter_shape(g, kind, n_b, limit);
+  if (kind == POLFED_F32 && f.lpr == 8 && f.slice > ((size_t)160 << 20) && g.rec_stride == 16)
+    return slices_of(g, kind, n_b, limit, 4);
   return f;
 }
 
@@ -1080,7 +1095,7 @@ static int filter_slices(HamPlan& plan, int kind, const FilterShape& f, const Co
 
 int filter_block(HamPlan& plan, int kind, const double* c, int K, double invD, const void* in, void* out, int n_b,
                  int abi_kind, FilterScratch& scr, cudaStream_t s) {
-  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_rows(plan.geo, kind, n_b, kSliceSet);
   return filter_slices(plan, kind, f, [c](int n) { return c[n]; }, K, invD, nullptr, in, out, n_b, abi_kind, scr, s);
 }
 
