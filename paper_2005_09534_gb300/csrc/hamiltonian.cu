@@ -318,7 +318,6 @@ __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, c
   if (i < (1 << g.b)) {
     const uint32_t a = (uint32_t)i, r = rank_lo(a);
     const int pos = g.cls_off[__popc(a)] + (int)r;
-    t.T_lo[i] = (uint16_t)r;
     t.U_lo[pos] = (uint16_t)i;
     double d = 0.0;
     for (int q = 0; q < g.n_low1 + g.n_low2; q++) {
@@ -581,7 +580,7 @@ static int lpr_index(int lpr) { return lpr == 8 ? 3 : (lpr == 4 ? 2 : (lpr == 2 
 
 // Offsets of the tables of a geometry in one allocation.
 struct PlanLayout {
-  size_t Tlo, Ulo, Thi, Ord, Flo, Fhi, Cx, Grp, Err, Rec, total;
+  size_t Ulo, Thi, Ord, Flo, Fhi, Cx, Grp, Err, Rec, total;
   size_t rec1;  // bytes of one record table
   explicit PlanLayout(const HamGeometry& g) {
     const size_t nlo = (size_t)1 << g.b, nhi = (size_t)1 << g.nh, ncx = (size_t)1 << g.n_cross;
@@ -591,7 +590,6 @@ struct PlanLayout {
       total += (n + 255) & ~(size_t)255;
       return o;
     };
-    Tlo = carve(nlo * 2);
     Ulo = carve(nlo * 2);
     Thi = carve(nhi * 4);
     Ord = carve(nhi * 4);
@@ -619,7 +617,6 @@ static int typed_out(int kind, double e_lo, double e_hi, void* dst, TypedOut* ty
 // Point the plan's tables into `base` and enqueue the kernels that fill them.
 int HamPlan::bind(char* base, cudaStream_t s, int kind, double e_lo, double e_hi, void* typed_dst) {
   const PlanLayout lay(geo);
-  tab.T_lo = (uint16_t*)(base + lay.Tlo);
   tab.U_lo = (uint16_t*)(base + lay.Ulo);
   tab.T_hi = (int32_t*)(base + lay.Thi);
   tab.order = (int32_t*)(base + lay.Ord);

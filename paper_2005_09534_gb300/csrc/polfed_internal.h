@@ -106,8 +106,7 @@ struct HamGeometry {
 
 // Device tables of a geometry (owned by HamPlan).
 struct HamTables {
-  uint16_t* T_lo;   // [2^b] rank of s_lo among b-bit strings of equal popcount
-  uint16_t* U_lo;   // [2^b] inverse: U_lo[cls_off[c] + k] = k-th b-bit string with popcount c
+  uint16_t* U_lo;   // [2^b] inverse of T_lo: U_lo[cls_off[c] + k] = k-th b-bit string with popcount c
   int32_t* T_hi;    // [2^nh] first row of group s_hi, -1 if the group is empty
   int32_t* order;   // [n_groups] groups, largest first
   double* F_lo;     // [2^b] diagonal part from low bonds and low fields (H units)
