@@ -253,6 +253,27 @@ __global__ void __launch_bounds__(kTriThreads) k_schmidt_tri(const double* __res
     }
   }
   __syncthreads();
+  // Scale by the power of two that brings the trace into [1/2, 1), so that the squares of the reduction
+  // neither overflow nor (above the tail it drops) underflow
+  if (warp == 0) {
+    double t = 0.0;
+    for (int i = lane; i < n; i += 32) t += A[i * P + i];
+    t = warp_sum(t);
+    if (lane == 0) {
+      int ex = 0;
+      frexp(t, &ex);
+      ex = max(ex, -1000);
+      const bool fin = t > 0.0 && isfinite(t);
+      sc[2] = ldexp(1.0, -ex);
+      sc[3] = fin ? 1.0 : 0.0;
+      // not fin: t is 0 (an empty block) or not finite
+      T[vc * tri_doubles(h) + (2 << h) + (blockIdx.y ? k1 : k0)] = fin ? ldexp(1.0, ex) : t;
+    }
+  }
+  __syncthreads();
+  if (sc[3] == 0.0) return;  // k_schmidt_values reads the scale alone
+  for (int e = tid; e < n * P; e += kTriThreads) A[e] *= sc[2];
+  __syncthreads();
   for (int k = 0; k + 2 < n; k++) {
     // v = x - alpha e_1, x = A[k+1.., k]; beta = 2 / |v|^2
     const int m = n - k - 1;
@@ -263,11 +284,13 @@ __global__ void __launch_bounds__(kTriThreads) k_schmidt_tri(const double* __res
         if (i > 0) s = fma(x[i * P], x[i * P], s);
       s = warp_sum(s);
       if (lane == 0) {
-        const double x0 = x[0], nx2 = fma(x0, x0, s);
+        const double x0 = x[0];
         double beta = 0.0, v0 = x0;
-        double off2 = nx2;
-        if (s > 0.0) {
-          const double nx = sqrt(nx2);
+        double off2 = x0 * x0;
+        // a tail below 2^-450 of the trace is taken as zero: its square would leave FP64's range
+        if (s > 0x1p-900) {
+          off2 = fma(x0, x0, s);
+          const double nx = sqrt(off2);
           v0 = x0 + (x0 >= 0.0 ? nx : -nx);
           beta = 2.0 / fma(v0, v0, s);
         }
@@ -326,27 +349,6 @@ __global__ void __launch_bounds__(kTriThreads) k_schmidt_tri(const double* __res
     d[n - 1] = A[(n - 1) * P + n - 1];
     e2[n - 1] = 0.0;
   }
-  __syncthreads();
-  // scale by the power of two that brings the trace into [1/2, 1)
-  if (warp == 0) {
-    double t = 0.0;
-    for (int i = lane; i < n; i += 32) t += d[i];
-    t = warp_sum(t);
-    if (lane == 0) {
-      int ex = 0;
-      frexp(t, &ex);
-      const bool fin = t > 0.0 && isfinite(t);
-      sc[2] = fin ? ldexp(1.0, -ex) : t;  // 0: an empty block; otherwise not finite
-      sc[3] = fin ? 1.0 : 0.0;
-      T[vc * tri_doubles(h) + (2 << h) + (blockIdx.y ? k1 : k0)] = fin ? ldexp(1.0, ex) : t;
-    }
-  }
-  __syncthreads();
-  if (sc[3] != 0.0)
-    for (int i = tid; i < n; i += kTriThreads) {
-      d[i] *= sc[2];
-      e2[i] *= sc[2] * sc[2];
-    }
 }
 
 // Number of eigenvalues below x of the tridiagonal (d, e2), by the signs of the
