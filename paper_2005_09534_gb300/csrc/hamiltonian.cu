@@ -813,8 +813,6 @@ static FilterShape filter_rows(const HamGeometry& g, int kind, int n_b, size_t l
   return f;
 }
 
-constexpr size_t kSliceSet = (size_t)96 << 20;  // of the 126 MB L2
-
 // The launches of a block: sets of ns slices, and the columns that do not fill
 // the last slice by themselves in a narrower one.  Small problems, whose slices
 // all run together, keep the padded slice: it shares their launch.  L = 20,
@@ -842,7 +840,7 @@ static std::vector<SlicePart> slice_parts(const HamGeometry& g, int kind, const 
 }
 
 size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b) {
-  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, plan.slice_set);
   return 3 * (size_t)f.ns * f.slice + 256;
 }
 
@@ -1092,20 +1090,20 @@ static int filter_slices(HamPlan& plan, int kind, const FilterShape& f, const Co
 
 int filter_block(HamPlan& plan, int kind, const double* c, int K, double invD, const void* in, void* out, int n_b,
                  int abi_kind, FilterScratch& scr, cudaStream_t s) {
-  const FilterShape f = filter_rows(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_rows(plan.geo, kind, n_b, plan.slice_set);
   return filter_slices(plan, kind, f, [c](int n) { return c[n]; }, K, invD, nullptr, in, out, n_b, abi_kind, scr, s);
 }
 
 int filter_block_cols(HamPlan& plan, const float* d_coef, int K, const void* in, void* out, int n_b, int abi_kind,
                       FilterScratch& scr, cudaStream_t s) {
   if (K < 1) return fail(POLFED_EINVAL, "per-column filter needs K >= 1");
-  const FilterShape f = filter_shape(plan.geo, POLFED_F32, n_b, kSliceSet);
+  const FilterShape f = filter_shape(plan.geo, POLFED_F32, n_b, plan.slice_set);
   return filter_slices(plan, POLFED_F32, f, [](int) { return 1.0; }, K, 1.0, d_coef, in, out, n_b, abi_kind, scr, s);
 }
 
 size_t moment_scratch_bytes(const HamPlan& plan, int kind, int n_b) {
   if (kind != POLFED_DF64) return 0;
-  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, plan.slice_set);
   return f.ns * f.slice;
 }
 
@@ -1133,7 +1131,7 @@ __global__ void k_moment_sums(const double2* __restrict__ part, int n_cta, doubl
 // about a third is the FP64 pipe (conversions, update and sums of 778k elements).
 int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
                  double* mu, FilterScratch& scr, cudaStream_t s) {
-  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, plan.slice_set);
   PF_CHECK(carve_scratch(scr, f));
   const int64_t dim = plan.geo.dim;
   const int abi = kind == POLFED_F32 ? POLFED_F32 : POLFED_F64;
@@ -1184,7 +1182,7 @@ bool apply_direct(int kind, int abi_kind, int n_b, const void* in, const void* o
 
 int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int abi_kind, FilterScratch& scr,
                 cudaStream_t s) {
-  const FilterShape f = filter_shape(plan.geo, kind, n_b, kSliceSet);
+  const FilterShape f = filter_shape(plan.geo, kind, n_b, plan.slice_set);
   if (apply_direct(kind, abi_kind, n_b, in, out)) {
     const size_t pitch = (size_t)n_b * elem_bytes(kind);
     PF_CHECK(check_operator(plan, kind));

@@ -96,6 +96,10 @@ struct polfed_ctx {
 
 namespace {
 
+// Several slices in one launch need several slices' buffers: a context with a
+// bounded workspace filters one at a time, in the least that the method needs.
+size_t slice_set(const polfed_ctx* c) { return c->ws_limit ? 0 : kSliceSet; }
+
 struct ScopedDevice {
   int prev = 0;
   explicit ScopedDevice(int d) {
@@ -976,6 +980,7 @@ int polfed_block_lanczos(polfed_ctx* c, const polfed_model* model, double e_lo, 
   if (n_b < 1 || n_b > 128) return fail(POLFED_EINVAL, "n_b must be in 1..128");
   ScopedDevice sd(c->device);
   HamPlan plan;
+  plan.slice_set = slice_set(c);
   PF_CHECK(plan.init(model, c->stream, false));
   const double hn = std::max(std::fabs(e_lo), std::fabs(e_hi));
   LanczosParams P{e_lo, e_hi, sigma, K, round_block(n_b), N_ev, c->opts, c->opts.tol_resid * hn / (0.5 * (e_hi - e_lo)),
@@ -1067,6 +1072,7 @@ int eigs_impl(polfed_ctx* c, const polfed_model* model, double eps_target, int32
   const double t0 = now_s();
   const Counters cn0 = counters();
   HamPlan plan;
+  plan.slice_set = slice_set(c);
   PF_CHECK(plan.init(model, c->stream, false, hook ? hook->plan_b(model->L) : -1));
   count_launch(4);  // table kernels
   const int64_t dim = plan.geo.dim;
@@ -1340,6 +1346,7 @@ int polfed_spectral_bounds(polfed_ctx* c, const polfed_model* model, double* bou
   if (!bounds) return fail(POLFED_EINVAL, "bounds is NULL");
   ScopedDevice sd(c->device);
   HamPlan plan;
+  plan.slice_set = slice_set(c);
   PF_CHECK(plan.init(model, c->stream, false));
   polfed_opts o = c->opts;
   if (!c->have_opts) polfed_opts_default(&o);
@@ -1357,6 +1364,7 @@ int polfed_spectral_labels(polfed_ctx* c, const polfed_model* model, double eps_
   if (R < 1 || R > 128) return fail(POLFED_EINVAL, "R must be in 1..128");
   ScopedDevice sd(c->device);
   HamPlan plan;
+  plan.slice_set = slice_set(c);
   PF_CHECK(plan.init(model, c->stream, false));
   polfed_opts o = c->opts;
   if (!c->have_opts) polfed_opts_default(&o);

@@ -136,6 +136,8 @@ struct alignas(16) GroupRec {
 
 int build_geometry(const polfed_model* m, int b_override, HamGeometry* g);
 
+constexpr size_t kSliceSet = (size_t)96 << 20;  // of the 126 MB L2
+
 class HamPlan {
  public:
   HamGeometry geo;
@@ -150,6 +152,7 @@ class HamPlan {
   double typed_lo[3] = {0, 0, 0}, typed_hi[3] = {0, 0, 0};
   cudaStream_t stream = nullptr;
   bool stream_alloc = false;  // tables from cudaMallocAsync
+  size_t slice_set = kSliceSet;  // bytes of the column slices that run in one launch; 0: one slice at a time
 
   // All of these only enqueue work on the stream.
   // kind >= 0: with the scaled tables of that storage type (prepare_typed in the same launch)
