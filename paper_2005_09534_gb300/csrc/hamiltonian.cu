@@ -959,8 +959,11 @@ struct StepTimer {
     b0 = counters().all_alg_bytes[kind];
     if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) cudaEventRecord(e0, s);
   }
-  int stop() {
-    if (!e0 || !e1) return POLFED_OK;
+  int stop() {  // synchronizes
+    if (!e0 || !e1) {
+      PF_CUDA(cudaStreamSynchronize(s));
+      return POLFED_OK;
+    }
     PF_CUDA(cudaEventRecord(e1, s));
     PF_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -1035,6 +1038,7 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
   const int chunk = steps_per_launch(row);
   std::lock_guard<std::mutex> lk(coop_mutex());
+  StepTimer tm(s, kind);  // under the lock: the time of these launches, not of other threads' before them
   for (int st = 0; st < K; st += chunk) {
     run.st0 = st;
     run.st1 = std::min(K, st + chunk);
@@ -1054,7 +1058,7 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
     plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
     count_step(kind, alg);
   }
-  PF_CUDA(cudaStreamSynchronize(s));  // the lock is released when the last launch is done
+  PF_CHECK(tm.stop());  // synchronizes: the lock is released when the last launch is done
   *res = (K % 2 == 0) ? b.ba : b.bb;
   return POLFED_OK;
 }
@@ -1079,9 +1083,7 @@ static int filter_slices(HamPlan& plan, int kind, const FilterShape& f, const Co
     PF_CHECK(slice_in(kind, abi_kind, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.xs, b.ba, col ? 1.0 : coef(K), scr.flag,
                       s, col ? col + (size_t)K * f.W : nullptr, colstride));
     char* res = nullptr;
-    StepTimer tm(s, kind);
     PF_CHECK(run_steps(plan, kind, p.f, p.ns, coef, K, invD, col, colstride, f.W, b, s, &res));
-    PF_CHECK(tm.stop());
     PF_CHECK(check_timeout(plan, s));
     PF_CHECK(slice_out(kind, abi_kind, res, dim, p.f, p.ns, p.ncols, out, n_b, p.col0, scr.flag, s));
   }
@@ -1341,12 +1343,12 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
     run.bar = (unsigned*)(base + Lo.bar_off);
     run.err = (int*)(base + Lo.bar_off + 64);
     run.cap = wait_cap(kBarrierWaitPolls);
-    StepTimer tm(s, kind);
     int grid;
     int e = 0;
     const double g0 = counters().step_gpu_s;
     {
       std::lock_guard<std::mutex> lk(coop_mutex());
+      StepTimer tm(s, kind);
       grid = launch_rows(run, kind, kBatchLpr, j2, kFilter, max_group, groups, true, s,
                          ctas_per_sm == 1 ? kMaxTeams / 2 : kMaxTeams);
       if (grid < 0) return grid;
