@@ -172,7 +172,8 @@ int polfed_h_apply(const polfed_model* model, const uint32_t* d_states, int64_t 
  *            Y = sum_n coeffs[n] T_n(H~) X.
  *   other arguments as in polfed_h_apply.
  * Runs the K steps of the block's column slices in a few cooperative launches
- * (one at a time per device in a process); synchronizes the
+ * (one at a time per device in a process; threads take turns of at most about a
+ * quarter of a second); synchronizes the
  * stream before returning (it owns stream-ordered scratch).  Returns
  * POLFED_EBOUNDS if the output is not finite (spectrum outside [e_lo, e_hi]). */
 int polfed_cheb_filter(const polfed_model* model, const uint32_t* d_states, int64_t dim, double e_lo, double e_hi,
@@ -428,10 +429,11 @@ int polfed_mlp_predict(polfed_mlp* net, const polfed_model* model, double W, dou
  * per compute node; this is the single-GPU form of that parallelism).
  * ------------------------------------------------------------------------ */
 
-/* Eq. (2) filter of many realizations in ONE cooperative kernel launch: every
- * (realization, 128-byte column slice) job runs its own Clenshaw recurrence of
+/* Eq. (2) filter of many realizations together, in cooperative launches of
+ * all of them (turns as in polfed_cheb_filter): every (realization,
+ * 128-byte column slice) job runs its own Clenshaw recurrence of
  * order K[i] with the paper's coefficients for sigma[i], on its own H~ (plans
- * with a low/high split of their own).  Launch step t performs step t
+ * with a low/high split of their own).  Step t of the launches performs step t
  * of every job with t < K[i]; CTAs meet at a grid barrier between steps
  * (bounded wait: POLFED_ETIMEOUT, never a hang).
  *   n_inst       : number of realizations (>= 1); all with J2 == 0 or all with J2 != 0.
@@ -452,7 +454,7 @@ int polfed_cheb_filter_batched(int32_t n_inst, const polfed_model* models, const
 typedef struct polfed_batch_info {
   int32_t n_b;              /* block width of realization 0 */
   int32_t ctas_per_sm;      /* team setting of the batched filter (as in polfed_cheb_filter_batched) */
-  int32_t rounds;           /* batched filter launches */
+  int32_t rounds;           /* batched filter calls */
   int32_t workers;          /* host threads */
   int32_t n_width16, n_width32, n_width64; /* realizations per block width */
   int32_t reserved;

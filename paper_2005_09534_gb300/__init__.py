@@ -489,7 +489,7 @@ def _models_array(models):
 
 
 def cheb_filter_batched(models, e_lo, e_hi, sigma, K, Xs, Ys, n_b, dtype, ctas_per_sm=0, stream=None):
-    """polfed_cheb_filter_batched: all realizations' filters in one cooperative launch."""
+    """polfed_cheb_filter_batched: all realizations' filters in the same cooperative launches."""
     n = len(models)
     keep, arr = _models_array(models)
     lo = np.ascontiguousarray(e_lo, dtype=np.float64)

@@ -5,8 +5,8 @@
 // fills a fraction of the 152 SMs and pays a kernel launch per Chebyshev
 // step.  Here every realization runs the polfed_eigs driver on its own host
 // thread, context and stream, and their filter calls meet at a rendezvous:
-// once every running realization has asked for its filter, one cooperative
-// launch (filter_batched) advances all of their Clenshaw recurrences, each
+// once every running realization has asked for its filter, the cooperative
+// launches of filter_batched advance all of their Clenshaw recurrences, each
 // with its own operator, order K and block.  Everything else (bounds, block
 // Gram-Schmidt, Cholesky QR, the projected eigenproblem, Rayleigh-Ritz) runs
 // concurrently on the realizations' own streams.

@@ -29,6 +29,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <atomic>
+#include <condition_variable>
 #include <mutex>
 #include <type_traits>
 
@@ -770,12 +771,49 @@ static int launch_rows(const StepRun& run, int kind, int lpr, bool j2, StepMode 
 }
 
 // A cooperative grid fills the GPU and its CTAs wait for one another, so only
-// one is in flight per device: the lock is held from launch to completion.
-static std::mutex& coop_mutex() {
-  static std::mutex mu[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  return mu[dev & 63];
+// one is in flight per device: a thread holds a turn from a launch to its
+// completion.  Turns are given in the order of asking, and a call of many
+// launches gives its turn up about every kTurnSeconds, so that a short call of
+// another thread does not wait for the end of a long one.
+class Turn {
+  struct Queue {
+    std::mutex mu;
+    std::condition_variable cv;
+    uint64_t next = 0, serving = 0;
+  };
+  static Queue& queue() {
+    static Queue q[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return q[dev & 63];
+  }
+  Queue& q_;
+
+ public:
+  Turn() : q_(queue()) {
+    std::unique_lock<std::mutex> lk(q_.mu);
+    const uint64_t mine = q_.next++;
+    q_.cv.wait(lk, [&] { return q_.serving == mine; });
+  }
+  ~Turn() {
+    {
+      std::lock_guard<std::mutex> lk(q_.mu);
+      q_.serving++;
+    }
+    q_.cv.notify_all();
+  }
+  Turn(const Turn&) = delete;
+  Turn& operator=(const Turn&) = delete;
+};
+
+constexpr double kTurnSeconds = 0.25;
+
+// An upper estimate of a step's seconds, by the bytes of its slices (measured: 1.7 to 3.6 TB/s in FP32 and
+// float-float; half of that and less where FP64 bounds it) and by the rows of the busiest team (0.1 to 0.2 us each
+// of 128 bytes).  Launches and turns are cut by it; a turn's end costs about 20 us.
+static double step_seconds(double row_bytes, int64_t items, int max_group) {
+  const int64_t teams = 152 * kMaxTeams, rounds = (items + teams - 1) / teams;
+  return 5e-6 + std::max(4.0 * row_bytes / 0.5e12, 0.4e-6 * (double)rounds * max_group);
 }
 
 // ------------------------------------------------------------ filter engine
@@ -1015,11 +1053,6 @@ static int cooperative_run(HamPlan& plan, int kind, const FilterShape& f, int ns
   return POLFED_OK;
 }
 
-// steps of a launch: it stays under about a quarter of a second, and its coefficients fit the parameters
-static int steps_per_launch(double row_bytes) {
-  return std::min(kParamSteps, std::max(2, (int)(0.25 * 3e12 / (4.0 * row_bytes) + 1)));
-}
-
 // The Clenshaw steps k = K-1..1 and the final step of Eq. (2) of `ns` slices
 // (b_K in ba, X in xs), several steps to a cooperative launch: K = 200 at
 // L = 14 costs one launch instead of 200.  coef(n) gives c_n; col (device) the
@@ -1036,29 +1069,34 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
   run.one.colw = colw;
   const int64_t items = (int64_t)plan.geo.n_groups * ns;
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
-  const int chunk = steps_per_launch(row);
-  std::lock_guard<std::mutex> lk(coop_mutex());
-  StepTimer tm(s, kind);  // under the lock: the time of these launches, not of other threads' before them
-  for (int st = 0; st < K; st += chunk) {
-    run.st0 = st;
-    run.st1 = std::min(K, st + chunk);
-    run.bar_base = plan.bar_base;
-    double alg = 0.0;
-    for (int q = run.st0; q < run.st1; q++) {
-      const int k = K - 1 - q;
-      double c = col ? 1.0 : coef(k);
-      if (!col) {
-        if (k == 0) c *= invD;
-        run.cx[q - st] = typed_const(kind, c);
+  const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
+  for (int t0 = 0; t0 < K; t0 += turn_steps) {
+    {
+      const Turn turn;
+      StepTimer tm(s, kind);  // within the turn: the time of these launches, not of other threads' before them
+      for (int st = t0, end = std::min(K, t0 + turn_steps); st < end; st = run.st1) {
+        run.st0 = st;
+        run.st1 = std::min(end, st + kParamSteps);
+        run.bar_base = plan.bar_base;
+        double alg = 0.0;
+        for (int q = run.st0; q < run.st1; q++) {
+          const int k = K - 1 - q;
+          double c = col ? 1.0 : coef(k);
+          if (!col) {
+            if (k == 0) c *= invD;
+            run.cx[q - st] = typed_const(kind, c);
+          }
+          alg += row * (3.0 + (c != 0.0 ? 1.0 : 0.0));
+        }
+        const int grid = launch_rows(run, kind, f.lpr, j2, col ? kFilterCols : kFilter, plan.geo.max_group, items, true, s);
+        if (grid < 0) return grid;
+        plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
+        count_step(kind, alg);
       }
-      alg += row * (3.0 + (c != 0.0 ? 1.0 : 0.0));
+      PF_CHECK(tm.stop());  // synchronizes: the turn ends when its last launch is done
     }
-    const int grid = launch_rows(run, kind, f.lpr, j2, col ? kFilterCols : kFilter, plan.geo.max_group, items, true, s);
-    if (grid < 0) return grid;
-    plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
-    count_step(kind, alg);
+    PF_CHECK(check_timeout(plan, s));
   }
-  PF_CHECK(tm.stop());  // synchronizes: the lock is released when the last launch is done
   *res = (K % 2 == 0) ? b.ba : b.bb;
   return POLFED_OK;
 }
@@ -1084,7 +1122,6 @@ static int filter_slices(HamPlan& plan, int kind, const FilterShape& f, const Co
                       s, col ? col + (size_t)K * f.W : nullptr, colstride));
     char* res = nullptr;
     PF_CHECK(run_steps(plan, kind, p.f, p.ns, coef, K, invD, col, colstride, f.W, b, s, &res));
-    PF_CHECK(check_timeout(plan, s));
     PF_CHECK(slice_out(kind, abi_kind, res, dim, p.f, p.ns, p.ncols, out, n_b, p.col0, scr.flag, s));
   }
   return POLFED_OK;
@@ -1139,7 +1176,6 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
   const int abi = kind == POLFED_F32 ? POLFED_F32 : POLFED_F64;
   const bool j2 = plan.geo.rec_stride == 32;
   PF_CUDA(cudaMemsetAsync(mu, 0, (size_t)2 * half * sizeof(double), s));
-  std::lock_guard<std::mutex> lk(coop_mutex());
   for (const SlicePart& p : slice_parts(plan.geo, kind, f, n_b)) {
     const SliceBufs b(scr, p.f);
     PF_CHECK(slice_in(kind, abi, in, dim, n_b, p.col0, p.ncols, p.f, p.ns, b.ba, nullptr, 0.0, nullptr, s));
@@ -1155,22 +1191,30 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
     const int64_t items = (int64_t)plan.geo.n_groups * p.ns;
     const double row = (double)dim * p.f.W * elem_bytes(kind) * p.ns;
     const int64_t per_step = std::min<int64_t>(items, kMaxMomentCtas) * sizeof(double2);
-    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(steps_per_launch(row), (int64_t)part_bytes / per_step));
-    for (int st = 0; st < half; st += chunk) {
-      run.st0 = st;
-      run.st1 = std::min(half, st + chunk);
-      run.bar_base = plan.bar_base;
-      const int n = run.st1 - run.st0;
-      const int grid = launch_rows(run, kind, p.f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
-      if (grid < 0) return grid;
-      plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
-      count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
-      k_moment_sums<<<n, 32, 0, s>>>((const double2*)part, grid, mu + 2 * st);
-      PF_CUDA(cudaGetLastError());
-      count_launch();
+    const int launch_steps = (int)std::max<int64_t>(1, std::min<int64_t>(kParamSteps, (int64_t)part_bytes / per_step));
+    const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
+    for (int t0 = 0; t0 < half; t0 += turn_steps) {
+      {
+        const Turn turn;
+        for (int st = t0, end = std::min(half, t0 + turn_steps); st < end; st = run.st1) {
+          run.st0 = st;
+          run.st1 = std::min(end, st + launch_steps);
+          run.bar_base = plan.bar_base;
+          const int n = run.st1 - run.st0;
+          const int grid = launch_rows(run, kind, p.f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
+          if (grid < 0) return grid;
+          plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
+          count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
+          k_moment_sums<<<n, 32, 0, s>>>((const double2*)part, grid, mu + 2 * st);
+          PF_CUDA(cudaGetLastError());
+          count_launch();
+        }
+        PF_CUDA(cudaStreamSynchronize(s));
+      }
+      PF_CHECK(check_timeout(plan, s));
     }
   }
-  return check_timeout(plan, s);
+  return POLFED_OK;
 }
 
 // Rows that are whole slices of 16-byte chunks are gathered where they lie: 64
@@ -1343,17 +1387,31 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
     run.bar = (unsigned*)(base + Lo.bar_off);
     run.err = (int*)(base + Lo.bar_off + 64);
     run.cap = wait_cap(kBarrierWaitPolls);
-    int grid;
-    int e = 0;
+    int grid = 0;
     const double g0 = counters().step_gpu_s;
-    {
-      std::lock_guard<std::mutex> lk(coop_mutex());
-      StepTimer tm(s, kind);
-      grid = launch_rows(run, kind, kBatchLpr, j2, kFilter, max_group, groups, true, s,
-                         ctas_per_sm == 1 ? kMaxTeams / 2 : kMaxTeams);
-      if (grid < 0) return grid;
-      count_step(kind, alg);  // one launch carrying every job's steps
-      PF_CHECK(tm.stop());
+    double row = 0.0;  // of a step that every job takes part in
+    for (const auto& it : items) {
+      const FilterShape f = batch_shape(it.plan->geo, kind, it.n_b);
+      row += (double)it.plan->geo.dim * f.W * elem_bytes(kind) * f.nsl;
+    }
+    const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, groups, max_group)));
+    for (int st = 0; st < n_steps; st += turn_steps) {
+      run.st0 = st;
+      run.st1 = std::min(n_steps, st + turn_steps);
+      {
+        const Turn turn;
+        StepTimer tm(s, kind);
+        grid = launch_rows(run, kind, kBatchLpr, j2, kFilter, max_group, groups, true, s,
+                           ctas_per_sm == 1 ? kMaxTeams / 2 : kMaxTeams);
+        if (grid < 0) return grid;
+        count_step(kind, alg * (run.st1 - run.st0) / n_steps);  // one launch carries every job's steps
+        PF_CHECK(tm.stop());
+      }
+      run.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
+      int e = 0;
+      PF_CUDA(cudaMemcpyAsync(&e, run.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+      PF_CUDA(cudaStreamSynchronize(s));
+      if (e) return fail(POLFED_ETIMEOUT, "a grid barrier of the batched filter timed out");
     }
     if (bst) {
       bst->n_jobs = (int)jobs.size();
@@ -1362,9 +1420,6 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
       bst->gpu_s = counters().step_gpu_s - g0;
       bst->alg_bytes = alg;
     }
-    PF_CUDA(cudaMemcpyAsync(&e, run.err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    PF_CUDA(cudaStreamSynchronize(s));
-    if (e) return fail(POLFED_ETIMEOUT, "a grid barrier of the batched filter timed out");
   }
   // outputs: the buffer written by each job's last step
   pos = Lo.slices_off;

@@ -199,7 +199,7 @@ size_t moment_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 size_t filter_scratch_bytes(const HamPlan& plan, int kind, int n_b);
 int choose_lpr(int kind, int n_b);
 
-// Batched filter: one cooperative launch runs the Clenshaw recurrences of
+// Batched filter: cooperative launches advance the Clenshaw recurrences of
 // many (realization, 128-byte column slice) jobs, each with its own plan,
 // order and coefficients (F32 or DF64 storage; all jobs J2 == 0 or all not).
 constexpr int kBatchLpr = 8;  // 128-byte slices
