@@ -158,6 +158,7 @@ __global__ void k_mlp_init(float* p, int n, uint64_t seed, int d_in, int H, int 
 
 // ------------------------------------------------------- fused batch rows
 constexpr int kFusedMax = 512;  // inputs and hidden units of the fused kernels
+constexpr int kMaxOut = 64;
 constexpr int kRowThreads = 256;
 
 struct RowArgs {
@@ -489,13 +490,10 @@ int run_rows(polfed_mlp* n, const float* x, const float* t, int B, float* y, con
                   w.dz2, w.dz1, w.lossp, y, B, n->d_in, n->H, n->d_out};
   const size_t smem = rows_smem(w.tb, n->d_in, n->H, n->d_out);
   const int grid = (B + w.tb - 1) / w.tb;
-  if (w.tb == 4) {
-    if (smem > 48 * 1024) PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (w.tb == 4)
     k_mlp_rows<4><<<grid, kRowThreads, smem, s>>>(A);
-  } else {
-    if (smem > 48 * 1024) PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  else
     k_mlp_rows<8><<<grid, kRowThreads, smem, s>>>(A);
-  }
   PF_CUDA(cudaGetLastError());
   count_launch();
   return POLFED_OK;
@@ -511,6 +509,15 @@ int forward(polfed_mlp* n, const float* x, int B, cudaStream_t s, Work* w) {
   k_mlp_layer<<<nblk(B * n->d_out), 256, 0, s>>>(v.W3, v.b3, w->a2, B, n->H, n->d_out, 0, w->y);
   PF_CUDA(cudaGetLastError());
   count_launch(4);
+  return POLFED_OK;
+}
+
+// The shared memory that the largest fused network takes, for every network: the limit belongs to the kernel,
+// and a call that set its own could lower it under another thread's launch.
+int allow_rows_smem() {
+  const int big = (int)rows_smem(8, kFusedMax, kFusedMax, kMaxOut);
+  PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  PF_CUDA(cudaFuncSetAttribute(k_mlp_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   return POLFED_OK;
 }
 
@@ -602,7 +609,7 @@ void polfed_mlp_destroy(polfed_mlp* n) {
 
 int polfed_mlp_create(int32_t d_in, int32_t hidden, int32_t d_out, uint64_t seed, polfed_mlp** out) {
   if (!out) return fail(POLFED_EINVAL, "out is NULL");
-  if (d_in < 1 || d_in > 1024 || d_out < 1 || d_out > 64 || hidden < d_out || hidden > 4096)
+  if (d_in < 1 || d_in > 1024 || d_out < 1 || d_out > kMaxOut || hidden < d_out || hidden > 4096)
     return fail(POLFED_EINVAL, "need 1 <= d_in <= 1024, 1 <= d_out <= 64, d_out <= hidden <= 4096");
   polfed_mlp* n = new polfed_mlp();
   n->d_in = d_in;
@@ -619,6 +626,10 @@ int polfed_mlp_create(int32_t d_in, int32_t hidden, int32_t d_out, uint64_t seed
     cudaGetLastError();
     polfed_mlp_destroy(n);
     return fail(POLFED_ENOMEM, "MLP allocation failed");
+  }
+  if (const int e = allow_rows_smem()) {
+    polfed_mlp_destroy(n);
+    return e;
   }
   n->h_scale.assign(2 * d_in + 2 * d_out, 0.f);
   for (int i = 0; i < d_in; i++) n->h_scale[d_in + i] = 1.f;

@@ -9,11 +9,11 @@ from gpu_common import lib, torch_dev
 pytestmark = pytest.mark.gpu
 
 
-def test_two_networks_on_two_threads():
+def test_networks_of_two_sizes_on_eight_threads():
     torch, dev = torch_dev()
     pf = lib()
     # 8 batch rows x (inputs + 3 x hidden + 2 x outputs) floats: 65 and 55 KB
-    nets = [pf.MLP(512, 512, 3, 1), pf.MLP(512, 400, 3, 2)]
+    nets = [pf.MLP(512, 512 if i % 2 else 400, 3, i) for i in range(8)]
     B = 1100
     X = torch.randn(B, 512, device=dev)
     want = []
@@ -37,7 +37,7 @@ def test_two_networks_on_two_threads():
         if not torch.equal(y, want[i]):
             errors.append(f"network {i}: other outputs")
 
-    ts = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(8)]
     [t.start() for t in ts]
     [t.join() for t in ts]
     assert not errors, (len(errors), errors[:3])
