@@ -12,6 +12,7 @@
 //   W1 [H x d_in] row-major, b1 [H], W2 [H x H], b2 [H], W3 [d_out x H], b3 [d_out].
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <vector>
 
@@ -702,7 +703,11 @@ int polfed_mlp_forward(polfed_mlp* n, const float* d_x, int32_t B, float* d_y, p
   Work w;
   if (fused(n)) {
     PF_CHECK(ensure_work(n, B, &w));
-    PF_CHECK(run_rows(n, d_x, nullptr, B, d_y, w, s));
+    // the CTAs of the row kernel read x and write y in any order: outputs over the inputs go through a copy
+    const size_t xb = (size_t)B * n->d_in * sizeof(float), yb = (size_t)B * n->d_out * sizeof(float);
+    const bool over = (uintptr_t)d_x < (uintptr_t)d_y + yb && (uintptr_t)d_y < (uintptr_t)d_x + xb;
+    PF_CHECK(run_rows(n, d_x, nullptr, B, over ? w.y : d_y, w, s));
+    if (over) PF_CUDA(cudaMemcpyAsync(d_y, w.y, yb, cudaMemcpyDeviceToDevice, s));
     PF_CUDA(cudaStreamSynchronize(s));
     return POLFED_OK;
   }
