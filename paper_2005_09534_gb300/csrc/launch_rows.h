@@ -48,7 +48,8 @@ int launch_rows_t(const StepRun& run, int max_group, int64_t items, bool coopera
   int teams = std::min(max_teams, cache.d[dev].maxdyn / per_team);
   if (teams < 1) return fail(POLFED_EINVAL, "slice tile does not fit in shared memory");
   // one CTA per SM; as many teams as there are work items for them
-  const int grid = (int)std::min<int64_t>(nsm, items);
+  // (moments: as many CTAs as the buffer of their sums holds)
+  const int grid = (int)std::min<int64_t>(MODE == kMoments ? std::min(nsm, kMaxMomentCtas) : nsm, items);
   teams = (int)std::min<int64_t>(teams, (items + grid - 1) / grid);
   StepRun r = run;
   void* args[] = {(void*)&r, (void*)&tile};

@@ -191,7 +191,7 @@ int apply_block(HamPlan& plan, int kind, const void* in, void* out, int n_b, int
 // mu[2k] = t_k . t_k, mu[2k + 1] = t_{k+1} . t_k summed over n_b columns, t_{k+1} = 2 H~ t_k - t_{k-1}, k < half
 // (device, overwritten).  t_odd: moment_scratch_bytes (float-float keeps t_n in FP64); part: room for the sums of
 // kMaxMomentCtas CTAs of one step at least, more steps to a launch with more.  Synchronizes.
-constexpr int kMaxMomentCtas = 304;  // one per SM
+constexpr int kMaxMomentCtas = 304;  // the launch takes one per SM, and no more than these
 int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, void* t_odd, void* part, size_t part_bytes,
                  double* mu, FilterScratch& scr, cudaStream_t s);
 int moments_b(int kind, int L);  // low bits of a plan for moments, 0: the plan's own choice
