@@ -69,7 +69,7 @@ cudaMemPool_t scratch_pool(bool create) {
     size_t free_b = 0, total = 0;
     cudaMemPool_t q = nullptr;
     if (cudaMemGetInfo(&free_b, &total) == cudaSuccess && cudaMemPoolCreate(&q, &props) == cudaSuccess) {
-      uint64_t keep = total / 64;
+      uint64_t keep = total / 256;
       if (cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
         g_pools.pool[dev] = q;
       else
