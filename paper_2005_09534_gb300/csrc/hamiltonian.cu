@@ -271,13 +271,17 @@ __global__ void __launch_bounds__(kTableThreads) k_tables(const HamGeometry g, c
       r->hn_base[e] = m ? rank_hi(grp ^ m) : 0;
     } else {
       const int k = e - kMaxHigh;
-      int base = 0;
+      int base = 0, n = 0;
       if (k < g.n_cross) {
         const uint32_t g2 = grp ^ (1u << g.cross_hi[k]);
         // rows with the bond antiparallel exist only if the neighbouring class is valid
-        if (valid(g2)) base = rank_hi(g2);
+        if (valid(g2)) {
+          base = rank_hi(g2);
+          n = (int)B[g.b][g.n_up - __popc(g2)];
+        }
       }
       r->cr_base[k] = base;
+      r->cr_n[k] = n;
     }
     return;
   }

@@ -134,6 +134,7 @@ struct alignas(16) GroupRec {
   int r0, n_g, cls_base, n_hn1, n_hn, need_mask, pad0, pad1;
   int hn_base[kMaxHigh];  // first row of each neighbouring group through an antiparallel high bond
   int cr_base[8];         // first row of the group reached through cross bond k
+  int cr_n[8];            // rows of that group (0 if no row of this group has the bond antiparallel)
 };
 
 int build_geometry(const polfed_model* m, int b_override, HamGeometry* g);
