@@ -10,7 +10,6 @@ int launch_rows_df(const StepRun& run, int lpr, bool j2, StepMode mode, int max_
     case kMoments: return launch_rows_mode<RDF, kMoments>(run, lpr, j2, max_group, items, cooperative, max_teams, s);
     default: return fail(POLFED_EINVAL, "step mode needs FP32 or FP64 storage");
   }
-  return fail(POLFED_EINVAL, "unsupported step mode");
 }
 
 }  // namespace polfed

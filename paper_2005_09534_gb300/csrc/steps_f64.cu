@@ -11,7 +11,6 @@ int launch_rows_f64(const StepRun& run, int lpr, bool j2, StepMode mode, int max
     case kMoments: return launch_rows_mode<RF64, kMoments>(run, lpr, j2, max_group, items, cooperative, max_teams, s);
     default: return fail(POLFED_EINVAL, "per-column coefficients need FP32 storage");
   }
-  return fail(POLFED_EINVAL, "unsupported step mode");
 }
 
 }  // namespace polfed
