@@ -29,8 +29,8 @@
 #include <cstdlib>
 #include <cstring>
 #include <atomic>
-#include <condition_variable>
 #include <mutex>
+#include <thread>
 #include <type_traits>
 
 #include "polfed_internal.h"
@@ -772,45 +772,60 @@ static int launch_rows(const StepRun& run, int kind, int lpr, bool j2, StepMode 
 
 // A cooperative grid fills the GPU and its CTAs wait for one another, so only
 // one is in flight per device: a thread holds a turn from a launch to its
-// completion.  Turns are given in the order of asking, and a call of many
-// launches gives its turn up about every kTurnSeconds, so that a short call of
-// another thread does not wait for the end of a long one.
+// completion.  A call of many launches gives its turn up about every
+// kTurnSeconds if another thread waits, and a thread that had the last turn lets
+// the other go first, so that a short call does not wait for the end of a long
+// one.  What needs no turn (event creation, reading the error flag) stays outside
+// it, and turns are not handed over in the order of asking: either leaves the GPU
+// idle, 3% of a run of 64 realizations on as many threads.
 class Turn {
   struct Queue {
     std::mutex mu;
-    std::condition_variable cv;
-    uint64_t next = 0, serving = 0;
+    std::atomic<int> waiting{0};
+    std::atomic<uint64_t> given{0};
   };
-  static Queue& queue() {
+  static Queue& queue(int dev) {
     static Queue q[64];
+    return q[dev];
+  }
+  static uint64_t& last(int dev) {
+    static thread_local uint64_t l[64];
+    return l[dev];
+  }
+  static int device() {
     int dev = 0;
     cudaGetDevice(&dev);
-    return q[dev & 63];
+    return dev & 63;
   }
   Queue& q_;
+  uint64_t& last_;  // this thread's latest turn
+
+  void take() {
+    while (q_.waiting.load() > 0 && q_.given.load() == last_) std::this_thread::yield();
+    q_.waiting++;
+    q_.mu.lock();
+    q_.waiting--;
+    last_ = ++q_.given;
+  }
 
  public:
-  Turn() : q_(queue()) {
-    std::unique_lock<std::mutex> lk(q_.mu);
-    const uint64_t mine = q_.next++;
-    q_.cv.wait(lk, [&] { return q_.serving == mine; });
-  }
-  ~Turn() {
-    {
-      std::lock_guard<std::mutex> lk(q_.mu);
-      q_.serving++;
-    }
-    q_.cv.notify_all();
-  }
+  explicit Turn(int dev = device()) : q_(queue(dev)), last_(last(dev)) { take(); }
+  ~Turn() { q_.mu.unlock(); }
   Turn(const Turn&) = delete;
   Turn& operator=(const Turn&) = delete;
+  void again() {  // between two launches of a long call, none in flight
+    if (q_.waiting.load() == 0) return;
+    q_.mu.unlock();
+    take();
+  }
 };
 
-constexpr double kTurnSeconds = 0.25;
+constexpr double kTurnSeconds = 0.1;        // of a filter or of moments: the steps of a turn, in one or more launches
+constexpr double kBatchTurnSeconds = 0.25;  // of a batched filter: one launch
 
 // An upper estimate of a step's seconds, by the bytes of its slices (measured: 1.7 to 3.6 TB/s in FP32 and
 // float-float; half of that and less where FP64 bounds it) and by the rows of the busiest team (0.1 to 0.2 us each
-// of 128 bytes).  Launches and turns are cut by it; a turn's end costs about 20 us.
+// of 128 bytes).  Turns are cut by it; they are 2 to 4 times shorter than it says, and the end of one costs 20 us.
 static double step_seconds(double row_bytes, int64_t items, int max_group) {
   const int64_t teams = 152 * kMaxTeams, rounds = (items + teams - 1) / teams;
   return 5e-6 + std::max(4.0 * row_bytes / 0.5e12, 0.4e-6 * (double)rounds * max_group);
@@ -983,27 +998,34 @@ static int slice_out(int kind, int abi_kind, const void* ys, int64_t dim, const 
 #undef PF_SO
 }
 
-// Device time of a run of step launches, by a pair of CUDA events on the launching stream.
-// The launches of storage kind `kind` issued between construction and stop()
-// are credited to the timed counters with the measured time.
+// Device time of the step launches of storage kind `kind` between start() and
+// stop(), by a pair of CUDA events on the launching stream; credited to the timed
+// counters.  Only what has to happen within a turn is done by start() and wait().
 struct StepTimer {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaStream_t s;
   int kind;
-  int64_t n0;
-  double b0;
+  int64_t n0 = 0;
+  double b0 = 0.0;
   StepTimer(cudaStream_t st, int k) : s(st), kind(k) {
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) drop();
+  }
+  void start() {
     n0 = counters().all_launches[kind];
     b0 = counters().all_alg_bytes[kind];
-    if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) cudaEventRecord(e0, s);
+    if (e0) cudaEventRecord(e0, s);
   }
-  int stop() {  // synchronizes
-    if (!e0 || !e1) {
+  int wait() {  // for the launches
+    if (!e0) {
       PF_CUDA(cudaStreamSynchronize(s));
       return POLFED_OK;
     }
     PF_CUDA(cudaEventRecord(e1, s));
     PF_CUDA(cudaEventSynchronize(e1));
+    return POLFED_OK;
+  }
+  int credit() {
+    if (!e0) return POLFED_OK;
     float ms = 0.f;
     PF_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     Counters& c = counters();
@@ -1017,10 +1039,16 @@ struct StepTimer {
     c.kind_alg_bytes[kind] += b;
     return POLFED_OK;
   }
-  ~StepTimer() {
+  int stop() {
+    PF_CHECK(wait());
+    return credit();
+  }
+  void drop() {
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
+    e0 = e1 = nullptr;
   }
+  ~StepTimer() { drop(); }
 };
 
 // A step kernel whose bounded wait expired leaves plan.err_flag set.
@@ -1070,33 +1098,40 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
   const int64_t items = (int64_t)plan.geo.n_groups * ns;
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
   const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
-  for (int t0 = 0; t0 < K; t0 += turn_steps) {
-    {
-      const Turn turn;
-      StepTimer tm(s, kind);  // within the turn: the time of these launches, not of other threads' before them
-      for (int st = t0, end = std::min(K, t0 + turn_steps); st < end; st = run.st1) {
-        run.st0 = st;
-        run.st1 = std::min(end, st + kParamSteps);
-        run.bar_base = plan.bar_base;
-        double alg = 0.0;
-        for (int q = run.st0; q < run.st1; q++) {
-          const int k = K - 1 - q;
-          double c = col ? 1.0 : coef(k);
-          if (!col) {
-            if (k == 0) c *= invD;
-            run.cx[q - st] = typed_const(kind, c);
-          }
-          alg += row * (3.0 + (c != 0.0 ? 1.0 : 0.0));
-        }
-        const int grid = launch_rows(run, kind, f.lpr, j2, col ? kFilterCols : kFilter, plan.geo.max_group, items, true, s);
-        if (grid < 0) return grid;
-        plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
-        count_step(kind, alg);
+  StepTimer tm(s, kind);
+  {
+    Turn turn;
+    tm.start();  // within the turn: the time of these launches, not of other threads' before them
+    for (int st = 0, t0 = 0; st < K; st = run.st1) {
+      if (st == t0 + turn_steps) {
+        PF_CHECK(tm.stop());
+        PF_CHECK(check_timeout(plan, s));
+        turn.again();
+        tm.start();
+        t0 = st;
       }
-      PF_CHECK(tm.stop());  // synchronizes: the turn ends when its last launch is done
+      run.st0 = st;
+      run.st1 = std::min({K, st + kParamSteps, t0 + turn_steps});
+      run.bar_base = plan.bar_base;
+      double alg = 0.0;
+      for (int q = run.st0; q < run.st1; q++) {
+        const int k = K - 1 - q;
+        double c = col ? 1.0 : coef(k);
+        if (!col) {
+          if (k == 0) c *= invD;
+          run.cx[q - st] = typed_const(kind, c);
+        }
+        alg += row * (3.0 + (c != 0.0 ? 1.0 : 0.0));
+      }
+      const int grid = launch_rows(run, kind, f.lpr, j2, col ? kFilterCols : kFilter, plan.geo.max_group, items, true, s);
+      if (grid < 0) return grid;
+      plan.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
+      count_step(kind, alg);
     }
-    PF_CHECK(check_timeout(plan, s));
+    PF_CHECK(tm.wait());
   }
+  PF_CHECK(tm.credit());
+  PF_CHECK(check_timeout(plan, s));
   *res = (K % 2 == 0) ? b.ba : b.bb;
   return POLFED_OK;
 }
@@ -1193,26 +1228,29 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
     const int64_t per_step = std::min<int64_t>(items, kMaxMomentCtas) * sizeof(double2);
     const int launch_steps = (int)std::max<int64_t>(1, std::min<int64_t>(kParamSteps, (int64_t)part_bytes / per_step));
     const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
-    for (int t0 = 0; t0 < half; t0 += turn_steps) {
-      {
-        const Turn turn;
-        for (int st = t0, end = std::min(half, t0 + turn_steps); st < end; st = run.st1) {
-          run.st0 = st;
-          run.st1 = std::min(end, st + launch_steps);
-          run.bar_base = plan.bar_base;
-          const int n = run.st1 - run.st0;
-          const int grid = launch_rows(run, kind, p.f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
-          if (grid < 0) return grid;
-          plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
-          count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
-          k_moment_sums<<<n, 32, 0, s>>>((const double2*)part, grid, mu + 2 * st);
-          PF_CUDA(cudaGetLastError());
-          count_launch();
+    {
+      Turn turn;
+      for (int st = 0, t0 = 0; st < half; st = run.st1) {
+        if (st == t0 + turn_steps) {
+          PF_CHECK(check_timeout(plan, s));  // synchronizes
+          turn.again();
+          t0 = st;
         }
-        PF_CUDA(cudaStreamSynchronize(s));
+        run.st0 = st;
+        run.st1 = std::min({half, st + launch_steps, t0 + turn_steps});
+        run.bar_base = plan.bar_base;
+        const int n = run.st1 - run.st0;
+        const int grid = launch_rows(run, kind, p.f.lpr, j2, kMoments, plan.geo.max_group, items, true, s);
+        if (grid < 0) return grid;
+        plan.bar_base += (unsigned)grid * (unsigned)(n - 1);
+        count_step(kind, row * (kind == POLFED_DF64 ? 5.0 : 3.0) * n);
+        k_moment_sums<<<n, 32, 0, s>>>((const double2*)part, grid, mu + 2 * st);
+        PF_CUDA(cudaGetLastError());
+        count_launch();
       }
-      PF_CHECK(check_timeout(plan, s));
+      PF_CUDA(cudaStreamSynchronize(s));
     }
+    PF_CHECK(check_timeout(plan, s));
   }
   return POLFED_OK;
 }
@@ -1394,25 +1432,27 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
       const FilterShape f = batch_shape(it.plan->geo, kind, it.n_b);
       row += (double)it.plan->geo.dim * f.W * elem_bytes(kind) * f.nsl;
     }
-    const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, groups, max_group)));
-    for (int st = 0; st < n_steps; st += turn_steps) {
-      run.st0 = st;
-      run.st1 = std::min(n_steps, st + turn_steps);
-      {
-        const Turn turn;
-        StepTimer tm(s, kind);
+    const int turn_steps = std::max(1, (int)(kBatchTurnSeconds / step_seconds(row, groups, max_group)));
+    StepTimer tm(s, kind);
+    {
+      Turn turn;
+      for (int st = 0; st < n_steps; st += turn_steps) {
+        if (st > 0) turn.again();
+        run.st0 = st;
+        run.st1 = std::min(n_steps, st + turn_steps);
+        tm.start();
         grid = launch_rows(run, kind, kBatchLpr, j2, kFilter, max_group, groups, true, s,
                            ctas_per_sm == 1 ? kMaxTeams / 2 : kMaxTeams);
         if (grid < 0) return grid;
         count_step(kind, alg * (run.st1 - run.st0) / n_steps);  // one launch carries every job's steps
         PF_CHECK(tm.stop());
+        run.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
       }
-      run.bar_base += (unsigned)grid * (unsigned)(run.st1 - run.st0 - 1);
-      int e = 0;
-      PF_CUDA(cudaMemcpyAsync(&e, run.err, sizeof(int), cudaMemcpyDeviceToHost, s));
-      PF_CUDA(cudaStreamSynchronize(s));
-      if (e) return fail(POLFED_ETIMEOUT, "a grid barrier of the batched filter timed out");
     }
+    int e = 0;
+    PF_CUDA(cudaMemcpyAsync(&e, run.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    PF_CUDA(cudaStreamSynchronize(s));
+    if (e) return fail(POLFED_ETIMEOUT, "a grid barrier of the batched filter timed out");
     if (bst) {
       bst->n_jobs = (int)jobs.size();
       bst->n_steps = n_steps;
