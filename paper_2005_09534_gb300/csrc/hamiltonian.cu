@@ -824,11 +824,13 @@ constexpr double kTurnSeconds = 0.1;        // of a filter or of moments: the st
 constexpr double kBatchTurnSeconds = 0.25;  // of a batched filter: one launch
 
 // An upper estimate of a step's seconds, by the bytes of its slices (measured: 1.7 to 3.6 TB/s in FP32 and
-// float-float; half of that and less where FP64 bounds it) and by the rows of the busiest team (0.1 to 0.2 us each
-// of 128 bytes).  Turns are cut by it; they are 2 to 4 times shorter than it says, and the end of one costs 20 us.
-static double step_seconds(double row_bytes, int64_t items, int max_group) {
+// float-float; half of that and less in FP64, whose pipe bounds it) and by the rows of the busiest team (0.1 to 0.2 us
+// each of 128 bytes).  Turns are cut by it.  The end of one costs up to 0.2 ms: an L = 22 run's filters take 56.3 to
+// 56.7 s with launches of 448 steps, 56.8 with turns of 196 and 56.9 with turns of 138.
+static double step_seconds(int kind, double row_bytes, int64_t items, int max_group) {
   const int64_t teams = 152 * kMaxTeams, rounds = (items + teams - 1) / teams;
-  return 5e-6 + std::max(4.0 * row_bytes / 0.5e12, 0.4e-6 * (double)rounds * max_group);
+  const double rate = kind == POLFED_F64 ? 0.5e12 : 1.5e12;
+  return 5e-6 + std::max(4.0 * row_bytes / rate, 0.4e-6 * (double)rounds * max_group);
 }
 
 // ------------------------------------------------------------ filter engine
@@ -1097,7 +1099,7 @@ static int run_steps(HamPlan& plan, int kind, const FilterShape& f, int ns, cons
   run.one.colw = colw;
   const int64_t items = (int64_t)plan.geo.n_groups * ns;
   const double row = (double)plan.geo.dim * f.W * elem_bytes(kind) * ns;
-  const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
+  const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(kind, row, items, plan.geo.max_group)));
   StepTimer tm(s, kind);
   {
     Turn turn;
@@ -1227,7 +1229,7 @@ int moment_steps(HamPlan& plan, int kind, const void* in, int n_b, int half, voi
     const double row = (double)dim * p.f.W * elem_bytes(kind) * p.ns;
     const int64_t per_step = std::min<int64_t>(items, kMaxMomentCtas) * sizeof(double2);
     const int launch_steps = (int)std::max<int64_t>(1, std::min<int64_t>(kParamSteps, (int64_t)part_bytes / per_step));
-    const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(row, items, plan.geo.max_group)));
+    const int turn_steps = std::max(1, (int)(kTurnSeconds / step_seconds(kind, row, items, plan.geo.max_group)));
     {
       Turn turn;
       for (int st = 0, t0 = 0; st < half; st = run.st1) {
@@ -1432,7 +1434,7 @@ int filter_batched(std::vector<BatchFilterItem>& items, int kind, int abi_kind, 
       const FilterShape f = batch_shape(it.plan->geo, kind, it.n_b);
       row += (double)it.plan->geo.dim * f.W * elem_bytes(kind) * f.nsl;
     }
-    const int turn_steps = std::max(1, (int)(kBatchTurnSeconds / step_seconds(row, groups, max_group)));
+    const int turn_steps = std::max(1, (int)(kBatchTurnSeconds / step_seconds(kind, row, groups, max_group)));
     StepTimer tm(s, kind);
     {
       Turn turn;
