@@ -75,8 +75,9 @@ void upload_binomials() {
 
 // -------------------------------------------------------------- geometry
 // Low bits of a plan.  Large L: b = 10, a group block of at most C(10,5) * 128 B
-// = 32 KB (six teams to an SM).  Smaller L: few enough rows per group that the
-// groups feed all 912 teams.  Measured on GB300 (whole calls, b one lower / chosen /
+// = 32 KB (six teams to an SM).  Smaller L: smaller groups, so that there are
+// more of them for the 912 teams (by L alone; a block of several slices has that
+// many more work items).  Measured on GB300 (whole calls, b one lower / chosen /
 // one higher): L = 14 FP64 K = 200: 1.20, 1.14, 1.37 ms; L = 18 float-float 256
 // moments: 3.16, 2.85, 3.33 ms; L = 20 J1-J2 float-float K = 64: 7.93, 7.23, 7.48 ms
 // (FP32 per column: 3.74, 3.14, 3.04); L = 22 FP32 K = 200 at b = 8 / 9 / 10: 45.1,
@@ -859,7 +860,7 @@ static FilterShape filter_shape(const HamGeometry& g, int kind, int n_b, size_t 
 
 // The FP32 filter takes 64-byte rows where a slice of 128-byte ones, the gather
 // source, is beyond L2 (346 MB at L = 24) and rows gather few neighbours: XXZ,
-// 32 columns, K = 40: 18.5 ms with 128 bytes, 17.2 with 64 (21.2 with 32).  Within L2
+// 32 columns, K = 40: 18.5 ms with 128 bytes, 17.0 with 64 (21.2 with 32).  Within L2
 // (L = 22) they cost 7%; J1-J2 gains nothing (38.1 and 38.3 ms at L = 24).
 static FilterShape filter_rows(const HamGeometry& g, int kind, int n_b, size_t limit) {
   const FilterShape f = filter_shape(g, kind, n_b, limit);
