@@ -841,7 +841,7 @@ def run_batched(args, pf, torch, dev, world, rank, local, dist):
                        "l2": "instances of 12870-48620 rows: filter working sets partly L2-resident, no flush"},
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(achieved / peak, 4), "traffic": None, "peak_kind": f"of {peak_kind}",
-                         "kernel": "k_step_rows (all realizations' Clenshaw steps, one cooperative launch)",
+                         "kernel": "k_step_rows (all realizations' Clenshaw steps; bytes and time per round of launches)",
                          "alg_bytes_per_launch": fa / max(1, sum(i["rounds"] for i in infos)),
                          "avg_launch_us": round(1e6 * fg / max(1, sum(i["rounds"] for i in infos)), 1)},
             "e2e": {"value": round(pairs_all / wall_s, 4), "unit": "eigenpairs/s",
